@@ -57,6 +57,7 @@ int dg_build_tables(int N, DgTables *t) {
     LN[j] = L[N];
     t->xi[j] = (double)x[j];
     t->w[j] = (double)(2.0L / ((ld)N * (N + 1) * L[N] * L[N]));
+    t->wl[j] = 2.0L / ((ld)N * (N + 1) * L[N] * L[N]);
     t->invw[j] = (double)(((ld)N * (N + 1) * L[N] * L[N]) / 2.0L);
   }
   for (int i = 0; i < n; ++i)
@@ -67,6 +68,7 @@ int dg_build_tables(int N, DgTables *t) {
       else if (i == N) v = (ld)N * (N + 1) / 4.0L;
       else v = 0.0L;
       t->D[i * n + m] = (double)v;
+      t->Q[i * n + m] = i == m ? 0.0L : t->wl[i] * v;
     }
   for (int k = 0; k < n; ++k) {
     ld g = (k < N) ? 1.0L : (ld)(2 * N + 1) / (ld)N;

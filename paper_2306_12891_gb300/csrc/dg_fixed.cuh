@@ -1,0 +1,539 @@
+// dg_fixed.cuh -- the FP64 volume kernel for the Kennedy-Gruber and Pirozzoli fluxes without the blend,
+// its two-point fluxes and viscous divergence evaluated in 64-bit fixed point on the integer pipes. Part
+// of dg_kernels.cuh (same unnamed namespace); works on the degree constants defined there.
+//
+// Why: GB300 issues FP64 arithmetic at 2 lanes per clock and SM, IMAD.WIDE at 25 and 64-bit integer adds
+// at 55 (measured). A pair flux is 30 FP64 instructions (~16 clocks per lane and SM); in fixed point it is
+// 13 products of three IMAD.WIDE each and ~40 adds and shifts (~2 clocks).
+//
+// Format: per element every quantity is scaled by a power of two taken from the element's largest value of
+// it, X = x 2^s with |X| < 2^62 (rho, p) or 2^60 (the rest): an FP64 significand has 53 bits, so an input
+// is exact down to 2^-7 of the element's maximum. A product keeps the high 64 of 128 bits: with X = 2^32 h +
+// l, h and l signed 32-bit halves, it is h h' + (h l' + l h') / 2^32; the dropped l l' is below a quarter
+// unit. Every product is rounded to nearest in a window chosen per element (FxScale), so that the largest
+// value it can take fills the word. Pair sums, sums over a line and over directions are exact integer adds,
+// so with the pair symmetry Q_im = -Q_mi of the SBP operator Q = W D a pair's two shares cancel exactly.
+// Precision: all rounding happens at about 2^-61 of the largest flux sum the element can have, where FP64
+// rounds each flux and each partial sum at 2^-53 of itself. An element takes the general FP64 path of the
+// same kernel (fx_general_node) instead when a value is not finite, rho, p or h (e) is not positive or
+// spans more than 2^8 within the element, or the exponents leave a safe range.
+#pragma once
+
+namespace {
+
+typedef long long fx_t;
+
+__constant__ int2 c_Qx[nn];                       // Q_im = w_i D_im, zero diagonal, 2^63, halves (h, l)
+// rows of the viscous divergence, 2^62: n even, row i < n/2 the even half of Q, row N - i the odd half (n/2 each);
+// n odd, Q itself
+constexpr int FX_QV = n % 2 == 0 ? EO_H : n;
+__constant__ int2 c_QV[n * FX_QV];
+constexpr int FX_H = (n + 1) / 2;                 // distinct node weights
+__constant__ int2 c_rho[FX_H * FX_H];             // min(w_a, w_b) / w_a, 2^62: [a][b], a, b = distance to the face
+
+__device__ __forceinline__ fx_t fx_mad(int a, int b, fx_t c) {
+  fx_t r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+// balanced halves of X = 2^32 h + l, l in [-2^31, 2^31), from X + 2^31
+struct FxD {
+  int h, l;
+};
+constexpr fx_t FX_BIAS = 0x80000000ll;
+__device__ __forceinline__ FxD fx_biased(fx_t x) { return FxD{(int)(x >> 32), (int)x ^ (int)0x80000000}; }
+__device__ __forceinline__ FxD fx_split(fx_t x) { return fx_biased(x + FX_BIAS); }
+__device__ __forceinline__ FxD fx_const(int2 q) { return FxD{q.x, q.y}; }
+// one sum of products: hi collects h h', lo collects h l' + l h'
+struct FxSum {
+  fx_t hi, lo;
+};
+__device__ __forceinline__ void fx_acc(FxSum &s, FxD a, FxD b) {
+  s.lo = fx_mad(a.h, b.l, s.lo);
+  s.lo = fx_mad(a.l, b.h, s.lo);
+  s.hi = fx_mad(a.h, b.h, s.hi);
+}
+// the sum / 2^64 times 2^a (0 <= a < 32): lo starts at half a unit of that window, which rounds; with hi
+// starting at the same number the value comes out with the bias that fx_biased takes
+__device__ __forceinline__ FxSum fx_zero(int a) { return FxSum{0, (fx_t)(0x80000000u >> a)}; }
+__device__ __forceinline__ FxSum fx_zero_biased(int a) { return FxSum{(fx_t)(0x80000000u >> a), (fx_t)(0x80000000u >> a)}; }
+__device__ __forceinline__ fx_t fx_value(const FxSum &s, int a) { return (s.hi << a) + (s.lo >> (32 - a)); }
+__device__ __forceinline__ FxD fx_mul(FxD a, FxD b) {
+  FxSum s = fx_zero_biased(0);
+  fx_acc(s, a, b);
+  return fx_biased(fx_value(s, 0));
+}
+__device__ __forceinline__ fx_t fx_shr(fx_t x, int k) {  // x / 2^k rounded, 0 <= k <= 62
+  return (x + ((1ll << k) >> 1)) >> k;
+}
+
+// |x| 2^(...) truncated, with x's sign: the leading significand bit of a double with biased exponent E
+// lands on bit 62 - drop (E >= the exponent of x)
+__device__ __forceinline__ fx_t fx_from(double x, int E, int drop) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int ex = (hi >> 20) & 0x7ff;
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const unsigned long long M = (((unsigned long long)mh << 32) | lo) << 10;
+  const int s = min(E - ex + drop, 63);
+  const fx_t X = (fx_t)(M >> s);
+  return hi < 0 ? -X : X;
+}
+// biased exponent that bounds a magnitude whose high word is at most `hi` (with 2^-16 to spare, so that a
+// sum of two values at the bound still splits into signed halves)
+__device__ __forceinline__ int fx_exponent(int hi) { return (hi + 0x10) >> 20; }
+__device__ __forceinline__ int fx_hi_abs(double x) { return __double2hiint(x) & 0x7fffffff; }
+
+// per-element scales, from the maxima (high words) of the staged quantities, the metric terms and the
+// viscous flux
+struct FxScale {
+  int ok;
+  int er, eu, ep, ex, ej;  // exponents E of rho, velocity, p, h (or e), metric terms
+  int dp, dx;              // extra bits dropped from p and h (e)
+  int av, ag;              // windows of V and G
+  int kg, kv;              // right shifts of G before the momentum product, of V before p V (KG)
+  int vm, ve;              // fx_from exponents of the viscous flux (momentum, energy)
+  int k0, km, ke;          // results are fixed value x 2^k x (1/w)
+};
+constexpr int FX_AM = 3;  // window of the momentum and energy products
+
+// upper bound of log2 of a magnitude whose high word is at most hi, in 2^-20: log2 m <= (m - 1) + 0.0861
+__device__ __forceinline__ int fx_lg(int hi) { return hi - (1023 << 20) + 0x16200; }
+// largest row sum R of |Q|: 0.5, 1.34, 1.87, 2.44, 2.79, 3.15, 3.41 (N = 1..7): its log2 in 2^-20, and ceil(log2 R)
+constexpr int FX_LGR = N == 1 ? -1048576 : N == 2 ? 443000 : N == 3 ? 947000 : N == 4 ? 1350000 : N == 5 ? 1552000
+                     : N == 6 ? 1736000 : 1856000;
+constexpr int FX_RB = N == 1 ? 0 : N <= 3 ? 1 : 2;
+
+// Bounds (value x scale, log2): S_rho < 63, S_u, S_Ja, S_h < 61, S_p < 63; T = Q S_rho < 62; V = u.Ja <=
+// max|u| max_d sum_c |Ja^d_c| fills 62.9, G = T V fills 62.3; momentum and energy operands are shifted
+// right until a line's sum of advective terms stays below 61.7; the viscous share adds at most 59.8. The
+// halved sum of three directions then stays below 62.9, and the cross sums h l' + l h' of every product
+// group below 63.
+template <int VF>
+__device__ __forceinline__ FxScale fx_scales(const int *mx, int2 mj, int mvm, int mve, bool ns) {
+  // mx: high words: rho max, rho min, |u| max, p max, p min, x max, x min (minima signed); mj: of the
+  // largest |Ja^d_c| and the largest sum_c |Ja^d_c|
+  FxScale s;
+  s.er = fx_exponent(mx[0]); s.ep = fx_exponent(mx[3]); s.ex = fx_exponent(mx[5]); s.ej = fx_exponent(mj.x);
+  s.eu = max(fx_exponent(mx[2]), (1996 - s.er + s.ep) >> 1);  // floor 2^-26 sqrt(p / rho): kg stays within 62
+  const int lo = min(min(s.er, s.ep), min(s.ex, min(s.ej, s.eu)));
+  const int hi = max(max(s.er, s.ep), max(s.ex, max(s.ej, s.eu)));
+  const int lr = fx_lg(mx[0]), lu = max(fx_lg(mx[2]), (s.eu - 1023) << 20), lp = fx_lg(mx[3]), lx = fx_lg(mx[5]), lj = fx_lg(mj.y);
+  const int lv = lu + lj;                                      // log2 of the V bound
+  constexpr int L = 1 << 20, LIM = (int)(61.7 * L);
+  // scales: fixed = value 2^s
+  const int st = 1084 - s.er, sv0 = 2102 - s.eu - s.ej;
+  s.av = min((((int)(62.9 * L) - lv) >> 20) - sv0, 6);
+  const int sv = sv0 + s.av;
+  s.ag = min((((int)(62.3 * L) - lr - lv) >> 20) - (st + sv - 64), 4);
+  const int sg = st + sv - 64 + s.ag;
+  const int xa = sg + 1022 - s.eu, xp = 2106 - s.ep - s.ej;    // momentum from G u, from p Ja
+  int xm = min(min(xa, xp), (LIM - (FX_LGR + L + max(lr + lv + lu, lp + lj))) >> 20);
+  const int evm = fx_exponent(mvm), eve = fx_exponent(mve);
+  if (ns) xm = min(xm, 1081 - evm);
+  s.kg = xa - xm;
+  s.dp = xp - xm;
+  const int xe0 = sg + 1022 - s.ex;                            // energy from G h (G e)
+  int be = lr + lv + lx, xe = xe0, xq = 0;
+  if (VF == VF_KG) {  // and from (Q S_p) V
+    xq = 3123 - s.dp - s.ep - s.eu - s.ej + s.av;
+    xe = min(xe, xq);
+    be = max(be, lp + lv) + L;
+  }
+  xe = min(xe, (LIM - (FX_LGR + be)) >> 20);
+  if (ns) xe = min(xe, 1081 - eve);
+  s.dx = xe0 - xe;
+  s.kv = VF == VF_KG ? 2 + xq - xe : 0;
+  s.vm = 1084 - xm;  // (the rows c_QV carry one bit less than Q)
+  s.ve = 1084 - xe;
+  s.k0 = 2 - (sg - FX_RB); s.km = 2 - xm; s.ke = 2 - xe;  // 2 D F, and the halved sum of directions
+  const int kmax = max(max(abs(s.k0), abs(s.km)), abs(s.ke));
+  s.ok = mx[1] > 0 && mx[4] > 0 && mx[6] > 0 && s.er - (mx[1] >> 20) <= 8 && s.ep - (mx[4] >> 20) <= 8 &&
+         s.ex - (mx[6] >> 20) <= 8 && lo >= 700 && hi <= 1350 && kmax <= 900 && s.av >= 0 && s.ag >= 0 &&
+         s.kg >= 0 && s.kg <= 62 && s.dp >= 0 && s.dx >= 0 && s.kv <= 62 && (!ns || (evm < 2000 && eve < 2000));
+  return s;
+}
+
+// staging index of node (i, j, k): strides chosen so that the lanes of a half warp (two lines' nodes along any
+// direction) meet few bank conflicts (n = 8: strides 10 and 82, 2 mod 4: none along eta and zeta)
+constexpr int FX_SJ = n == 8 ? 10 : n + 1, FX_SK = n == 8 ? 82 : n * (n + 1) + 1;
+constexpr int FX_PS = N * (1 + FX_SJ + FX_SK) + 1;
+__device__ __forceinline__ int fx_idx(int node) { return node % n + FX_SJ * ((node / n) % n) + FX_SK * (node / nn); }
+
+// element slots (fx_t, FX_PS each): 0-5 rho, u, v, w, p, h|e; 6 + 3 dir + c metric terms; after a line thread
+// has finished node i, its direction's sums (5) replace the three metric slots of (dir, i) and slots
+// 15 + 2 dir, 16 + 2 dir
+constexpr int FX_SLOTS = 21;
+__device__ __forceinline__ int fx_slot(int dir, int v) { return v < 3 ? 6 + 3 * dir + v : 12 + 2 * dir + v; }
+
+struct FxNode {
+  fx_t r, u, v, w, p, x, jx, jy, jz;
+};
+__device__ __forceinline__ FxNode fx_load(const fx_t *__restrict__ S, int a, int dir) {
+  const fx_t *J = S + (6 + 3 * dir) * FX_PS + a;
+  return FxNode{S[a], S[FX_PS + a], S[2 * FX_PS + a], S[3 * FX_PS + a], S[4 * FX_PS + a], S[5 * FX_PS + a], J[0], J[FX_PS], J[2 * FX_PS]};
+}
+
+// the five fluxes of one pair, weighted with Q_im (see fx_scales for the scales); the staged values carry half
+// the bias each, so a pair sum splits without an add
+template <int VF>
+__device__ __forceinline__ void fx_pair(const FxNode &a, const FxNode &b, FxD q, int av, int ag, int kg, int kv,
+                                        fx_t F[5]) {
+  const FxD Sjx = fx_biased(a.jx + b.jx), Sjy = fx_biased(a.jy + b.jy), Sjz = fx_biased(a.jz + b.jz);
+  const FxD Su = fx_biased(a.u + b.u), Sv = fx_biased(a.v + b.v), Sw = fx_biased(a.w + b.w);
+  FxSum s = fx_zero_biased(av);
+  fx_acc(s, Su, Sjx);
+  fx_acc(s, Sv, Sjy);
+  fx_acc(s, Sw, Sjz);
+  const fx_t Vb = fx_value(s, av);
+  s = fx_zero_biased(ag);
+  fx_acc(s, fx_mul(q, fx_biased(a.r + b.r)), fx_biased(Vb));
+  const fx_t Gb = fx_value(s, ag), G = Gb - FX_BIAS;
+  const FxD P = fx_mul(q, fx_biased(a.p + b.p));
+  F[0] = (Gb + (((1 << FX_RB) >> 1) - FX_BIAS)) >> FX_RB;
+  const FxD Gm = fx_split(fx_shr(G, kg));
+  s = fx_zero(FX_AM);
+  fx_acc(s, Gm, Su); fx_acc(s, P, Sjx);
+  F[1] = fx_value(s, FX_AM);
+  s = fx_zero(FX_AM);
+  fx_acc(s, Gm, Sv); fx_acc(s, P, Sjy);
+  F[2] = fx_value(s, FX_AM);
+  s = fx_zero(FX_AM);
+  fx_acc(s, Gm, Sw); fx_acc(s, P, Sjz);
+  F[3] = fx_value(s, FX_AM);
+  s = fx_zero(FX_AM);
+  fx_acc(s, fx_biased(Gb), fx_biased(a.x + b.x));
+  if (VF == VF_KG) fx_acc(s, P, fx_split(fx_shr(Vb - FX_BIAS, kv)));
+  F[4] = fx_value(s, FX_AM);
+}
+
+// Lanes of the pair phase: a warp takes FX_LPW lines of one direction, one lane per node, a line's nodes in
+// neighbouring lanes
+constexpr int FX_LPW = 32 / n;
+
+// viscous divergence of the lane's node along its line: -sum_m Q_im Fv_m / 2 for the four quantities.
+// n even: lane i < n/2 forms the sum with the even half of Q, lane N - i that with the odd half
+// (n^2/2 products per line and quantity instead of n^2)
+__device__ __forceinline__ void fx_viscous(const double *__restrict__ Fn, const int2 *__restrict__ sQ, int idx, int l0,
+                                           int vm, int ve, fx_t acc[5]) {
+  const int2 *row = sQ + idx * FX_QV;
+  double f64[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) f64[q] = __ldg(Fn + q * nnn);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const fx_t f = fx_from(f64[q], q < 3 ? vm : ve, 0);
+    FxSum s = fx_zero(0);
+    if constexpr (n % 2 == 0) {
+      const bool low = idx < EO_H;
+      const int opp = l0 + N - idx;
+      const fx_t g = __shfl_sync(0xffffffffu, f, opp);
+      const fx_t h = low ? f + g : g - f;  // the even sum, or the odd difference of the low node
+#pragma unroll
+      for (int m = 0; m < EO_H; ++m)
+        fx_acc(s, fx_const(row[m]), fx_split(__shfl_sync(0xffffffffu, h, l0 + (low ? m : N - m))));
+      const fx_t y = fx_value(s, 0), z = __shfl_sync(0xffffffffu, y, opp);
+      acc[1 + q] = low ? -(y + z) : z - y;
+    } else {
+#pragma unroll
+      for (int m = 0; m < n; ++m)  // (the diagonal of Q is zero)
+        fx_acc(s, fx_const(row[m]), fx_split(__shfl_sync(0xffffffffu, f, l0 + m)));
+      acc[1 + q] = -fx_value(s, 0);
+    }
+  }
+}
+
+// general path of one node in FP64: flux differencing and viscous divergence, from the staged quantities
+// rho, u, v, w, p, h|e (doubles, slots 0-5)
+template <int VF>
+__device__ __noinline__ void fx_general_node(const DgDevice &d, const double *S, size_t e, int node, double s[5]) {
+  const int ijk[3] = {node % n, (node / n) % n, node / nn};
+  const int a = fx_idx(node);
+  for (int v = 0; v < 5; ++v) s[v] = 0.0;
+  for (int dd = 0; dd < 3; ++dd) {
+    const int id = ijk[dd];
+    const int st = dd == 0 ? 1 : dd == 1 ? n : nn, pst = dd == 0 ? 1 : dd == 1 ? FX_SJ : FX_SK;
+    const double *Jd = d.Ja + (e * 3 + dd) * 3 * nnn + node;
+    for (int m = 0; m < n; ++m) {
+      if (m == id) continue;
+      const int b = a + (m - id) * pst, off = (m - id) * st;
+      const double Sj[3] = {Jd[0] + Jd[off], Jd[nnn] + Jd[nnn + off], Jd[2 * nnn] + Jd[2 * nnn + off]};
+      const double Su = S[FX_PS + a] + S[FX_PS + b], Sv = S[2 * FX_PS + a] + S[2 * FX_PS + b], Sw = S[3 * FX_PS + a] + S[3 * FX_PS + b];
+      const double Vp = Su * Sj[0] + Sv * Sj[1] + Sw * Sj[2];
+      const double Sp = S[4 * FX_PS + a] + S[4 * FX_PS + b], F0 = (S[a] + S[b]) * Vp;
+      double F4 = F0 * (S[5 * FX_PS + a] + S[5 * FX_PS + b]);
+      if (VF == VF_KG) F4 += 2.0 * Sp * Vp;
+      const double c = c_De[id * n + m];
+      s[0] += c_Dq[id * n + m] * F0;
+      s[1] += c * (F0 * Su + 4.0 * Sp * Sj[0]);
+      s[2] += c * (F0 * Sv + 4.0 * Sp * Sj[1]);
+      s[3] += c * (F0 * Sw + 4.0 * Sp * Sj[2]);
+      s[4] += c * F4;
+      if (d.equations == 1) {
+        const double *Fv = d.Fv + (e * 12 + dd * 4) * nnn + node + off;
+        for (int q = 0; q < 4; ++q) s[1 + q] -= c_D[id * n + m] * Fv[q * nnn];
+      }
+    }
+  }
+}
+
+// One thread per node. What bounds it: instruction issue (55 % of the slots) with the FP64 pipe at 36 %, FMA-heavy
+// (IMAD.WIDE) at 44 %, ALU at 52 % and DRAM at 15 %; 64 registers and 21 slots of shared memory keep two CTAs
+// (32 warps) per SM at N = 7. A thread per line (half the pair evaluations' overhead, sums in 80 registers,
+// 168 in all) held 12 warps and measured 2.43 ms per launch at N = 7, 24^3, Navier-Stokes, Pirozzoli; this form
+// 1.74 ms, the FP64 line kernel before it 6.21 ms (N = 5, 24 x 12 x 12 channel: 0.197 against 0.586 ms).
+// Elements per CTA: one; CTAs of one or two warps at the lowest degrees, so that small meshes spread over the SMs
+constexpr int FX_EPB = N == 1 ? 8 : N == 2 ? 2 : 1;
+constexpr int FX_THREADS = round32(FX_EPB * nnn);
+constexpr size_t FX_SMEM = sizeof(fx_t) * FX_EPB * FX_SLOTS * FX_PS;
+constexpr int FX_MINB = 1024 / FX_THREADS < 32 ? 1024 / FX_THREADS : 32;  // 64 registers per thread
+
+template <int VF>
+__global__ void __launch_bounds__(FX_THREADS, FX_MINB)
+    k_volume_fx(const DgDevice d, const double *U, double *out, double *__restrict__ g, int mode, int first, double dt,
+                double A, double B) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  fx_t *S = reinterpret_cast<fx_t *>(sm_raw);  // [EPB][FX_SLOTS][FX_PS]
+  __shared__ int s_mx[FX_EPB][8];
+  __shared__ FxScale s_sc[FX_EPB];
+  __shared__ int2 s_rho[FX_H * FX_H], s_Q[nn], s_QV[n * FX_QV];
+  const int e0 = blockIdx.x * FX_EPB, tid = threadIdx.x;
+  const bool ns = d.equations == 1;
+  const double gm1 = d.gm1;
+  for (int t = tid; t < FX_EPB * 8; t += FX_THREADS) {
+    const int k = t & 7;
+    s_mx[t >> 3][k] = (k == 1 || k == 4 || k == 6) ? 0x7fffffff : 0;
+  }
+  for (int t = tid; t < FX_H * FX_H; t += FX_THREADS) s_rho[t] = c_rho[t];
+  for (int t = tid; t < nn; t += FX_THREADS) s_Q[t] = c_Qx[t];
+  for (int t = tid; t < n * FX_QV; t += FX_THREADS) s_QV[t] = c_QV[t];
+  __syncthreads();
+  // phase A: primitive quantities of the thread's node and the element maxima
+  const int le = tid / nnn, node = tid % nnn, e = e0 + le;
+  const bool on = tid < FX_EPB * nnn && e < d.nE;
+  double q[6], J[9];
+  {
+    int m0 = 0, n0 = 0x7fffffff, mu_ = 0, m3 = 0, n3 = 0x7fffffff, m5 = 0, n5 = 0x7fffffff;
+    if (on) {
+      double Uv[5];
+      load_state<double>(d, U, e, node, Uv);
+      const double *Je = d.Ja + (size_t)e * 9 * nnn + node;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) J[k] = __ldg(Je + k * nnn);
+      const double r = Uv[0], ir = 1.0 / r;
+      const double u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
+      const double p = gm1 * (Uv[4] - 0.5 * (Uv[1] * u + Uv[2] * v + Uv[3] * w));
+      const double x = VF == VF_PIR ? (Uv[4] + p) * ir : Uv[4] * ir;
+      q[0] = r; q[1] = u; q[2] = v; q[3] = w; q[4] = p; q[5] = x;
+      if (!(r > 0.0) || !(p > 0.0) || !isfinite(Uv[4])) flag_set(d.flag, 1);
+      // minima keep the sign (a negative high word fails the scale test), maxima are of magnitudes
+      m0 = fx_hi_abs(r); n0 = __double2hiint(r);
+      mu_ = max(max(fx_hi_abs(u), fx_hi_abs(v)), fx_hi_abs(w));
+      m3 = fx_hi_abs(p); n3 = __double2hiint(p);
+      m5 = fx_hi_abs(x); n5 = __double2hiint(x);
+    }
+    bool each = on;  // whether this lane adds its own maxima
+    if (FX_EPB == 1) {
+      m0 = __reduce_max_sync(0xffffffffu, m0); n0 = __reduce_min_sync(0xffffffffu, n0);
+      mu_ = __reduce_max_sync(0xffffffffu, mu_);
+      m3 = __reduce_max_sync(0xffffffffu, m3); n3 = __reduce_min_sync(0xffffffffu, n3);
+      m5 = __reduce_max_sync(0xffffffffu, m5); n5 = __reduce_min_sync(0xffffffffu, n5);
+      each = (tid & 31) == 0 && on;
+    }
+    if (each) {
+      atomicMax(&s_mx[le][0], m0); atomicMin(&s_mx[le][1], n0); atomicMax(&s_mx[le][2], mu_);
+      atomicMax(&s_mx[le][3], m3); atomicMin(&s_mx[le][4], n3);
+      atomicMax(&s_mx[le][5], m5); atomicMin(&s_mx[le][6], n5);
+    }
+  }
+  __syncthreads();
+  int good = 1;
+  if (tid < FX_EPB && e0 + tid < d.nE) {
+    const int et = e0 + tid;
+    s_sc[tid] = fx_scales<VF>(s_mx[tid], d.jmax[et], ns ? d.fvmax[2 * et] : 0, ns ? d.fvmax[2 * et + 1] : 0, ns);
+    good = s_sc[tid].ok;
+  }
+  const bool ok = __syncthreads_and(good);
+  if (ok) {
+    if (on) {
+      const FxScale &c = s_sc[le];
+      fx_t *Se = S + le * FX_SLOTS * FX_PS + fx_idx(node);
+      constexpr fx_t HB = FX_BIAS / 2;
+      Se[0] = fx_from(q[0], c.er, 1) + HB;
+      Se[FX_PS] = fx_from(q[1], c.eu, 3) + HB;
+      Se[2 * FX_PS] = fx_from(q[2], c.eu, 3) + HB;
+      Se[3 * FX_PS] = fx_from(q[3], c.eu, 3) + HB;
+      Se[4 * FX_PS] = fx_from(q[4], c.ep, 1 + c.dp) + HB;
+      Se[5 * FX_PS] = fx_from(q[5], c.ex, 3 + c.dx) + HB;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) Se[(6 + k) * FX_PS] = fx_from(J[k], c.ej, 3) + HB;
+    }
+    __syncthreads();
+    // phase B: one lane per node of a line. Lane i forms the pairs (i, i + s mod n), s <= (n - 1) / 2, adds its
+    // share and hands the partner's on by a shuffle; at s = n / 2 (n even) both nodes form the pair.
+    constexpr int GROUPS = (FX_EPB * nn + FX_LPW - 1) / FX_LPW;  // warps' worth of lines per direction
+    const int lane = tid & 31;
+    for (int gr = tid >> 5; gr < 3 * GROUPS; gr += FX_THREADS / 32) {
+      const int dir = gr / GROUPS, g0 = (gr % GROUPS) * FX_LPW;
+      const int idx = lane % n, l = (lane / n) % FX_LPW, l0 = l * n;
+      // lanes without a line of their own repeat the group's first one
+      const bool own = lane < FX_LPW * n && g0 + l < FX_EPB * nn;
+      const int ln = own ? g0 + l : g0;
+      const int lel = ln / nn, ll = ln % nn;
+      const int la = ll % n, lb = ll / n;
+      const int gb = dir == 0 ? n * (la + n * lb) : dir == 1 ? la + nn * lb : la + n * lb;
+      const int gs = dir == 0 ? 1 : dir == 1 ? n : nn, ps = dir == 0 ? 1 : dir == 1 ? FX_SJ : FX_SK;
+      const int pb = dir == 0 ? FX_SJ * la + FX_SK * lb : dir == 1 ? la + FX_SK * lb : la + FX_SJ * lb;
+      const FxScale &c = s_sc[lel];
+      fx_t *Se = S + lel * FX_SLOTS * FX_PS;
+      const int ai = pb + idx * ps;
+      fx_t acc[5] = {0, 0, 0, 0, 0};
+      if (ns) {
+        const size_t el = min(e0 + lel, d.nE - 1);
+        fx_viscous(d.Fv + (el * 12 + dir * 4) * nnn + gb + idx * gs, s_QV, idx, l0, c.vm, c.ve, acc);
+      }
+      const int av = c.av, ag = c.ag, kg = c.kg, kv = c.kv;
+      const FxNode ni = fx_load(Se, ai, dir);
+#pragma unroll 1
+      for (int s = 1; s <= n / 2; ++s) {
+        const int m = idx + s < n ? idx + s : idx + s - n;
+        const FxNode nm = fx_load(Se, pb + m * ps, dir);
+        fx_t F[5];
+        fx_pair<VF>(ni, nm, fx_const(s_Q[idx * n + m]), av, ag, kg, kv, F);
+        const bool both = 2 * s == n;
+        const int src = l0 + (idx >= s ? idx - s : idx - s + n);
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          acc[v] += F[v];
+          if (!both) acc[v] -= __shfl_sync(0xffffffffu, F[v], src);
+        }
+      }
+      __syncwarp();
+      if (own) {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) Se[fx_slot(dir, v) * FX_PS + ai] = acc[v];
+      }
+    }
+  } else if (on) {
+    double *Se = reinterpret_cast<double *>(S) + le * FX_SLOTS * FX_PS + fx_idx(node);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) Se[k * FX_PS] = q[k];
+  }
+  __syncthreads();
+  if (!on) return;
+  // phase C: per node -- directions summed, surface terms, neighbour's viscous flux, Jacobian, output / LSERK
+  const int ijk[3] = {node % n, (node / n) % n, node / nn};
+  double s[5];
+  if (ok) {
+    const fx_t *Se = S + le * FX_SLOTS * FX_PS + fx_idx(node);
+    const int a0 = min(ijk[0], N - ijk[0]), a1 = min(ijk[1], N - ijk[1]), a2 = min(ijk[2], N - ijk[2]);
+    const int am = min(a0, min(a1, a2));  // the direction with the smallest weight
+    const FxD r0 = fx_const(s_rho[a0 * FX_H + am]), r1 = fx_const(s_rho[a1 * FX_H + am]),
+              r2 = fx_const(s_rho[a2 * FX_H + am]);
+    const double iw = c_invw[am];
+    const int iwh = __double2hiint(iw), iwl = __double2loint(iw);
+    const int k0 = s_sc[le].k0, km = s_sc[le].km, ke = s_sc[le].ke;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      FxSum f0{0, 0x40000000ll}, f1 = f0, f2 = f0;  // the three lo sums do not fit one
+      fx_acc(f0, r0, fx_split(Se[fx_slot(0, v) * FX_PS]));
+      fx_acc(f1, r1, fx_split(Se[fx_slot(1, v) * FX_PS]));
+      fx_acc(f2, r2, fx_split(Se[fx_slot(2, v) * FX_PS]));
+      // half the sum of the three directions (the factors carry 2^62)
+      const fx_t sum = ((f0.hi + f1.hi + f2.hi) << 1) + (f0.lo >> 31) + (f1.lo >> 31) + (f2.lo >> 31);
+      s[v] = (double)sum * __hiloint2double(iwh + (int)((unsigned)(v == 0 ? k0 : v < 4 ? km : ke) << 20), iwl);
+    }
+  } else {
+    double sg[5];
+    fx_general_node<VF>(d, reinterpret_cast<const double *>(S) + le * FX_SLOTS * FX_PS, e, node, sg);
+#pragma unroll
+    for (int v = 0; v < 5; ++v) s[v] = sg[v];
+  }
+#pragma unroll
+  for (int dd = 0; dd < 3; ++dd) {
+    const int id = ijk[dd];
+    if (id != 0 && id != N) continue;
+    const int f = 2 * dd + (id == N ? 1 : 0);
+    const int pp = dd == 0 ? ijk[1] : ijk[0], qq = dd == 2 ? ijk[1] : ijk[2];
+    const double iwb = c_invw[0];
+    const double *fs = d.Fsurf + ((size_t)e * 6 + f) * 5 * nn + pp + n * qq;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) s[v] += iwb * fs[v * nn];
+    if (ns) {  // -(1/(2 w_b)) phi_nb, phi_nb = neighbour's outward normal viscous flux; or the wall's
+      const int *ef = d.ef + ((size_t)e * 6 + f) * 4;
+      const int nb = ef[0], fnb = ef[1], o = ef[2];
+      if (nb < 0) {
+        const double *fw = d.Fwall + (size_t)ef[3] * 4 * nn + pp + n * qq;
+        const double hs = (id == N) ? 0.5 : -0.5;
+        const double *Fve = d.Fv + ((size_t)e * 12 + dd * 4) * nnn + node;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) s[1 + v] -= iwb * (fw[v * nn] - hs * Fve[v * nnn]);
+      } else {
+        int p2, q2;
+        orient_map(o, pp, qq, p2, q2);
+        const double sg = (fnb & 1) ? 0.5 * iwb : -0.5 * iwb;
+        const double *Fvn = d.Fv + ((size_t)nb * 12 + (fnb >> 1) * 4) * nnn + face_node(fnb, p2, q2);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) s[1 + v] += sg * Fvn[v * nnn];
+      }
+    }
+  }
+  const double miJ = -d.invJ[(size_t)e * nnn + node];
+  const size_t gi = (size_t)e * 5 * nnn + node;
+  if (mode == 0) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) out[gi + v * nnn] = miJ * s[v];
+  } else {
+    const double fac = dt * miJ;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const double du = fac * s[v];
+      const double gv = first ? du : A * g[gi + v * nnn] + du;
+      g[gi + v * nnn] = gv;
+      out[gi + v * nnn] = U[gi + v * nnn] + B * gv;
+    }
+  }
+}
+
+// largest |Ja^d_c| and largest sum_c |Ja^d_c| of each element (high words), for the fixed-point scales
+__global__ void __launch_bounds__(128) k_metric_max(const DgDevice d) {
+  __shared__ int m[2];
+  if (threadIdx.x < 2) m[threadIdx.x] = 0;
+  __syncthreads();
+  int h = 0, h1 = 0;
+  for (int t = threadIdx.x; t < 3 * nnn; t += blockDim.x) {
+    const double *J = d.Ja + ((size_t)blockIdx.x * 3 + t / nnn) * 3 * nnn + t % nnn;
+    const double a = fabs(J[0]), b = fabs(J[nnn]), c = fabs(J[2 * nnn]);
+    h = max(max(h, fx_hi_abs(a)), max(fx_hi_abs(b), fx_hi_abs(c)));
+    h1 = max(h1, fx_hi_abs(a + b + c));
+  }
+  atomicMax(&m[0], h);
+  atomicMax(&m[1], h1);
+  __syncthreads();
+  if (threadIdx.x == 0) d.jmax[blockIdx.x] = int2{m[0], m[1]};
+}
+
+// fixed-point tables from the extended-precision Q = W D and weights (host)
+cudaError_t fx_upload(const DgTables &t) {
+  auto halves = [](long double v, int bits) {  // v 2^bits rounded to nearest, balanced halves
+    const long long x = std::llrint(std::ldexp(v, bits));
+    const int l = (int)(unsigned)(x & 0xffffffffll);
+    return int2{(int)((x - l) >> 32), l};
+  };
+  int2 Q[nn], QV[n * FX_QV], rho[FX_H * FX_H];
+  for (int i = 0; i < nn; ++i) Q[i] = halves(t.Q[i], 63);
+  for (int i = 0; i < n; ++i)
+    for (int m = 0; m < FX_QV; ++m) {
+      long double v = t.Q[i * n + m];
+      if (n % 2 == 0 && i < n / 2) v = (v + t.Q[i * n + N - m]) / 2;
+      else if (n % 2 == 0) v = (t.Q[(N - i) * n + m] - t.Q[(N - i) * n + N - m]) / 2;
+      QV[i * FX_QV + m] = halves(v, 62);
+    }
+  for (int a = 0; a < FX_H; ++a)
+    for (int b = 0; b < FX_H; ++b) rho[a * FX_H + b] = halves(t.wl[a < b ? a : b] / t.wl[a], 62);
+  cudaError_t err = cudaMemcpyToSymbol(c_Qx, Q, sizeof(Q));
+  err = err ? err : cudaMemcpyToSymbol(c_QV, QV, sizeof(QV));
+  return err ? err : cudaMemcpyToSymbol(c_rho, rho, sizeof(rho));
+}
+
+}  // namespace

@@ -16,6 +16,8 @@ struct DgTables {
   double D[(DG_NMAX + 1) * (DG_NMAX + 1)];     // D[i*n+m] = l_m'(xi_i)
   double Vinv[(DG_NMAX + 1) * (DG_NMAX + 1)];  // inverse orthonormal-Legendre Vandermonde
   double xh[DG_NMAX + 2];                      // FV subcell interfaces -1 + cumulative weights
+  long double wl[DG_NMAX + 1];                 // weights and Q_im = w_i D_im (zero diagonal) before rounding
+  long double Q[(DG_NMAX + 1) * (DG_NMAX + 1)];
 };
 
 // Plain view of a context's device state, passed by value to every kernel.
@@ -44,6 +46,8 @@ struct DgDevice {
   double *Ja;          // [nE][3 d][3 c][n^3]
   double *J;           // [nE][n^3]
   double *invJ;        // [nE][n^3]
+  int2 *jmax;          // [nE] high words of the largest |Ja^d_c| and sum_c |Ja^d_c| (fixed-point scales)
+  int *fvmax;          // [nE][2] high words of the largest viscous flux |Fv| (momentum, energy), by the lifting
   float *Jaf;          // FP32 copy of Ja for the FP32-bulk path (or null)
   double *nrm;         // [nF][4][n^2]: unit normal (x,y,z) outward from L, area factor s
   float *nrm_f;        // FP32 copy of nrm for the FP32-bulk path (or null)

@@ -28,6 +28,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "dg_convert.cuh"
@@ -599,7 +600,8 @@ template <typename R, bool PRE = false>
 __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *__restrict__ W,
                                           const R (*__restrict__ sD)[n + 1], const R *__restrict__ Jae,
                                           const R *__restrict__ Wse, R iJ, R mu, R kappa, R *__restrict__ out,
-                                          const R *__restrict__ S = nullptr, double *__restrict__ tau = nullptr) {
+                                          const R *__restrict__ S = nullptr, double *__restrict__ tau = nullptr,
+                                          int *fvm = nullptr) {
   // PRE: the reference derivatives D_dd w_q of this element come precomputed in S [3 dd][4 q][nnn]
   const int ijk[3] = {node % n, (node / n) % n, node / nn};
   R Ja[3][3];
@@ -667,8 +669,24 @@ __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *
 #pragma unroll
   for (int dd = 0; dd < 3; ++dd)
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      out[(dd * 4 + q) * nnn + node] = Ja[dd][0] * Fc[0][q] + Ja[dd][1] * Fc[1][q] + Ja[dd][2] * Fc[2][q];
+    for (int q = 0; q < 4; ++q) {
+      const R f = Ja[dd][0] * Fc[0][q] + Ja[dd][1] * Fc[1][q] + Ja[dd][2] * Fc[2][q];
+      out[(dd * 4 + q) * nnn + node] = f;
+      // FP64: high words of the largest momentum and energy components, the volume kernel's scale
+      if constexpr (std::is_same<R, double>::value) fvm[q / 3] = max(fvm[q / 3], __double2hiint(f) & 0x7fffffff);
+    }
+}
+
+// the element maxima of the viscous flux: the warp's lanes reduced first where they share an element
+__device__ __forceinline__ void lift_fvmax(int (*s_fv)[2], int le, bool on, const int fvm[2]) {
+  const int le0 = __shfl_sync(0xffffffffu, le, 0);
+  if (__all_sync(0xffffffffu, !on || le == le0)) {
+    const int m0 = __reduce_max_sync(0xffffffffu, on ? fvm[0] : 0), m1 = __reduce_max_sync(0xffffffffu, on ? fvm[1] : 0);
+    if ((threadIdx.x & 31) == 0 && on) { atomicMax(&s_fv[le][0], m0); atomicMax(&s_fv[le][1], m1); }
+  } else if (on) {
+    atomicMax(&s_fv[le][0], fvm[0]);
+    atomicMax(&s_fv[le][1], fvm[1]);
+  }
 }
 
 template <typename R>
@@ -677,6 +695,8 @@ __global__ void __launch_bounds__(LIFT_THREADS, lift_min_blocks<R>()) k_lift(con
   __shared__ R W[LIFT_EPB][4][nnn];
   __shared__ R sD[n][n + 1];  // D, rows padded: lanes read different rows without bank conflicts
   for (int t = threadIdx.x; t < nn; t += blockDim.x) sD[t / n][t % n] = Tab<R>::D(t);
+  __shared__ int s_fv[LIFT_EPB][2];
+  if (threadIdx.x < 2 * LIFT_EPB) s_fv[threadIdx.x / 2][threadIdx.x & 1] = 0;
   const int e0 = blockIdx.x * LIFT_EPB;
   const R gm1 = Cst<R>::gm1(d), iR = Cst<R>::iR(d);
   const R pref = Cst<R>::pref(d);
@@ -695,14 +715,21 @@ __global__ void __launch_bounds__(LIFT_THREADS, lift_min_blocks<R>()) k_lift(con
 #pragma unroll
   for (int rr = 0; rr < (LIFT_EPB * nnn + LIFT_THREADS - 1) / LIFT_THREADS; ++rr) {
     const int t = threadIdx.x + rr * LIFT_THREADS;
-    if (t >= LIFT_EPB * nnn) continue;
     const int le = t / nnn, node = t % nnn, e = e0 + le;
-    if (e >= d.nE) continue;
-    const R iJ = kShift<R> ? (R)d.invJf[(size_t)e * nnn + node] : (R)d.invJ[(size_t)e * nnn + node];
-    lift_node<R>(d, node, &W[le][0][0], sD, Buf<R>::Ja(d) + (size_t)e * 9 * nnn,
-                 Buf<R>::Wsurf(d) + (size_t)e * 6 * 4 * nn, iJ, mu, kappa, Buf<R>::Fv(d) + (size_t)e * 12 * nnn,
-                 nullptr, tau ? tau + (size_t)e * 6 * nnn : nullptr);
+    const bool on = t < LIFT_EPB * nnn && e < d.nE;
+    int fvm[2] = {0, 0};
+    if (on) {
+      const R iJ = kShift<R> ? (R)d.invJf[(size_t)e * nnn + node] : (R)d.invJ[(size_t)e * nnn + node];
+      lift_node<R>(d, node, &W[le][0][0], sD, Buf<R>::Ja(d) + (size_t)e * 9 * nnn,
+                   Buf<R>::Wsurf(d) + (size_t)e * 6 * 4 * nn, iJ, mu, kappa, Buf<R>::Fv(d) + (size_t)e * 12 * nnn,
+                   nullptr, tau ? tau + (size_t)e * 6 * nnn : nullptr, fvm);
+    }
+    if (!kShift<R>) lift_fvmax(s_fv, le, on, fvm);
   }
+  if (kShift<R>) return;
+  __syncthreads();
+  if (threadIdx.x < 2 * LIFT_EPB && e0 + threadIdx.x / 2 < d.nE)
+    d.fvmax[2 * e0 + threadIdx.x] = s_fv[threadIdx.x / 2][threadIdx.x & 1];
 }
 
 // FP64 lifting with the reference derivatives formed along lines (used at N = 7): one thread per line of the
@@ -720,6 +747,8 @@ __global__ void __launch_bounds__(LIFT_THREADS, lift_min_blocks<double>()) k_lif
     double *W = reinterpret_cast<double *>(sm_raw);  // [EPB][4][nnn]
     double *S = W + LIFT_EPB * 4 * nnn;              // [EPB][12][nnn]
     __shared__ double sD[n][n + 1];
+    __shared__ int s_fv[LIFT_EPB][2];
+    if (threadIdx.x < 2 * LIFT_EPB) s_fv[threadIdx.x / 2][threadIdx.x & 1] = 0;
     for (int t = threadIdx.x; t < nn; t += blockDim.x) sD[t / n][t % n] = c_D[t];
     const int e0 = blockIdx.x * LIFT_EPB;
     const double gm1 = d.gm1, iR = d.iR;
@@ -768,14 +797,19 @@ __global__ void __launch_bounds__(LIFT_THREADS, lift_min_blocks<double>()) k_lif
 #pragma unroll
     for (int rr = 0; rr < (LIFT_EPB * nnn + LIFT_THREADS - 1) / LIFT_THREADS; ++rr) {
       const int t = threadIdx.x + rr * LIFT_THREADS;
-      if (t >= LIFT_EPB * nnn) continue;
       const int le = t / nnn, node = t % nnn, e = e0 + le;
-      if (e >= d.nE) continue;
-      lift_node<double, true>(d, node, W + le * 4 * nnn, sD, d.Ja + (size_t)e * 9 * nnn,
-                              d.Wsurf + (size_t)e * 6 * 4 * nn, d.invJ[(size_t)e * nnn + node], mu, kappa,
-                              d.Fv + (size_t)e * 12 * nnn, S + le * 12 * nnn,
-                              tau ? tau + (size_t)e * 6 * nnn : nullptr);
+      const bool on = t < LIFT_EPB * nnn && e < d.nE;
+      int fvm[2] = {0, 0};
+      if (on)
+        lift_node<double, true>(d, node, W + le * 4 * nnn, sD, d.Ja + (size_t)e * 9 * nnn,
+                                d.Wsurf + (size_t)e * 6 * 4 * nn, d.invJ[(size_t)e * nnn + node], mu, kappa,
+                                d.Fv + (size_t)e * 12 * nnn, S + le * 12 * nnn,
+                                tau ? tau + (size_t)e * 6 * nnn : nullptr, fvm);
+      lift_fvmax(s_fv, le, on, fvm);
     }
+    __syncthreads();
+    if (threadIdx.x < 2 * LIFT_EPB && e0 + threadIdx.x / 2 < d.nE)
+      d.fvmax[2 * e0 + threadIdx.x] = s_fv[threadIdx.x / 2][threadIdx.x & 1];
   }
 }
 
@@ -1181,7 +1215,8 @@ __global__ void __launch_bounds__(vol_threads<R, SC>(), vol_min_blocks<R, SC>())
 
 }  // namespace
 
-#include "dg_fp32.cuh"  // the FP32-bulk volume and lifting kernels without the blend
+#include "dg_fixed.cuh"  // the FP64 volume kernel in 64-bit fixed point (KG and Pirozzoli fluxes, no blend)
+#include "dg_fp32.cuh"   // the FP32-bulk volume and lifting kernels without the blend
 
 namespace {
 
@@ -1397,7 +1432,7 @@ cudaError_t upload(const DgTables &t) {
   ihx[0] = 0.0;
   for (int i = 1; i < n; ++i) ihx[i] = 1.0 / (t.xi[i] - t.xi[i - 1]);
   for (int i = 0; i < n; ++i) fihx[i] = (float)ihx[i];
-  cudaError_t err = cudaSuccess;
+  cudaError_t err = fx_upload(t);
   err = err ? err : cudaMemcpyToSymbol(c_ihx, ihx, sizeof(double) * n);
   err = err ? err : cudaMemcpyToSymbol(c_VP, vp, sizeof(vp));
   err = err ? err : cudaMemcpyToSymbol(c_VM, vm, sizeof(vm));
@@ -1437,6 +1472,7 @@ void launch_face_normals(const DgDevice &d, cudaStream_t s) {
   const long long pts = (long long)d.nF * nn;
   k_face_normals<<<(unsigned)((pts + 255) / 256), 256, 0, s>>>(d);
   if (d.precision == 1) k_round_geometry<<<4 * 152, 256, 0, s>>>(d);
+  else k_metric_max<<<d.nE, 128, 0, s>>>(d);
 }
 
 template <typename R>
@@ -1497,6 +1533,17 @@ void launch_volume_t(const DgDevice &d, const double *U, double *out, double *g,
   }
   k_volume<R, VF, SC><<<(d.nE + VOL_EPB - 1) / VOL_EPB, vol_threads<R, SC>(), smem, s>>>(d, U, out, g, mode, first, dt, A,
                                                                                     B);
+}
+
+template <int VF>
+void launch_volume_fx(const DgDevice &d, const double *U, double *out, double *g, int mode, int first, double dt,
+                      double A, double B, cudaStream_t s) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaFuncSetAttribute(k_volume_fx<VF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
+    attr_set = true;
+  }
+  k_volume_fx<VF><<<(d.nE + FX_EPB - 1) / FX_EPB, FX_THREADS, FX_SMEM, s>>>(d, U, out, g, mode, first, dt, A, B);
 }
 
 template <int VF>
@@ -1562,42 +1609,37 @@ void launch_volume_f32(const DgDevice &d, const double *U, double *out, double *
   k_volume_f32<VF><<<(d.nE + NODE_EPB - 1) / NODE_EPB, NODE_THREADS, smem, s>>>(d, U, out, g, mode, first, dt, A, B);
 }
 
-template <typename R>
-void launch_volume_r(const DgDevice &d, const double *U, double *out, double *g, int mode, int first, double dt,
-                     double A, double B, cudaStream_t s) {
-  const bool sc = d.shock_capturing != 0;
-  if (std::is_same<R, float>::value && !sc) {  // FP32-bulk without the blend: node-per-thread kernel
-    switch (d.vflux) {
-      case VF_KG: launch_volume_f32<VF_KG>(d, U, out, g, mode, first, dt, A, B, s); return;
-      case VF_PIR: launch_volume_f32<VF_PIR>(d, U, out, g, mode, first, dt, A, B, s); return;
-      case VF_EC: launch_volume_f32<VF_EC>(d, U, out, g, mode, first, dt, A, B, s); return;
-      default: launch_volume_f32<VF_CEN>(d, U, out, g, mode, first, dt, A, B, s); return;
-    }
+// the blend (any flux), and in FP64 the fluxes that have no fixed-point form (EC, central): k_volume
+template <typename R, bool SC>
+void launch_volume_lines(const DgDevice &d, const double *U, double *out, double *g, int mode, int first, double dt,
+                         double A, double B, cudaStream_t s) {
+  if constexpr (SC) {
+    if (d.vflux == VF_KG) { launch_volume_t<R, VF_KG, SC>(d, U, out, g, mode, first, dt, A, B, s); return; }
+    if (d.vflux == VF_PIR) { launch_volume_t<R, VF_PIR, SC>(d, U, out, g, mode, first, dt, A, B, s); return; }
   }
-  switch (d.vflux) {
-    case VF_KG:
-      if (sc) launch_volume_t<R, VF_KG, true>(d, U, out, g, mode, first, dt, A, B, s);
-      else launch_volume_t<R, VF_KG, false>(d, U, out, g, mode, first, dt, A, B, s);
-      break;
-    case VF_PIR:
-      if (sc) launch_volume_t<R, VF_PIR, true>(d, U, out, g, mode, first, dt, A, B, s);
-      else launch_volume_t<R, VF_PIR, false>(d, U, out, g, mode, first, dt, A, B, s);
-      break;
-    case VF_EC:
-      if (sc) launch_volume_t<R, VF_EC, true>(d, U, out, g, mode, first, dt, A, B, s);
-      else launch_volume_t<R, VF_EC, false>(d, U, out, g, mode, first, dt, A, B, s);
-      break;
-    default:
-      if (sc) launch_volume_t<R, VF_CEN, true>(d, U, out, g, mode, first, dt, A, B, s);
-      else launch_volume_t<R, VF_CEN, false>(d, U, out, g, mode, first, dt, A, B, s);
-      break;
-  }
+  if (d.vflux == VF_EC) launch_volume_t<R, VF_EC, SC>(d, U, out, g, mode, first, dt, A, B, s);
+  else launch_volume_t<R, VF_CEN, SC>(d, U, out, g, mode, first, dt, A, B, s);
 }
 
 void launch_volume(const DgDevice &d, const double *U, double *out, double *g, int mode, int first, double dt,
                    double A, double B, cudaStream_t s) {
-  if (d.precision == 1) launch_volume_r<float>(d, U, out, g, mode, first, dt, A, B, s);
-  else launch_volume_r<double>(d, U, out, g, mode, first, dt, A, B, s);
+  if (d.shock_capturing) {
+    if (d.precision == 1) launch_volume_lines<float, true>(d, U, out, g, mode, first, dt, A, B, s);
+    else launch_volume_lines<double, true>(d, U, out, g, mode, first, dt, A, B, s);
+  } else if (d.precision == 1) {
+    switch (d.vflux) {
+      case VF_KG: launch_volume_f32<VF_KG>(d, U, out, g, mode, first, dt, A, B, s); break;
+      case VF_PIR: launch_volume_f32<VF_PIR>(d, U, out, g, mode, first, dt, A, B, s); break;
+      case VF_EC: launch_volume_f32<VF_EC>(d, U, out, g, mode, first, dt, A, B, s); break;
+      default: launch_volume_f32<VF_CEN>(d, U, out, g, mode, first, dt, A, B, s); break;
+    }
+  } else if (d.vflux == VF_KG) {
+    launch_volume_fx<VF_KG>(d, U, out, g, mode, first, dt, A, B, s);
+  } else if (d.vflux == VF_PIR) {
+    launch_volume_fx<VF_PIR>(d, U, out, g, mode, first, dt, A, B, s);
+  } else {
+    launch_volume_lines<double, false>(d, U, out, g, mode, first, dt, A, B, s);
+  }
 }
 
 void launch_indicator(const DgDevice &d, const double *U, cudaStream_t s) {

@@ -1,0 +1,93 @@
+"""The FP64 volume kernel's fixed-point arithmetic (KG and Pirozzoli fluxes) where its scales can go
+wrong: flows at rest and at extreme Mach numbers, viscous fluxes above and far below the advective
+ones, units far from 1, and elements whose values span too much for one scale (the kernel's general
+FP64 path), at every degree parity and with ragged element counts per block. The bound is the normwise one
+of the other FP64 parity tests, ULP_FACTOR times the oracle's own spread under one-ulp perturbations of its
+inputs (tests/helpers.py); their flux scale holds the advective flux only, which is not the largest term here.
+"""
+import numpy as np
+import pytest
+
+from helpers import ULP_FACTOR, per_var_max, ulp_spread
+from paper_2306_12891_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env(oracle_mod):
+    import torch
+
+    from paper_2306_12891_gb300 import build, dg
+
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    build.build()
+    dg.lib()
+    return dg, oracle_mod, torch
+
+
+def _map(x, y, z):
+    return (x + 0.1 * np.sin(y) * np.cos(z), y + 0.1 * np.sin(z) * np.sin(x), z + 0.1 * np.sin(x) * np.cos(y))
+
+
+def _fields(xyz, seed, mach):
+    """rho, velocity and p of O(1) variation at the given Mach number (p = 1 / gamma)."""
+    x, y, z = xyz[:, 0], xyz[:, 1], xyz[:, 2]
+    r = np.random.default_rng(seed)
+    a = r.uniform(0, 6, 5)
+    rho = 1.0 + 0.2 * np.sin(x + a[0]) * np.cos(y)
+    vel = [mach * np.sin(x + y + a[1]), mach * np.cos(y + z + a[2]), mach * 0.5 * np.sin(z + a[3])]
+    p = (1.0 + 0.2 * np.cos(x - z + a[4])) / 1.4
+    return rho, vel, p
+
+
+STATES = ["rest", "mach_1e-6", "mach_1", "mach_30", "viscous", "units", "range_ok", "range_general"]
+
+
+def _state(kind, xyz, N):
+    mach = {"rest": 0.0, "mach_1e-6": 1e-6, "mach_30": 30.0}.get(kind, 0.5)
+    rho, vel, p = _fields(xyz, N, mach)
+    mu = {"viscous": 50.0, "rest": 0.1}.get(kind, 1e-3)
+    if kind == "units":
+        rho, p, mu = 1e-9 * rho, 1e5 * p, 1e-12
+        vel = [1e6 * v for v in vel]
+    if kind in ("range_ok", "range_general"):  # one corner of the box is thin: max / min of rho and p
+        ratio = 100.0 if kind == "range_ok" else 3000.0
+        dip = ratio ** -np.exp(-((xyz[:, 0] - 1) ** 2 + (xyz[:, 1] - 1) ** 2 + (xyz[:, 2] - 1) ** 2))
+        rho, p = rho * dip, p * dip
+    return W.cons_from_prim(rho, *vel, p), mu
+
+
+@pytest.mark.parametrize("kind", STATES)
+@pytest.mark.parametrize("N,nel,vf", [(1, (5, 2, 1), "pirozzoli"), (2, (3, 1, 1), "kg"), (5, (3, 1, 1), "pirozzoli"),
+                                      (6, (1, 2, 1), "pirozzoli"), (7, (2, 1, 1), "kg")])
+def test_fixed_point_volume_terms(env, kind, N, nel, vf):
+    dg, orc, torch = env
+    xyz, faces = W.box_mesh(N, nel, mapping=_map)
+    U0, mu = _state(kind, xyz, N)
+    phys = dict(equations="ns", vflux=vf, sflux="llf", mu=mu)
+    gpu, ref = dg.DG(N, xyz, faces, **phys), orc.Oracle(N, xyz, faces, **phys)
+    Ut = gpu.rhs(torch.from_numpy(U0).cuda()).cpu().numpy()
+    gpu.check()
+    spread, Ur = ulp_spread(lambda X, V: orc.Oracle(N, X, faces, **phys).rhs(V), xyz, U0, base=ref.rhs(U0))
+    err = per_var_max(Ut - Ur)
+    print(f"FIXED-POINT {kind} N={N} {vf}: error / bound {err / np.maximum(ULP_FACTOR * spread, 1e-300)}")
+    assert (err <= ULP_FACTOR * spread).all(), (err, ULP_FACTOR * spread)
+
+
+@pytest.mark.parametrize("N", [3, 5])
+def test_nonfinite_values_pass_through_and_are_flagged(env, N):
+    """A NaN stays in its element and the elements that share faces with it, and dg_check reports it."""
+    dg, orc, torch = env
+    xyz, faces = W.box_mesh(N, (4, 3, 3))
+    s = dg.DG(N, xyz, faces, equations="euler", vflux="pirozzoli", sflux="llf")
+    U = torch.from_numpy(W.random_smooth_state(xyz, seed=N, amp=0.1)).cuda()
+    clean = s.rhs(U).cpu()
+    s.check()
+    U[0, 4, 1, 1, 1] = float("nan")
+    Ut = s.rhs(U).cpu()
+    with pytest.raises(dg.DGError):
+        s.check()
+    assert torch.isnan(Ut[0]).any()
+    # elements are grouped per block: the block's others take the general path, equal to rounding
+    assert torch.allclose(Ut[1:], clean[1:], rtol=0, atol=1e-11 * float(clean.abs().max()))
