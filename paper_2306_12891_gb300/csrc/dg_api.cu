@@ -523,8 +523,9 @@ dg_status dg_init(const dg_mesh *mesh, int N, int nodes, const dg_params *prm, v
       DG_ALLOC(d.Fv_f, (size_t)nE * 12 * nnn);
     }
   } else {
-    DG_ALLOC(d.jmax, (size_t)nE);
-    DG_ALLOC(d.fvmax, (size_t)nE * 2);
+    DG_ALLOC(d.ijmax, (size_t)nE * 3);  // ijmax, jmax and fvmax, 8 bytes per element each
+    d.jmax = reinterpret_cast<int2 *>(d.ijmax + nE);
+    d.fvmax = reinterpret_cast<int *>(d.ijmax + 2 * (size_t)nE);
     DG_ALLOC(d.Fsurf, (size_t)nE * 6 * 5 * nn);
     if (prm->equations == DG_NAVIER_STOKES) {
       DG_ALLOC(d.Wsurf, (size_t)nE * 6 * 4 * nn);

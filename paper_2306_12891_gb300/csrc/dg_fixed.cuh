@@ -495,42 +495,57 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
   }
 }
 
-// largest |Ja^d_c| and largest sum_c |Ja^d_c| of each element (high words), for the fixed-point scales
-__global__ void __launch_bounds__(128) k_metric_max(const DgDevice d) {
-  __shared__ int m[2];
-  if (threadIdx.x < 2) m[threadIdx.x] = 0;
-  __syncthreads();
+// largest |Ja^d_c| and largest sum_c |Ja^d_c| of each element (high words) and largest 1/J, for the fixed-point
+// scales (1/J: zero where it spans more than 2^8 in the element, which sends the lifting to its general path)
+__global__ void __launch_bounds__(128) k_metric_max(const DgDevice d) {  // one warp per element
+  const int e = blockIdx.x * 4 + threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (e >= d.nE) return;
   int h = 0, h1 = 0;
-  for (int t = threadIdx.x; t < 3 * nnn; t += blockDim.x) {
-    const double *J = d.Ja + ((size_t)blockIdx.x * 3 + t / nnn) * 3 * nnn + t % nnn;
-    const double a = fabs(J[0]), b = fabs(J[nnn]), c = fabs(J[2 * nnn]);
-    h = max(max(h, fx_hi_abs(a)), max(fx_hi_abs(b), fx_hi_abs(c)));
-    h1 = max(h1, fx_hi_abs(a + b + c));
+  double lo = 1e300, hi = 0.0;
+  for (int t = lane; t < nnn; t += 32) {
+    const double ij = d.invJ[(size_t)e * nnn + t];
+    lo = fmin(lo, ij);
+    hi = fmax(hi, ij);
+#pragma unroll
+    for (int dd = 0; dd < 3; ++dd) {
+      const double *J = d.Ja + ((size_t)e * 3 + dd) * 3 * nnn + t;
+      const double a = fabs(J[0]), b = fabs(J[nnn]), c = fabs(J[2 * nnn]);
+      h = max(max(h, fx_hi_abs(a)), max(fx_hi_abs(b), fx_hi_abs(c)));
+      h1 = max(h1, fx_hi_abs(a + b + c));
+    }
   }
-  atomicMax(&m[0], h);
-  atomicMax(&m[1], h1);
-  __syncthreads();
-  if (threadIdx.x == 0) d.jmax[blockIdx.x] = int2{m[0], m[1]};
+  h = __reduce_max_sync(0xffffffffu, h);
+  h1 = __reduce_max_sync(0xffffffffu, h1);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (lane == 0) {
+    d.jmax[e] = int2{h, h1};
+    d.ijmax[e] = hi <= 256.0 * lo ? hi : 0.0;
+  }
+}
+
+int2 fx_halves(long double v, int bits) {  // v 2^bits rounded to nearest, balanced halves (host)
+  const long long x = std::llrint(std::ldexp(v, bits));
+  const int l = (int)(unsigned)(x & 0xffffffffll);
+  return int2{(int)((x - l) >> 32), l};
 }
 
 // fixed-point tables from the extended-precision Q = W D and weights (host)
 cudaError_t fx_upload(const DgTables &t) {
-  auto halves = [](long double v, int bits) {  // v 2^bits rounded to nearest, balanced halves
-    const long long x = std::llrint(std::ldexp(v, bits));
-    const int l = (int)(unsigned)(x & 0xffffffffll);
-    return int2{(int)((x - l) >> 32), l};
-  };
   int2 Q[nn], QV[n * FX_QV], rho[FX_H * FX_H];
-  for (int i = 0; i < nn; ++i) Q[i] = halves(t.Q[i], 63);
+  for (int i = 0; i < nn; ++i) Q[i] = fx_halves(t.Q[i], 63);
   for (int i = 0; i < n; ++i)
     for (int m = 0; m < FX_QV; ++m) {
       long double v = t.Q[i * n + m];
       if (n % 2 == 0 && i < n / 2) v = (v + t.Q[i * n + N - m]) / 2;
       else if (n % 2 == 0) v = (t.Q[(N - i) * n + m] - t.Q[(N - i) * n + N - m]) / 2;
-      QV[i * FX_QV + m] = halves(v, 62);
+      QV[i * FX_QV + m] = fx_halves(v, 62);
     }
   for (int a = 0; a < FX_H; ++a)
-    for (int b = 0; b < FX_H; ++b) rho[a * FX_H + b] = halves(t.wl[a < b ? a : b] / t.wl[a], 62);
+    for (int b = 0; b < FX_H; ++b) rho[a * FX_H + b] = fx_halves(t.wl[a < b ? a : b] / t.wl[a], 62);
   cudaError_t err = cudaMemcpyToSymbol(c_Qx, Q, sizeof(Q));
   err = err ? err : cudaMemcpyToSymbol(c_QV, QV, sizeof(QV));
   return err ? err : cudaMemcpyToSymbol(c_rho, rho, sizeof(rho));

@@ -47,6 +47,7 @@ struct DgDevice {
   double *J;           // [nE][n^3]
   double *invJ;        // [nE][n^3]
   int2 *jmax;          // [nE] high words of the largest |Ja^d_c| and sum_c |Ja^d_c| (fixed-point scales)
+  double *ijmax;       // [nE] largest 1/J (0 where it spans more than 2^8)
   int *fvmax;          // [nE][2] high words of the largest viscous flux |Fv| (momentum, energy), by the lifting
   float *Jaf;          // FP32 copy of Ja for the FP32-bulk path (or null)
   double *nrm;         // [nF][4][n^2]: unit normal (x,y,z) outward from L, area factor s

@@ -61,8 +61,6 @@ __constant__ double c_ihx[n];  // 1 / (xi_i - xi_{i-1}), i = 1..N (minmod slopes
 constexpr int EO_H = (n % 2 == 0) ? n / 2 : 1;
 __constant__ double c_VP[EO_H * EO_H], c_VM[EO_H * EO_H];
 __constant__ float f_VP[EO_H * EO_H], f_VM[EO_H * EO_H];
-// the same halves of the full D (diagonal included; D_NN = -D_00 keeps the symmetry), for the lifting
-__constant__ double c_FP[EO_H * EO_H], c_FM[EO_H * EO_H];
 __constant__ double c_Vinv[nn];
 __constant__ float f_D[nn], f_D2[nn], f_Dq[nn], f_De[nn];
 __constant__ float f_w[n], f_invw[n], f_xi[n], f_xh[n + 1], f_ihx[n];
@@ -575,9 +573,6 @@ __global__ void __launch_bounds__(256) k_face(const DgDevice d, const double *__
 // BR1 lifting + viscous flux: grad w = (1/J)[sum_d Ja^d D_d w + sum_faces (1/w_b) s n_out (w* - w)],
 // then Fv^d = sum_c Ja^d_c Fv_c(U, grad w) stored per node (4 components: momentum, energy).
 // ---------------------------------------------------------------------------------------------
-// resident 256-thread CTAs per SM the register budget must allow: FP32 five (48 registers), FP64 three
-template <typename R> __host__ __device__ constexpr int lift_min_blocks() { return std::is_same<R, float>::value ? 5 : 3; }
-
 // (u, v, w, T) of one node from its state values (lifted quantities of BR1)
 template <typename R>
 __device__ __forceinline__ void lift_prim(const R Uv[5], R gm1, R iR, R pref, R Wn[4]) {
@@ -596,13 +591,11 @@ __device__ __forceinline__ void lift_prim(const R Uv[5], R gm1, R iR, R pref, R 
 // iJ this node's 1/J; writes the element's Fv [3 d][4][nnn] at `node` (out = the element's Fv).
 // tau (FP64 only, optional): the element's viscous stress record [6][nnn] (xx, yy, zz, xy, xz, yz),
 // which the adjoint's viscous kernel reads instead of forming the gradients again
-template <typename R, bool PRE = false>
+template <typename R>
 __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *__restrict__ W,
                                           const R (*__restrict__ sD)[n + 1], const R *__restrict__ Jae,
                                           const R *__restrict__ Wse, R iJ, R mu, R kappa, R *__restrict__ out,
-                                          const R *__restrict__ S = nullptr, double *__restrict__ tau = nullptr,
-                                          int *fvm = nullptr) {
-  // PRE: the reference derivatives D_dd w_q of this element come precomputed in S [3 dd][4 q][nnn]
+                                          double *__restrict__ tau = nullptr, int *fvm = nullptr) {
   const int ijk[3] = {node % n, (node / n) % n, node / nn};
   R Ja[3][3];
 #pragma unroll
@@ -623,12 +616,8 @@ __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       s[q] = R(0);
-      if constexpr (PRE) {
-        s[q] = S[(dd * 4 + q) * nnn + node];
-      } else {
 #pragma unroll
-        for (int m = 0; m < n; ++m) s[q] += sD[id][m] * W[q * nnn + base + m * st];
-      }
+      for (int m = 0; m < n; ++m) s[q] += sD[id][m] * W[q * nnn + base + m * st];
     }
     if (id == 0 || id == N) {
       const int f = 2 * dd + (id == N ? 1 : 0);
@@ -677,139 +666,31 @@ __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *
     }
 }
 
-// the element maxima of the viscous flux: the warp's lanes reduced first where they share an element
-__device__ __forceinline__ void lift_fvmax(int (*s_fv)[2], int le, bool on, const int fvm[2]) {
-  const int le0 = __shfl_sync(0xffffffffu, le, 0);
-  if (__all_sync(0xffffffffu, !on || le == le0)) {
-    const int m0 = __reduce_max_sync(0xffffffffu, on ? fvm[0] : 0), m1 = __reduce_max_sync(0xffffffffu, on ? fvm[1] : 0);
-    if ((threadIdx.x & 31) == 0 && on) { atomicMax(&s_fv[le][0], m0); atomicMax(&s_fv[le][1], m1); }
-  } else if (on) {
-    atomicMax(&s_fv[le][0], fvm[0]);
-    atomicMax(&s_fv[le][1], fvm[1]);
-  }
-}
-
-template <typename R>
-__global__ void __launch_bounds__(LIFT_THREADS, lift_min_blocks<R>()) k_lift(const DgDevice d, const double *__restrict__ U,
-                                                                             double *__restrict__ tau) {
-  __shared__ R W[LIFT_EPB][4][nnn];
-  __shared__ R sD[n][n + 1];  // D, rows padded: lanes read different rows without bank conflicts
-  for (int t = threadIdx.x; t < nn; t += blockDim.x) sD[t / n][t % n] = Tab<R>::D(t);
-  __shared__ int s_fv[LIFT_EPB][2];
-  if (threadIdx.x < 2 * LIFT_EPB) s_fv[threadIdx.x / 2][threadIdx.x & 1] = 0;
+// FP32 lifting, a thread per node (the FP64 one is k_lift_fx)
+__global__ void __launch_bounds__(LIFT_THREADS, 5) k_lift(const DgDevice d) {
+  __shared__ float W[LIFT_EPB][4][nnn];
+  __shared__ float sD[n][n + 1];  // D, rows padded: lanes read different rows without bank conflicts
+  for (int t = threadIdx.x; t < nn; t += blockDim.x) sD[t / n][t % n] = f_D[t];
   const int e0 = blockIdx.x * LIFT_EPB;
-  const R gm1 = Cst<R>::gm1(d), iR = Cst<R>::iR(d);
-  const R pref = Cst<R>::pref(d);
   for (int t = threadIdx.x; t < LIFT_EPB * nnn; t += blockDim.x) {
     const int le = t / nnn, node = t % nnn, e = e0 + le;
     if (e >= d.nE) continue;
-    R Uv[5], Wn[4];
-    load_state<R>(d, U, e, node, Uv);
-    lift_prim<R>(Uv, gm1, iR, pref, Wn);
+    float Uv[5], Wn[4];
+    load_state<float>(d, nullptr, e, node, Uv);
+    lift_prim<float>(Uv, d.gm1_f, d.iR_f, d.p_ref_f, Wn);
 #pragma unroll
     for (int q = 0; q < 4; ++q) W[le][q][node] = Wn[q];
   }
   __syncthreads();
-  const R mu = Cst<R>::mu(d), kappa = Cst<R>::kappa(d);
   // the thread's nodes unrolled, so that their metric loads are in flight together
 #pragma unroll
   for (int rr = 0; rr < (LIFT_EPB * nnn + LIFT_THREADS - 1) / LIFT_THREADS; ++rr) {
     const int t = threadIdx.x + rr * LIFT_THREADS;
+    if (t >= LIFT_EPB * nnn) continue;
     const int le = t / nnn, node = t % nnn, e = e0 + le;
-    const bool on = t < LIFT_EPB * nnn && e < d.nE;
-    int fvm[2] = {0, 0};
-    if (on) {
-      const R iJ = kShift<R> ? (R)d.invJf[(size_t)e * nnn + node] : (R)d.invJ[(size_t)e * nnn + node];
-      lift_node<R>(d, node, &W[le][0][0], sD, Buf<R>::Ja(d) + (size_t)e * 9 * nnn,
-                   Buf<R>::Wsurf(d) + (size_t)e * 6 * 4 * nn, iJ, mu, kappa, Buf<R>::Fv(d) + (size_t)e * 12 * nnn,
-                   nullptr, tau ? tau + (size_t)e * 6 * nnn : nullptr, fvm);
-    }
-    if (!kShift<R>) lift_fvmax(s_fv, le, on, fvm);
-  }
-  if (kShift<R>) return;
-  __syncthreads();
-  if (threadIdx.x < 2 * LIFT_EPB && e0 + threadIdx.x / 2 < d.nE)
-    d.fvmax[2 * e0 + threadIdx.x] = s_fv[threadIdx.x / 2][threadIdx.x & 1];
-}
-
-// FP64 lifting with the reference derivatives formed along lines (used at N = 7): one thread per line of the
-// element(s) applies D to all four lifted quantities with the even-odd halves of D (the LGL D is
-// centro-antisymmetric), n^2/2 + 2n operations per line and quantity instead of the n^2 of n node-wise
-// sweeps; the derivatives go to shared memory, and the node-wise part (metric contraction, surface
-// terms, viscous flux, contravariant projection) is lift_node's. Dynamic shared memory:
-// W [EPB][4][nnn] and S [EPB][3][4][nnn] doubles.
-constexpr size_t LIFT_LINES_SMEM = sizeof(double) * LIFT_EPB * 16 * nnn;
-__global__ void __launch_bounds__(LIFT_THREADS, lift_min_blocks<double>()) k_lift_lines(const DgDevice d,
-                                                                                      const double *__restrict__ U,
-                                                                                      double *__restrict__ tau) {
-  if constexpr (n % 2 == 0) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    double *W = reinterpret_cast<double *>(sm_raw);  // [EPB][4][nnn]
-    double *S = W + LIFT_EPB * 4 * nnn;              // [EPB][12][nnn]
-    __shared__ double sD[n][n + 1];
-    __shared__ int s_fv[LIFT_EPB][2];
-    if (threadIdx.x < 2 * LIFT_EPB) s_fv[threadIdx.x / 2][threadIdx.x & 1] = 0;
-    for (int t = threadIdx.x; t < nn; t += blockDim.x) sD[t / n][t % n] = c_D[t];
-    const int e0 = blockIdx.x * LIFT_EPB;
-    const double gm1 = d.gm1, iR = d.iR;
-    for (int t = threadIdx.x; t < LIFT_EPB * nnn; t += blockDim.x) {
-      const int le = t / nnn, node = t % nnn, e = e0 + le;
-      if (e >= d.nE) continue;
-      double Uv[5], Wn[4];
-      load_state<double>(d, U, e, node, Uv);
-      lift_prim<double>(Uv, gm1, iR, 0.0, Wn);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) W[(le * 4 + q) * nnn + node] = Wn[q];
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < LIFT_EPB * 3 * nn; t += blockDim.x) {
-      const int le = t / (3 * nn), r = t % (3 * nn), dir = r / nn, line = r % nn;
-      if (e0 + le >= d.nE) continue;
-      const int a = line % n, b = line / n;
-      const int base = dir == 0 ? n * (a + n * b) : dir == 1 ? a + nn * b : a + n * b;
-      const int st = dir == 0 ? 1 : dir == 1 ? n : nn;
-      const double *We = W + le * 4 * nnn;
-      double *Se = S + (le * 12 + dir * 4) * nnn;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        double ev[EO_H], od[EO_H];
-#pragma unroll
-        for (int m = 0; m < EO_H; ++m) {
-          const double f0 = We[q * nnn + base + m * st], f1 = We[q * nnn + base + (N - m) * st];
-          ev[m] = f0 + f1;
-          od[m] = f0 - f1;
-        }
-#pragma unroll
-        for (int i = 0; i < EO_H; ++i) {
-          double pa = 0.0, pb = 0.0;
-#pragma unroll
-          for (int m = 0; m < EO_H; ++m) {
-            pa += c_FP[i * EO_H + m] * ev[m];
-            pb += c_FM[i * EO_H + m] * od[m];
-          }
-          Se[q * nnn + base + i * st] = pa + pb;
-          Se[q * nnn + base + (N - i) * st] = pb - pa;
-        }
-      }
-    }
-    __syncthreads();
-    const double mu = d.mu, kappa = d.kappa;
-#pragma unroll
-    for (int rr = 0; rr < (LIFT_EPB * nnn + LIFT_THREADS - 1) / LIFT_THREADS; ++rr) {
-      const int t = threadIdx.x + rr * LIFT_THREADS;
-      const int le = t / nnn, node = t % nnn, e = e0 + le;
-      const bool on = t < LIFT_EPB * nnn && e < d.nE;
-      int fvm[2] = {0, 0};
-      if (on)
-        lift_node<double, true>(d, node, W + le * 4 * nnn, sD, d.Ja + (size_t)e * 9 * nnn,
-                                d.Wsurf + (size_t)e * 6 * 4 * nn, d.invJ[(size_t)e * nnn + node], mu, kappa,
-                                d.Fv + (size_t)e * 12 * nnn, S + le * 12 * nnn,
-                                tau ? tau + (size_t)e * 6 * nnn : nullptr, fvm);
-      lift_fvmax(s_fv, le, on, fvm);
-    }
-    __syncthreads();
-    if (threadIdx.x < 2 * LIFT_EPB && e0 + threadIdx.x / 2 < d.nE)
-      d.fvmax[2 * e0 + threadIdx.x] = s_fv[threadIdx.x / 2][threadIdx.x & 1];
+    if (e >= d.nE) continue;
+    lift_node<float>(d, node, &W[le][0][0], sD, d.Jaf + (size_t)e * 9 * nnn, d.Wsurf_f + (size_t)e * 6 * 4 * nn,
+                     d.invJf[(size_t)e * nnn + node], d.mu_f, d.kappa_f, d.Fv_f + (size_t)e * 12 * nnn);
   }
 }
 
@@ -1216,6 +1097,7 @@ __global__ void __launch_bounds__(vol_threads<R, SC>(), vol_min_blocks<R, SC>())
 }  // namespace
 
 #include "dg_fixed.cuh"  // the FP64 volume kernel in 64-bit fixed point (KG and Pirozzoli fluxes, no blend)
+#include "dg_fixed_lift.cuh"  // the FP64 lifting in the same fixed point
 #include "dg_fp32.cuh"   // the FP32-bulk volume and lifting kernels without the blend
 
 namespace {
@@ -1414,7 +1296,7 @@ cudaError_t upload(const DgTables &t) {
     }
   for (int i = 0; i < n; ++i) { fw[i] = (float)t.w[i]; finvw[i] = (float)t.invw[i]; fxi[i] = (float)t.xi[i]; }
   for (int i = 0; i <= n; ++i) fxh[i] = (float)t.xh[i];
-  double vp[EO_H * EO_H] = {0.0}, vm[EO_H * EO_H] = {0.0}, fp_[EO_H * EO_H] = {0.0}, fm_[EO_H * EO_H] = {0.0};
+  double vp[EO_H * EO_H] = {0.0}, vm[EO_H * EO_H] = {0.0};
   float fvp[EO_H * EO_H] = {0.0f}, fvm[EO_H * EO_H] = {0.0f};
   if (n % 2 == 0)
     for (int i = 0; i < EO_H; ++i)
@@ -1424,8 +1306,6 @@ cudaError_t upload(const DgTables &t) {
         vm[i * EO_H + m] = 0.5 * (a - b);
         fvp[i * EO_H + m] = (float)vp[i * EO_H + m];
         fvm[i * EO_H + m] = (float)vm[i * EO_H + m];
-        fp_[i * EO_H + m] = 0.5 * (t.D[i * n + m] + t.D[i * n + (N - m)]);
-        fm_[i * EO_H + m] = 0.5 * (t.D[i * n + m] - t.D[i * n + (N - m)]);
       }
   double ihx[n];
   float fihx[n];
@@ -1433,13 +1313,12 @@ cudaError_t upload(const DgTables &t) {
   for (int i = 1; i < n; ++i) ihx[i] = 1.0 / (t.xi[i] - t.xi[i - 1]);
   for (int i = 0; i < n; ++i) fihx[i] = (float)ihx[i];
   cudaError_t err = fx_upload(t);
+  err = err ? err : fx_lift_upload(t);
   err = err ? err : cudaMemcpyToSymbol(c_ihx, ihx, sizeof(double) * n);
   err = err ? err : cudaMemcpyToSymbol(c_VP, vp, sizeof(vp));
   err = err ? err : cudaMemcpyToSymbol(c_VM, vm, sizeof(vm));
   err = err ? err : cudaMemcpyToSymbol(f_VP, fvp, sizeof(fvp));
   err = err ? err : cudaMemcpyToSymbol(f_VM, fvm, sizeof(fvm));
-  err = err ? err : cudaMemcpyToSymbol(c_FP, fp_, sizeof(fp_));
-  err = err ? err : cudaMemcpyToSymbol(c_FM, fm_, sizeof(fm_));
   err = err ? err : cudaMemcpyToSymbol(f_ihx, fihx, sizeof(float) * n);
   err = err ? err : cudaMemcpyToSymbol(c_D, t.D, sizeof(double) * nn);
   err = err ? err : cudaMemcpyToSymbol(c_D2, D2, sizeof(double) * nn);
@@ -1472,7 +1351,7 @@ void launch_face_normals(const DgDevice &d, cudaStream_t s) {
   const long long pts = (long long)d.nF * nn;
   k_face_normals<<<(unsigned)((pts + 255) / 256), 256, 0, s>>>(d);
   if (d.precision == 1) k_round_geometry<<<4 * 152, 256, 0, s>>>(d);
-  else k_metric_max<<<d.nE, 128, 0, s>>>(d);
+  else k_metric_max<<<(d.nE + 3) / 4, 128, 0, s>>>(d);
 }
 
 template <typename R>
@@ -1506,19 +1385,16 @@ void launch_lift(const DgDevice &d, const double *U, double *tau, cudaStream_t s
     k_lift_f32_tma<<<blocks, LT_THREADS, LT_SMEM, s>>>(d);
     return;
   }
-  const unsigned grid = (d.nE + LIFT_EPB - 1) / LIFT_EPB;
   if (d.precision == 1) {
-    k_lift<float><<<grid, LIFT_THREADS, 0, s>>>(d, U, nullptr);
-  } else if (n == 8) {  // measured faster at N = 7 (7.32 -> 7.00 ms at 32^3); slower at N = 5 (+3 %)
-    static bool attr_set = false;
-    if (!attr_set) {
-      cudaFuncSetAttribute(k_lift_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIFT_LINES_SMEM);
-      attr_set = true;
-    }
-    k_lift_lines<<<grid, LIFT_THREADS, LIFT_LINES_SMEM, s>>>(d, U, tau);
-  } else {
-    k_lift<double><<<grid, LIFT_THREADS, 0, s>>>(d, U, tau);
+    k_lift<<<(d.nE + LIFT_EPB - 1) / LIFT_EPB, LIFT_THREADS, 0, s>>>(d);
+    return;
   }
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaFuncSetAttribute(k_lift_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FXL_SMEM);
+    attr_set = true;
+  }
+  k_lift_fx<<<(d.nE + FX_EPB - 1) / FX_EPB, FX_THREADS, FXL_SMEM, s>>>(d, U, tau);
 }
 
 template <typename R, int VF, bool SC>

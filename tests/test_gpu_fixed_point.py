@@ -1,6 +1,6 @@
-"""The FP64 volume kernel's fixed-point arithmetic (KG and Pirozzoli fluxes) where its scales can go
-wrong: flows at rest and at extreme Mach numbers, viscous fluxes above and far below the advective
-ones, units far from 1, and elements whose values span too much for one scale (the kernel's general
+"""The fixed-point arithmetic of the FP64 volume kernel (KG and Pirozzoli fluxes) and lifting where its
+scales can go wrong: flows at rest and at extreme Mach numbers, viscous fluxes above and far below the advective
+ones or none at all (the lifting's general path), units far from 1, and elements whose values span too much for one scale (the kernel's general
 FP64 path), at every degree parity and with ragged element counts per block. The bound is the normwise one
 of the other FP64 parity tests, ULP_FACTOR times the oracle's own spread under one-ulp perturbations of its
 inputs (tests/helpers.py); their flux scale holds the advective flux only, which is not the largest term here.
@@ -41,13 +41,13 @@ def _fields(xyz, seed, mach):
     return rho, vel, p
 
 
-STATES = ["rest", "mach_1e-6", "mach_1", "mach_30", "viscous", "units", "range_ok", "range_general"]
+STATES = ["rest", "mach_1e-6", "mach_1", "mach_30", "viscous", "mu_0", "units", "range_ok", "range_general"]
 
 
 def _state(kind, xyz, N):
     mach = {"rest": 0.0, "mach_1e-6": 1e-6, "mach_30": 30.0}.get(kind, 0.5)
     rho, vel, p = _fields(xyz, N, mach)
-    mu = {"viscous": 50.0, "rest": 0.1}.get(kind, 1e-3)
+    mu = {"viscous": 50.0, "rest": 0.1, "mu_0": 0.0}.get(kind, 1e-3)
     if kind == "units":
         rho, p, mu = 1e-9 * rho, 1e5 * p, 1e-12
         vel = [1e6 * v for v in vel]
