@@ -42,8 +42,8 @@ enum { DG_EULER = 0, DG_NAVIER_STOKES = 1 };
 enum { DG_VFLUX_KG = 0, DG_VFLUX_PIROZZOLI = 1, DG_VFLUX_EC = 2, DG_VFLUX_CENTRAL = 3 };
 /* surface Riemann fluxes */
 enum { DG_SFLUX_LLF = 0, DG_SFLUX_ROE = 1, DG_SFLUX_EC = 2 };
-/* DG_FP64: FP64 state, geometry and results; all arithmetic FP64 or, in the volume operator of the KG and
- * Pirozzoli fluxes without the blend, 64-bit fixed point scaled per element, whose rounding error is below
+/* DG_FP64: FP64 state, geometry and results; all arithmetic FP64 or, in the lifting and in the volume
+ * operator of the KG and Pirozzoli fluxes, 64-bit fixed point scaled per element, whose rounding error is below
  * FP64's. DG_FP32_BULK: volume/surface/lifting arithmetic in FP32 with FP32
  * accumulation; LSERK state, metrics, Jacobian scaling and reductions stay FP64. U, Ut stay FP64. */
 enum { DG_FP64 = 0, DG_FP32_BULK = 1 };

@@ -1,5 +1,4 @@
-// dg_fixed.cuh -- the FP64 volume kernel for the Kennedy-Gruber and Pirozzoli fluxes without the blend,
-// its two-point fluxes and viscous divergence evaluated in 64-bit fixed point on the integer pipes. Part
+// dg_fixed.cuh -- the FP64 volume kernel for the Kennedy-Gruber and Pirozzoli fluxes, its two-point fluxes and viscous divergence evaluated in 64-bit fixed point on the integer pipes. Part
 // of dg_kernels.cuh (same unnamed namespace); works on the degree constants defined there.
 //
 // Why: GB300 issues FP64 arithmetic at 2 lanes per clock and SM, IMAD.WIDE at 25 and 64-bit integer adds
@@ -277,6 +276,82 @@ __device__ __noinline__ void fx_general_node(const DgDevice &d, const double *S,
   }
 }
 
+// FV subcell operator of the blend (Sec. 4.1), in FP64 (see line_fv for the operator). It is bound by the FP64 pipe
+// (~280 instructions per interface with LLF); one thread per interface keeps a troubled element's critical path at
+// three solves per thread, where a thread per line ran N of them in a row on half the threads. Right-hand side's
+// volume part per launch, N = 5, 24^3, LLF, blend on every element: 4.74 (FP64 line kernel) -> 3.51 ms; N = 3, 32^3:
+// 2.57 -> 2.40 ms; without troubled elements (blast, N = 5, 32^3): 3.91 -> 1.35 ms.
+// Staged slots of an
+// element under the blend, after the pair phase: 0-4 rho, u, v, w, p; from slot 6 on the interface fluxes
+// [3 dir][N interfaces][5][nn lines].
+__constant__ double c_Ct[N * n];  // interface metric i + 1/2 = sum_m c_Ct[i][m] Ja_m = Ja_0 + sum_{k <= i} w_k (D Ja)_k
+
+// minmod of two slopes; signs and magnitudes compared as integers, which keeps it off the FP64 pipe
+__device__ __forceinline__ double fv_minmod(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b), m = 0x7fffffffffffffffll;
+  return (x ^ y) < 0 || (x & m) == 0 || (y & m) == 0 ? 0.0 : ((x & m) < (y & m) ? a : b);
+}
+
+// a Riemann side from (rho, u, v, w, p)
+__device__ __forceinline__ void fv_side(const double q[5], double igm1, RSide<double> &s) {
+  s.rs = rsq(q[0]);
+  s.ir = s.rs * s.rs;
+  s.U[0] = q[0];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) { s.u[c] = q[1 + c]; s.U[1 + c] = q[0] * q[1 + c]; }
+  s.pm = s.p = q[4];
+  s.U[4] = q[4] * igm1 + 0.5 * (s.U[1] * q[1] + s.U[2] * q[2] + s.U[3] * q[3]);
+}
+
+// flux through interface i + 1/2 of one line, into out [5][nn]: the states of subcells i and i + 1 there (minmod
+// slopes inside, first order in the outer subcells and where a reconstruction loses positivity), each slope's
+// difference formed once
+__device__ __noinline__ void fv_interface(const DgDevice &d, const double *__restrict__ P, int pb, int ps,
+                                          const double *__restrict__ Jd, int gs, int i, double *__restrict__ out) {
+  double qL[5], qR[5], a[3], F[5];
+  {
+    const int p0 = pb + i * ps, bk = i > 0 ? -ps : 0, fw = i + 1 < N ? 2 * ps : ps;
+    const double hb = c_ihx[i], hc = c_ihx[i + 1], hf = i + 1 < N ? c_ihx[i + 2] : 0.0;
+    const double xL = c_xi[i], xR = c_xi[i + 1], lm = c_xh[i] - xL, lp = c_xh[i + 1] - xL, rm = c_xh[i + 1] - xR,
+                 rp = c_xh[i + 2] - xR;
+    double l0[5], r0[5];
+    bool okL = true, okR = true;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const double *Pv = P + v * FX_PS + p0;
+      const double q0 = Pv[0], q1 = Pv[ps], dc = (q1 - q0) * hc;
+      const double sL = fv_minmod((q0 - Pv[bk]) * hb, dc), sR = fv_minmod(dc, (Pv[fw] - q1) * hf);
+      l0[v] = q0;
+      r0[v] = q1;
+      qL[v] = q0 + sL * lp;
+      qR[v] = q1 + sR * rm;
+      if (v == 0 || v == 4) {
+        okL = okL && qL[v] > 0.0 && q0 + sL * lm > 0.0;
+        okR = okR && qR[v] > 0.0 && q1 + sR * rp > 0.0;
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      if (!okL) qL[v] = l0[v];
+      if (!okR) qR[v] = r0[v];
+    }
+  }
+  RSide<double> L, R;
+  fv_side(qL, d.igm1, L);
+  fv_side(qR, d.igm1, R);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    a[c] = 0.0;
+#pragma unroll
+    for (int m = 0; m < n; ++m) a[c] += c_Ct[i * n + m] * __ldg(Jd + c * nnn + m * gs);
+  }
+  const double a2 = a[0] * a[0] + a[1] * a[1] + a[2] * a[2], is = rsq(a2), s = a2 * is;
+  const double nv[3] = {a[0] * is, a[1] * is, a[2] * is};
+  riemann_sides<double>(d.sflux, L, R, nv, d.gamma, 0.0, 0.0, F);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) out[v * nn] = s * F[v];
+}
+
 // One thread per node. What bounds it: instruction issue (55 % of the slots) with the FP64 pipe at 36 %, FMA-heavy
 // (IMAD.WIDE) at 44 %, ALU at 52 % and DRAM at 15 %; 64 registers and 21 slots of shared memory keep two CTAs
 // (32 warps) per SM at N = 7. A thread per line (half the pair evaluations' overhead, sums in 80 registers,
@@ -288,7 +363,7 @@ constexpr int FX_THREADS = round32(FX_EPB * nnn);
 constexpr size_t FX_SMEM = sizeof(fx_t) * FX_EPB * FX_SLOTS * FX_PS;
 constexpr int FX_MINB = 1024 / FX_THREADS < 32 ? 1024 / FX_THREADS : 32;  // 64 registers per thread
 
-template <int VF>
+template <int VF, bool SC>
 __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
     k_volume_fx(const DgDevice d, const double *U, double *out, double *__restrict__ g, int mode, int first, double dt,
                 double A, double B) {
@@ -420,46 +495,111 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
     for (int k = 0; k < 6; ++k) Se[k * FX_PS] = q[k];
   }
   __syncthreads();
-  if (!on) return;
-  // phase C: per node -- directions summed, surface terms, neighbour's viscous flux, Jacobian, output / LSERK
+  // phase C: per node -- directions summed, surface terms, neighbour's viscous flux, blend, Jacobian, output / LSERK
   const int ijk[3] = {node % n, (node / n) % n, node / nn};
   double s[5];
-  if (ok) {
-    const fx_t *Se = S + le * FX_SLOTS * FX_PS + fx_idx(node);
-    const int a0 = min(ijk[0], N - ijk[0]), a1 = min(ijk[1], N - ijk[1]), a2 = min(ijk[2], N - ijk[2]);
-    const int am = min(a0, min(a1, a2));  // the direction with the smallest weight
-    const FxD r0 = fx_const(s_rho[a0 * FX_H + am]), r1 = fx_const(s_rho[a1 * FX_H + am]),
-              r2 = fx_const(s_rho[a2 * FX_H + am]);
-    const double iw = c_invw[am];
-    const int iwh = __double2hiint(iw), iwl = __double2loint(iw);
-    const int k0 = s_sc[le].k0, km = s_sc[le].km, ke = s_sc[le].ke;
+  if (on) {
+    if (ok) {
+      const fx_t *Se = S + le * FX_SLOTS * FX_PS + fx_idx(node);
+      const int a0 = min(ijk[0], N - ijk[0]), a1 = min(ijk[1], N - ijk[1]), a2 = min(ijk[2], N - ijk[2]);
+      const int am = min(a0, min(a1, a2));  // the direction with the smallest weight
+      const FxD r0 = fx_const(s_rho[a0 * FX_H + am]), r1 = fx_const(s_rho[a1 * FX_H + am]),
+                r2 = fx_const(s_rho[a2 * FX_H + am]);
+      const double iw = c_invw[am];
+      const int iwh = __double2hiint(iw), iwl = __double2loint(iw);
+      const int k0 = s_sc[le].k0, km = s_sc[le].km, ke = s_sc[le].ke;
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      FxSum f0{0, 0x40000000ll}, f1 = f0, f2 = f0;  // the three lo sums do not fit one
-      fx_acc(f0, r0, fx_split(Se[fx_slot(0, v) * FX_PS]));
-      fx_acc(f1, r1, fx_split(Se[fx_slot(1, v) * FX_PS]));
-      fx_acc(f2, r2, fx_split(Se[fx_slot(2, v) * FX_PS]));
-      // half the sum of the three directions (the factors carry 2^62)
-      const fx_t sum = ((f0.hi + f1.hi + f2.hi) << 1) + (f0.lo >> 31) + (f1.lo >> 31) + (f2.lo >> 31);
-      s[v] = (double)sum * __hiloint2double(iwh + (int)((unsigned)(v == 0 ? k0 : v < 4 ? km : ke) << 20), iwl);
+      for (int v = 0; v < 5; ++v) {
+        FxSum f0{0, 0x40000000ll}, f1 = f0, f2 = f0;  // the three lo sums do not fit one
+        fx_acc(f0, r0, fx_split(Se[fx_slot(0, v) * FX_PS]));
+        fx_acc(f1, r1, fx_split(Se[fx_slot(1, v) * FX_PS]));
+        fx_acc(f2, r2, fx_split(Se[fx_slot(2, v) * FX_PS]));
+        // half the sum of the three directions (the factors carry 2^62)
+        const fx_t sum = ((f0.hi + f1.hi + f2.hi) << 1) + (f0.lo >> 31) + (f1.lo >> 31) + (f2.lo >> 31);
+        s[v] = (double)sum * __hiloint2double(iwh + (int)((unsigned)(v == 0 ? k0 : v < 4 ? km : ke) << 20), iwl);
+      }
+    } else {
+      double sg[5];
+      fx_general_node<VF>(d, reinterpret_cast<const double *>(S) + le * FX_SLOTS * FX_PS, e, node, sg);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) s[v] = sg[v];
     }
-  } else {
-    double sg[5];
-    fx_general_node<VF>(d, reinterpret_cast<const double *>(S) + le * FX_SLOTS * FX_PS, e, node, sg);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) s[v] = sg[v];
+    for (int dd = 0; dd < 3; ++dd) {
+      const int id = ijk[dd];
+      if (id != 0 && id != N) continue;
+      const int f = 2 * dd + (id == N ? 1 : 0);
+      const int pp = dd == 0 ? ijk[1] : ijk[0], qq = dd == 2 ? ijk[1] : ijk[2];
+      const double *fs = d.Fsurf + ((size_t)e * 6 + f) * 5 * nn + pp + n * qq;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) s[v] += c_invw[0] * fs[v * nn];
+    }
   }
+  if constexpr (SC) {  // blend with the FV subcell operator where alpha > 0
+    const double al = on ? d.alpha[e] : 0.0;
+    if (__syncthreads_or(al > 0.0)) {
+      double *P0 = reinterpret_cast<double *>(S);
+      if (al > 0.0) {
+        double Uv[5];
+        load_state<double>(d, U, e, node, Uv);
+        const double ir = 1.0 / Uv[0];
+        const double u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
+        double *P = P0 + le * FX_SLOTS * FX_PS + fx_idx(node);
+        P[0] = Uv[0]; P[FX_PS] = u; P[2 * FX_PS] = v; P[3 * FX_PS] = w;
+        P[4 * FX_PS] = gm1 * (Uv[4] - 0.5 * (Uv[1] * u + Uv[2] * v + Uv[3] * w));
+      }
+      __syncthreads();
+      // one thread per interface of a line
+      for (int t = tid; t < FX_EPB * 3 * N * nn; t += FX_THREADS) {
+        const int lt = t / (3 * N * nn), r = t % (3 * N * nn), dir = r / (N * nn), i = (r / nn) % N, line = r % nn;
+        const int et = e0 + lt;
+        if (et >= d.nE || !(d.alpha[et] > 0.0)) continue;
+        const int la = line % n, lb = line / n;
+        const int ps = dir == 0 ? 1 : dir == 1 ? FX_SJ : FX_SK, gs = dir == 0 ? 1 : dir == 1 ? n : nn;
+        const int pb = dir == 0 ? FX_SJ * la + FX_SK * lb : dir == 1 ? la + FX_SK * lb : la + FX_SJ * lb;
+        const int gb = dir == 0 ? n * (la + n * lb) : dir == 1 ? la + nn * lb : la + n * lb;
+        double *P = P0 + lt * FX_SLOTS * FX_PS;
+        fv_interface(d, P, pb, ps, d.Ja + ((size_t)et * 3 + dir) * 3 * nnn + gb, gs, i,
+                     P + 6 * FX_PS + (dir * N + i) * 5 * nn + line);
+      }
+      __syncthreads();
+      if (al > 0.0) {
+        const double *Fi = P0 + le * FX_SLOTS * FX_PS + 6 * FX_PS;
+        double fv[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-  for (int dd = 0; dd < 3; ++dd) {
-    const int id = ijk[dd];
-    if (id != 0 && id != N) continue;
-    const int f = 2 * dd + (id == N ? 1 : 0);
-    const int pp = dd == 0 ? ijk[1] : ijk[0], qq = dd == 2 ? ijk[1] : ijk[2];
-    const double iwb = c_invw[0];
-    const double *fs = d.Fsurf + ((size_t)e * 6 + f) * 5 * nn + pp + n * qq;
+        for (int dd = 0; dd < 3; ++dd) {
+          const int id = ijk[dd];
+          const int line = (dd == 0 ? ijk[1] : ijk[0]) + n * (dd == 2 ? ijk[1] : ijk[2]);  // = the faces' point
+          const double *fl = id > 0 ? Fi + (dd * N + id - 1) * 5 * nn + line
+                                    : d.Fsurf + ((size_t)e * 6 + 2 * dd) * 5 * nn + line;
+          const double *fr = id < N ? Fi + (dd * N + id) * 5 * nn + line
+                                    : d.Fsurf + ((size_t)e * 6 + 2 * dd + 1) * 5 * nn + line;
+          const double iw = c_invw[min(id, N - id)];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) s[v] += iwb * fs[v * nn];
-    if (ns) {  // -(1/(2 w_b)) phi_nb, phi_nb = neighbour's outward normal viscous flux; or the wall's
+          for (int v = 0; v < 5; ++v) fv[v] += iw * (id > 0 ? fr[v * nn] - fl[v * nn] : fr[v * nn] + fl[v * nn]);
+        }
+#pragma unroll
+        for (int v = 0; v < 5; ++v) s[v] = al * fv[v] + (1.0 - al) * s[v];
+        if (ns)  // the line sums hold the viscous divergence too, which the blend must not weight
+          for (int dd = 0; dd < 3; ++dd) {
+            const int id = ijk[dd], st = dd == 0 ? 1 : dd == 1 ? n : nn;
+            const double *Fv = d.Fv + ((size_t)e * 12 + dd * 4) * nnn + node - id * st;
+            for (int m = 0; m < n; ++m)
+              if (m != id)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) s[1 + v] -= al * c_D[id * n + m] * Fv[v * nnn + m * st];
+          }
+      }
+    }
+  }
+  if (!on) return;
+  if (ns) {  // -(1/(2 w_b)) phi_nb, phi_nb = neighbour's outward normal viscous flux; or the wall's
+#pragma unroll
+    for (int dd = 0; dd < 3; ++dd) {
+      const int id = ijk[dd];
+      if (id != 0 && id != N) continue;
+      const int f = 2 * dd + (id == N ? 1 : 0);
+      const int pp = dd == 0 ? ijk[1] : ijk[0], qq = dd == 2 ? ijk[1] : ijk[2];
       const int *ef = d.ef + ((size_t)e * 6 + f) * 4;
       const int nb = ef[0], fnb = ef[1], o = ef[2];
       if (nb < 0) {
@@ -467,11 +607,11 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
         const double hs = (id == N) ? 0.5 : -0.5;
         const double *Fve = d.Fv + ((size_t)e * 12 + dd * 4) * nnn + node;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) s[1 + v] -= iwb * (fw[v * nn] - hs * Fve[v * nnn]);
+        for (int v = 0; v < 4; ++v) s[1 + v] -= c_invw[0] * (fw[v * nn] - hs * Fve[v * nnn]);
       } else {
         int p2, q2;
         orient_map(o, pp, qq, p2, q2);
-        const double sg = (fnb & 1) ? 0.5 * iwb : -0.5 * iwb;
+        const double sg = (fnb & 1) ? 0.5 * c_invw[0] : -0.5 * c_invw[0];
         const double *Fvn = d.Fv + ((size_t)nb * 12 + (fnb >> 1) * 4) * nnn + face_node(fnb, p2, q2);
 #pragma unroll
         for (int v = 0; v < 4; ++v) s[1 + v] += sg * Fvn[v * nnn];
@@ -546,7 +686,16 @@ cudaError_t fx_upload(const DgTables &t) {
     }
   for (int a = 0; a < FX_H; ++a)
     for (int b = 0; b < FX_H; ++b) rho[a * FX_H + b] = fx_halves(t.wl[a < b ? a : b] / t.wl[a], 62);
+  double Ct[N * n];
+  for (int m = 0; m < n; ++m) {
+    long double acc = m == 0 ? 1.0L : 0.0L;
+    for (int i = 0; i < N; ++i) {
+      acc += t.Q[i * n + m] + (i == m && i == 0 ? -0.5L : 0.0L);  // (D_ii = 0 inside, w_0 D_00 = -1/2)
+      Ct[i * n + m] = (double)acc;
+    }
+  }
   cudaError_t err = cudaMemcpyToSymbol(c_Qx, Q, sizeof(Q));
+  err = err ? err : cudaMemcpyToSymbol(c_Ct, Ct, sizeof(Ct));
   err = err ? err : cudaMemcpyToSymbol(c_QV, QV, sizeof(QV));
   return err ? err : cudaMemcpyToSymbol(c_rho, rho, sizeof(rho));
 }

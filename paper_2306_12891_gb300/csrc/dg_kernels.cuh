@@ -232,25 +232,23 @@ __global__ void __launch_bounds__(256) k_shadow(const DgDevice d, const double *
 __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
 
-// Euler flux through the (unit or metric) vector a, given ir = 1/rho; returns u.a and the true
-// pressure p
+// one side of a Riemann problem: conservative state, velocity, p' and the true pressure, 1/sqrt(rho), 1/rho
 template <typename R>
-__device__ __forceinline__ void euler_flux_ir(const R U[5], R ir, R gam, R pref, R href, const R a[3], R F[5], R &un,
-                                              R &p) {
-  const R u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
-  const R pm = (gam - R(1)) * (U[4] - R(0.5) * (U[1] * u + U[2] * v + U[3] * w));  // p'
-  un = u * a[0] + v * a[1] + w * a[2];
-  F[0] = U[0] * un;
-  F[1] = U[1] * un + pm * a[0];
-  F[2] = U[2] * un + pm * a[1];
-  F[3] = U[3] * un + pm * a[2];
-  if (kShift<R>) {
-    p = pm + pref;
-    F[4] = (U[4] + pm + href) * un;  // E + p = E' + p' + gamma p_ref/(gamma-1)
-  } else {
-    p = pm;
-    F[4] = (U[4] + pm) * un;
-  }
+struct RSide {
+  R U[5], u[3], pm, p, rs, ir;
+};
+
+// Euler flux of one side through the unit vector a; returns u.a
+template <typename R>
+__device__ __forceinline__ R euler_flux(const RSide<R> &s, R href, const R a[3], R F[5]) {
+  const R un = s.u[0] * a[0] + s.u[1] * a[1] + s.u[2] * a[2];
+  F[0] = s.U[0] * un;
+  F[1] = s.U[1] * un + s.pm * a[0];
+  F[2] = s.U[2] * un + s.pm * a[1];
+  F[3] = s.U[3] * un + s.pm * a[2];
+  // E + p = E' + p' + gamma p_ref/(gamma-1)
+  F[4] = kShift<R> ? (s.U[4] + s.pm + href) * un : (s.U[4] + s.pm) * un;
+  return un;
 }
 
 template <typename R>
@@ -283,27 +281,32 @@ __device__ __forceinline__ void ec_flux(R rL, R uL, R vL, R wL, R pL, R rR, R uR
          pref * (um * a[0] + vm * a[1] + wm * a[2]);
 }
 
-// Riemann flux F*(UL, UR, nv) for a unit normal nv; also returns each side's 1/rho and true pressure
-// (the face kernel's BR1 face values reuse them)
+// the side's velocity and pressure from its conservative state. One reciprocal square root: 1/sqrt(rho);
+// 1/rho is its square and sqrt(rho) = rho/sqrt(rho)
 template <typename R>
-__device__ __forceinline__ void riemann(int sf, const R UL[5], const R UR[5], const R nv[3], R gam, R pref, R href,
-                                        R F[5], R &irL, R &irR, R &pL, R &pR) {
+__device__ __forceinline__ void side_from_cons(R gm1, R pref, RSide<R> &s) {
+  s.rs = rsq(s.U[0]);
+  s.ir = s.rs * s.rs;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) s.u[c] = s.U[1 + c] * s.ir;
+  s.pm = gm1 * (s.U[4] - R(0.5) * (s.U[1] * s.u[0] + s.U[2] * s.u[1] + s.U[3] * s.u[2]));  // p'
+  s.p = kShift<R> ? s.pm + pref : s.pm;
+}
+
+// Riemann flux F*(L, R, nv) of two sides for a unit normal nv
+template <typename R>
+__device__ __forceinline__ void riemann_sides(int sf, const RSide<R> &L, const RSide<R> &Q, const R nv[3], R gam,
+                                              R pref, R href, R F[5]) {
   const R gm1 = gam - R(1);
-  // one reciprocal square root per side: 1/sqrt(rho); 1/rho is its square and sqrt(rho) = rho/sqrt(rho)
-  const R rsL = rsq(UL[0]), rsR = rsq(UR[0]);
-  irL = rsL * rsL;
-  irR = rsR * rsR;
+  const R *UL = L.U, *UR = Q.U;
+  const R irL = L.ir, irR = Q.ir, rsL = L.rs, rsR = Q.rs, pL = L.p, pR = Q.p;
+  const R uL = L.u[0], vL = L.u[1], wL = L.u[2], uR = Q.u[0], vR = Q.u[1], wR = Q.u[2];
   if (sf == SF_EC) {
-    const R uL = UL[1] * irL, vL = UL[2] * irL, wL = UL[3] * irL;
-    const R uR = UR[1] * irR, vR = UR[2] * irR, wR = UR[3] * irR;
-    pL = gm1 * (UL[4] - R(0.5) * (UL[1] * uL + UL[2] * vL + UL[3] * wL)) + (kShift<R> ? pref : R(0));
-    pR = gm1 * (UR[4] - R(0.5) * (UR[1] * uR + UR[2] * vR + UR[3] * wR)) + (kShift<R> ? pref : R(0));
     ec_flux<R>(UL[0], uL, vL, wL, pL, UR[0], uR, vR, wR, pR, nv, gam, kShift<R> ? pref : R(0), F);
     return;
   }
-  R FL[5], FR[5], unL, unR;
-  euler_flux_ir<R>(UL, irL, gam, pref, href, nv, FL, unL, pL);
-  euler_flux_ir<R>(UR, irR, gam, pref, href, nv, FR, unR, pR);
+  R FL[5], FR[5];
+  const R unL = euler_flux<R>(L, href, nv, FL), unR = euler_flux<R>(Q, href, nv, FR);
   if (sf == SF_LLF) {
     const R cL = sqrt(gam * pL * irL), cR = sqrt(gam * pR * irR);
     const R lam = fmax(fabs(unL) + cL, fabs(unR) + cR);
@@ -317,8 +320,6 @@ __device__ __forceinline__ void riemann(int sf, const R UL[5], const R UR[5], co
   const R sL = UL[0] * rsL, sR = UR[0] * rsR;
   const R iw = R(1) / (sL + sR);
   const R aL = rsL * iw, aR = rsR * iw;
-  const R uL = UL[1] * irL, vL = UL[2] * irL, wL = UL[3] * irL;
-  const R uR = UR[1] * irR, vR = UR[2] * irR, wR = UR[3] * irR;
   const R ut = aL * UL[1] + aR * UR[1], vt = aL * UL[2] + aR * UR[2], wt = aL * UL[3] + aR * UR[3];
   const R EpL = kShift<R> ? UL[4] + pL - pref + href : UL[4] + pL;  // E + p
   const R EpR = kShift<R> ? UR[4] + pR - pref + href : UR[4] + pR;
@@ -349,6 +350,20 @@ __device__ __forceinline__ void riemann(int sf, const R UL[5], const R UR[5], co
   D[4] = s15 * Ht + c15 * unt + l2a2 * R(0.5) * q2 + l2r * (ut * dut + vt * dvt + wt * dwt);
 #pragma unroll
   for (int v = 0; v < 5; ++v) F[v] = R(0.5) * (FL[v] + FR[v] - D[v]);
+}
+
+// the same from two conservative states; also returns each side's 1/rho and true pressure (the face kernel's BR1
+// face values reuse them)
+template <typename R>
+__device__ __forceinline__ void riemann(int sf, const R UL[5], const R UR[5], const R nv[3], R gam, R pref, R href,
+                                        R F[5], R &irL, R &irR, R &pL, R &pR) {
+  RSide<R> L, Q;
+#pragma unroll
+  for (int v = 0; v < 5; ++v) { L.U[v] = UL[v]; Q.U[v] = UR[v]; }
+  side_from_cons<R>(gam - R(1), pref, L);
+  side_from_cons<R>(gam - R(1), pref, Q);
+  irL = L.ir; irR = Q.ir; pL = L.p; pR = Q.p;
+  riemann_sides<R>(sf, L, Q, nv, gam, pref, href, F);
 }
 
 template <typename R>
@@ -1411,15 +1426,15 @@ void launch_volume_t(const DgDevice &d, const double *U, double *out, double *g,
                                                                                     B);
 }
 
-template <int VF>
+template <int VF, bool SC>
 void launch_volume_fx(const DgDevice &d, const double *U, double *out, double *g, int mode, int first, double dt,
                       double A, double B, cudaStream_t s) {
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_volume_fx<VF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
+    cudaFuncSetAttribute(k_volume_fx<VF, SC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
     attr_set = true;
   }
-  k_volume_fx<VF><<<(d.nE + FX_EPB - 1) / FX_EPB, FX_THREADS, FX_SMEM, s>>>(d, U, out, g, mode, first, dt, A, B);
+  k_volume_fx<VF, SC><<<(d.nE + FX_EPB - 1) / FX_EPB, FX_THREADS, FX_SMEM, s>>>(d, U, out, g, mode, first, dt, A, B);
 }
 
 template <int VF>
@@ -1485,11 +1500,11 @@ void launch_volume_f32(const DgDevice &d, const double *U, double *out, double *
   k_volume_f32<VF><<<(d.nE + NODE_EPB - 1) / NODE_EPB, NODE_THREADS, smem, s>>>(d, U, out, g, mode, first, dt, A, B);
 }
 
-// the blend (any flux), and in FP64 the fluxes that have no fixed-point form (EC, central): k_volume
+// k_volume: FP32 under the blend (any flux), and in FP64 the fluxes that have no fixed-point form (EC, central)
 template <typename R, bool SC>
 void launch_volume_lines(const DgDevice &d, const double *U, double *out, double *g, int mode, int first, double dt,
                          double A, double B, cudaStream_t s) {
-  if constexpr (SC) {
+  if constexpr (std::is_same<R, float>::value) {
     if (d.vflux == VF_KG) { launch_volume_t<R, VF_KG, SC>(d, U, out, g, mode, first, dt, A, B, s); return; }
     if (d.vflux == VF_PIR) { launch_volume_t<R, VF_PIR, SC>(d, U, out, g, mode, first, dt, A, B, s); return; }
   }
@@ -1499,9 +1514,9 @@ void launch_volume_lines(const DgDevice &d, const double *U, double *out, double
 
 void launch_volume(const DgDevice &d, const double *U, double *out, double *g, int mode, int first, double dt,
                    double A, double B, cudaStream_t s) {
-  if (d.shock_capturing) {
-    if (d.precision == 1) launch_volume_lines<float, true>(d, U, out, g, mode, first, dt, A, B, s);
-    else launch_volume_lines<double, true>(d, U, out, g, mode, first, dt, A, B, s);
+  const bool sc = d.shock_capturing != 0;
+  if (d.precision == 1 && sc) {
+    launch_volume_lines<float, true>(d, U, out, g, mode, first, dt, A, B, s);
   } else if (d.precision == 1) {
     switch (d.vflux) {
       case VF_KG: launch_volume_f32<VF_KG>(d, U, out, g, mode, first, dt, A, B, s); break;
@@ -1510,11 +1525,14 @@ void launch_volume(const DgDevice &d, const double *U, double *out, double *g, i
       default: launch_volume_f32<VF_CEN>(d, U, out, g, mode, first, dt, A, B, s); break;
     }
   } else if (d.vflux == VF_KG) {
-    launch_volume_fx<VF_KG>(d, U, out, g, mode, first, dt, A, B, s);
+    if (sc) launch_volume_fx<VF_KG, true>(d, U, out, g, mode, first, dt, A, B, s);
+    else launch_volume_fx<VF_KG, false>(d, U, out, g, mode, first, dt, A, B, s);
   } else if (d.vflux == VF_PIR) {
-    launch_volume_fx<VF_PIR>(d, U, out, g, mode, first, dt, A, B, s);
+    if (sc) launch_volume_fx<VF_PIR, true>(d, U, out, g, mode, first, dt, A, B, s);
+    else launch_volume_fx<VF_PIR, false>(d, U, out, g, mode, first, dt, A, B, s);
   } else {
-    launch_volume_lines<double, false>(d, U, out, g, mode, first, dt, A, B, s);
+    if (sc) launch_volume_lines<double, true>(d, U, out, g, mode, first, dt, A, B, s);
+    else launch_volume_lines<double, false>(d, U, out, g, mode, first, dt, A, B, s);
   }
 }
 
