@@ -1248,16 +1248,23 @@ __global__ void __launch_bounds__(256) k_invariants(const DgDevice d, const doub
   if (threadIdx.x < 8) d.red[blockIdx.x * 8 + threadIdx.x] = red[threadIdx.x][0];
 }
 
-__global__ void k_reduce_partials(const double *__restrict__ part, int nblocks, int width, int op_min, double *out) {
-  // one thread per output column, fixed summation order (deterministic)
-  const int c = threadIdx.x;
+// The partial results of the blocks, one warp per output column: lane l takes rows l, l + 32, ... in order, then a
+// shuffle tree (a fixed order: deterministic). One thread per column, 1024 dependent FP64 adds, took 34 us.
+__global__ void __launch_bounds__(256) k_reduce_partials(const double *__restrict__ part, int nblocks, int width,
+                                                         int op_min, double *out) {
+  const int c = threadIdx.x / 32, lane = threadIdx.x % 32;
   if (c >= width) return;
   double s = op_min ? part[c] : 0.0;
-  for (int b = op_min ? 1 : 0; b < nblocks; ++b) {
+  for (int b = lane; b < nblocks; b += 32) {
     const double x = part[b * width + c];
     s = op_min ? fmin(s, x) : s + x;
   }
-  out[c] = s;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double x = __shfl_down_sync(0xffffffffu, s, o);
+    s = op_min ? fmin(s, x) : s + x;
+  }
+  if (lane == 0) out[c] = s;
 }
 
 __global__ void __launch_bounds__(256) k_max_dt(const DgDevice d, const double *__restrict__ U) {
@@ -1551,7 +1558,7 @@ void launch_invariants(const DgDevice &d, const double *U, const double *Ut, dou
   int blocks = (int)((total + 255) / 256);
   if (blocks > DG_RED_BLOCKS) blocks = DG_RED_BLOCKS;
   k_invariants<<<blocks, 256, 0, s>>>(d, U, Ut);
-  k_reduce_partials<<<1, 32, 0, s>>>(d.red, blocks, 8, 0, out8);
+  k_reduce_partials<<<1, 256, 0, s>>>(d.red, blocks, 8, 0, out8);
 }
 
 void launch_max_dt(const DgDevice &d, const double *U, double *out, cudaStream_t s) {
