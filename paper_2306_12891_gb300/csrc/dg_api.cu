@@ -523,9 +523,6 @@ dg_status dg_init(const dg_mesh *mesh, int N, int nodes, const dg_params *prm, v
       DG_ALLOC(d.Fv_f, (size_t)nE * 12 * nnn);
     }
   } else {
-    DG_ALLOC(d.ijmax, (size_t)nE * 3);  // ijmax, jmax and fvmax, 8 bytes per element each
-    d.jmax = reinterpret_cast<int2 *>(d.ijmax + nE);
-    d.fvmax = reinterpret_cast<int *>(d.ijmax + 2 * (size_t)nE);
     DG_ALLOC(d.Fsurf, (size_t)nE * 6 * 5 * nn);
     if (prm->equations == DG_NAVIER_STOKES) {
       DG_ALLOC(d.Wsurf, (size_t)nE * 6 * 4 * nn);
@@ -540,8 +537,11 @@ dg_status dg_init(const dg_mesh *mesh, int N, int nodes, const dg_params *prm, v
       DG_ALLOC(d.Fwall, (size_t)nF * 4 * nn);
     }
   }
-  DG_ALLOC(d.alpha_raw, (size_t)nE);
-  DG_ALLOC(d.alpha, (size_t)nE);
+  DG_ALLOC(d.alpha_raw, (size_t)nE * 5);  // one allocation for the arrays with 8 bytes per element
+  d.alpha = d.alpha_raw + nE;
+  d.ijmax = d.alpha_raw + 2 * (size_t)nE;
+  d.jmax = reinterpret_cast<int2 *>(d.alpha_raw + 3 * (size_t)nE);
+  d.fvmax = reinterpret_cast<int *>(d.alpha_raw + 4 * (size_t)nE);
   DG_ALLOC(d.red, (size_t)DG_RED_DOUBLES);
   DG_ALLOC(d.flag, (size_t)1);
   DG_ALLOC(c->g, c->n_state);
