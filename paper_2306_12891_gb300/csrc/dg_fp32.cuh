@@ -23,7 +23,7 @@ constexpr int NODE_SLOTS = 7 + 9 + 12;  // staged primitives, metric terms, cont
 // P holds the staged quantities [7][nnn] (node index, no padding)
 template <int VF>
 __device__ __forceinline__ void pair_flux_f(const float *__restrict__ P, int a, int b, float Sjx, float Sjy,
-                                            float Sjz, float gam, float pref, float F[5]) {
+                                            float Sjz, float igm1, float pref, float F[5]) {
   const float ri = P[a], ui = P[nnn + a], vi = P[2 * nnn + a], wi = P[3 * nnn + a];
   const float rm = P[b], um = P[nnn + b], vm = P[2 * nnn + b], wm = P[3 * nnn + b];
   if (VF == VF_PIR || VF == VF_KG) {
@@ -39,7 +39,7 @@ __device__ __forceinline__ void pair_flux_f(const float *__restrict__ P, int a, 
   } else {
     const float av[3] = {0.5f * Sjx, 0.5f * Sjy, 0.5f * Sjz};
     if (VF == VF_EC) {
-      ec_flux<float>(ri, ui, vi, wi, P[6 * nnn + a], rm, um, vm, wm, P[6 * nnn + b], av, gam, pref, F);
+      ec_flux<float>(ri, ui, vi, wi, P[6 * nnn + a], rm, um, vm, wm, P[6 * nnn + b], av, igm1, pref, F);
     } else {
       const float Vi = ui * av[0] + vi * av[1] + wi * av[2], Vm = um * av[0] + vm * av[1] + wm * av[2];
       const float pm2 = 0.125f * (P[4 * nnn + a] + P[4 * nnn + b]);
@@ -66,7 +66,7 @@ __device__ __forceinline__ void f32_stage(const DgDevice &d, const float Uv[5], 
   Pn[0] = r; Pn[nnn] = u; Pn[2 * nnn] = v; Pn[3 * nnn] = w; Pn[4 * nnn] = 4.0f * pm;
   if (VF == VF_PIR) Pn[5 * nnn] = (Et + p) * ir;
   else if (VF == VF_KG) { Pn[5 * nnn] = Et * ir; Pn[6 * nnn] = 2.0f * p; }
-  else if (VF == VF_EC) Pn[6 * nnn] = p;
+  else if (VF == VF_EC) Pn[6 * nnn] = 0.5f * r / p;  // beta
   else Pn[5 * nnn] = Et + p;
 }
 
@@ -89,7 +89,7 @@ __device__ __forceinline__ void f32_node_terms(const DgDevice &d, const float *_
                                                const float *__restrict__ J, const float *__restrict__ F,
                                                const float *__restrict__ Fs, const float *__restrict__ Dz,
                                                int e, int node, float s[5]) {
-  const float gam = d.gamma_f, pref = d.p_ref_f;
+  const float igm1 = d.igm1_f, pref = d.p_ref_f;
   const bool ns = d.equations == 1;
   const int ijk[3] = {node % n, (node / n) % n, node / nn};
   float a[5];  // flux differencing with D
@@ -111,7 +111,7 @@ __device__ __forceinline__ void f32_node_terms(const DgDevice &d, const float *_
       const float c = Dr[m];
       float Fp[5];
       pair_flux_f<VF>(P, node, am, jx + J[(3 * dd) * nnn + am], jy + J[(3 * dd + 1) * nnn + am],
-                      jz + J[(3 * dd + 2) * nnn + am], gam, pref, Fp);
+                      jz + J[(3 * dd + 2) * nnn + am], igm1, pref, Fp);
 #pragma unroll
       for (int v = 0; v < 5; ++v) a[v] += c * Fp[v];
       if (ns) {  // viscous divergence along the line
@@ -587,7 +587,7 @@ __device__ __forceinline__ int ln_sw(int node) {
 template <int VF>
 __device__ __forceinline__ void pair_flux_reg(float ri, float ui, float vi, float wi, float p4i, float xi, float yi,
                                               float rm, float um, float vm, float wm, float p4m, float xm, float ym,
-                                              float Sjx, float Sjy, float Sjz, float gam, float pref, float F[5]) {
+                                              float Sjx, float Sjy, float Sjz, float igm1, float pref, float F[5]) {
   if (VF == VF_PIR || VF == VF_KG) {
     const float Su = ui + um, Sv = vi + vm, Sw = wi + wm;
     const float Vp = Su * Sjx + Sv * Sjy + Sw * Sjz;
@@ -601,7 +601,7 @@ __device__ __forceinline__ void pair_flux_reg(float ri, float ui, float vi, floa
   } else {
     const float av[3] = {0.5f * Sjx, 0.5f * Sjy, 0.5f * Sjz};
     if (VF == VF_EC) {
-      ec_flux<float>(ri, ui, vi, wi, yi, rm, um, vm, wm, ym, av, gam, pref, F);
+      ec_flux<float>(ri, ui, vi, wi, yi, rm, um, vm, wm, ym, av, igm1, pref, F);
     } else {
       const float Vi = ui * av[0] + vi * av[1] + wi * av[2], Vm = um * av[0] + vm * av[1] + wm * av[2];
       const float pm2 = 0.125f * (p4i + p4m);
@@ -621,19 +621,19 @@ struct LineRegs {
   float acc[n][5];
 };
 template <int VF, int I, int M>
-__device__ __forceinline__ void line_pairs(LineRegs &R, float gam, float pref) {
+__device__ __forceinline__ void line_pairs(LineRegs &R, float igm1, float pref) {
   if constexpr (I < n - 1) {
     float F[5];
     pair_flux_reg<VF>(R.r[I], R.u[I], R.v[I], R.w[I], R.p4[I], R.x[I], R.y[I], R.r[M], R.u[M], R.v[M], R.w[M],
-                      R.p4[M], R.x[M], R.y[M], R.jx[I] + R.jx[M], R.jy[I] + R.jy[M], R.jz[I] + R.jz[M], gam, pref, F);
+                      R.p4[M], R.x[M], R.y[M], R.jx[I] + R.jx[M], R.jy[I] + R.jy[M], R.jz[I] + R.jz[M], igm1, pref, F);
     const float ci = f_D[I * n + M], cm = f_D[M * n + I];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       R.acc[I][v] += ci * F[v];
       R.acc[M][v] += cm * F[v];
     }
-    if constexpr (M + 1 < n) line_pairs<VF, I, M + 1>(R, gam, pref);
-    else line_pairs<VF, I + 1, I + 2>(R, gam, pref);
+    if constexpr (M + 1 < n) line_pairs<VF, I, M + 1>(R, igm1, pref);
+    else line_pairs<VF, I + 1, I + 2>(R, igm1, pref);
   }
 }
 
@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(LN_THREADS, 1) k_volume_f32_line(const DgDevic
       const int dd = line ? ct / nn : 0, L = ct % nn, la = L % n, lb = L / n;
       const int st = dd == 0 ? 1 : dd == 1 ? n : nn;
       const int base = dd == 0 ? n * la + nn * lb : dd == 1 ? la + nn * lb : la + n * lb;
-      const float gam = d.gamma_f, pref = d.p_ref_f;
+      const float igm1 = d.igm1_f, pref = d.p_ref_f;
       const float iw0 = f_invw[0], iwN = f_invw[N];
       // face records of the line's two faces, loaded one element ahead (a warp issues in order: an
       // address computed from a just-loaded record would stall it for a full memory latency)
@@ -770,7 +770,7 @@ __global__ void __launch_bounds__(LN_THREADS, 1) k_volume_f32_line(const DgDevic
           for (int v = 0; v < 5; ++v) R.acc[i][v] = 0.0f;
         }
         // each pair (i, m), i < m, once: node i takes D_im F, node m takes D_mi F (F is symmetric)
-        line_pairs<VF, 0, 1>(R, gam, pref);
+        line_pairs<VF, 0, 1>(R, igm1, pref);
         float (&acc)[n][5] = R.acc;
         // surface terms: (1/w_b) times the outward face flux at the end nodes
 #pragma unroll
