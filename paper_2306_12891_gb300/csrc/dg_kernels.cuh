@@ -61,7 +61,6 @@ __constant__ double c_ihx[n];  // 1 / (xi_i - xi_{i-1}), i = 1..N (minmod slopes
 constexpr int EO_H = (n % 2 == 0) ? n / 2 : 1;
 __constant__ double c_VP[EO_H * EO_H], c_VM[EO_H * EO_H];
 __constant__ float f_VP[EO_H * EO_H], f_VM[EO_H * EO_H];
-__constant__ double c_Vinv[nn];
 __constant__ float f_D[nn], f_D2[nn], f_Dq[nn], f_De[nn];
 __constant__ float f_w[n], f_invw[n], f_xi[n], f_xh[n + 1], f_ihx[n];
 
@@ -1132,69 +1131,82 @@ namespace {
 // ---------------------------------------------------------------------------------------------
 // modified Persson indicator (Sec. 4.1, Eq. (7)) and the neighbour extension (FP64)
 // ---------------------------------------------------------------------------------------------
-// One warp per element (IND_WARPS elements per CTA): q = rho p staged in shared memory, its modal
-// coefficients by three tensor-product passes with the inverse Vandermonde (a padded shared-memory
-// copy, so lanes reading different rows do not serialise on constant memory), the shell energies
-// reduced with warp shuffles; no block-wide barrier after the table load. The kernel is bound by the
-// FP64 pipe, so it saves FP64 instructions:
-//  - q = rho p = (gamma - 1)(rho E - |m|^2 / 2), with no division;
-//  - each pass uses the parity of the Legendre modes on the symmetric LGL nodes,
-//    Vinv[a][N-i] = (-1)^a Vinv[a][i]: with q+-_i = q_i +- q_(N-i), output a needs the first half of
-//    row a against q+ (a even) or q- (a odd), n(n+1)/2 multiplies per line instead of n^2;
-//  - the threshold T of Eq. (7) and -s/T are per-context constants from the host.
+// One warp per element (IND_WARPS elements per CTA): q = rho p = (gamma - 1)(rho E - |m|^2 / 2) in FP64, its modal
+// coefficients by three tensor-product passes with the inverse Vandermonde in the 64-bit fixed point of
+// dg_fixed.cuh (scale: the element's largest |q|), the shell energies in FP64, reduced with warp shuffles; no
+// block-wide barrier after the table load. Each pass uses the parity of the Legendre modes on the symmetric
+// LGL nodes, Vinv[a][N-i] = (-1)^a Vinv[a][i]: output a needs the first half of row a against q_i + q_(N-i)
+// (a even) or q_i - q_(N-i) (a odd). Row sums of |Vinv| are below 1.5, so values stay below 2^59 x 1.5^3 and the
+// lo sums below 2^63. The threshold T of Eq. (7) and -s/T are per-context constants from the host. Measured at
+// N = 5, 32^3: 0.26 ms per launch, 0.61 with FP64 passes (FP64-bound).
 constexpr int IND_WARPS = 4;
 constexpr int IND_H = (n + 1) / 2;  // first half of a line, the middle node included when n is odd
+__constant__ int2 c_VI[n * IND_H];  // first halves of the rows of Vinv, 2^61 (the middle node's halved when n is odd)
 
 // one pass along a line of stride st starting at `base`: out[base + a st] = sum_i Vinv[a][i] in[base + i st]
-__device__ __forceinline__ void ind_pass(const double (*__restrict__ sV)[n + 1], const double *__restrict__ in,
-                                         double *__restrict__ out, int base, int st, int a) {
-  double s = 0.0;
-  const double sg = (a & 1) ? -1.0 : 1.0;
+__device__ __forceinline__ void ind_pass(const int2 *__restrict__ row, const fx_t *__restrict__ in,
+                                         fx_t *__restrict__ out, int base, int st, int a) {
+  FxSum s = fx_zero(3);
 #pragma unroll
-  for (int i = 0; i < n / 2; ++i) s += sV[a][i] * (in[base + i * st] + sg * in[base + (N - i) * st]);
-  if (n & 1) s += sV[a][N / 2] * in[base + (N / 2) * st];  // the middle node (odd n; zero for odd a)
-  out[base + a * st] = s;
+  for (int i = 0; i < IND_H; ++i) {
+    const fx_t x = in[base + i * st], y = in[base + (N - i) * st];
+    fx_acc(s, fx_const(row[i]), fx_split((a & 1) ? x - y : x + y));
+  }
+  out[base + a * st] = fx_value(s, 3);
 }
 
 __global__ void __launch_bounds__(32 * IND_WARPS) k_indicator(const DgDevice d, const double *__restrict__ U) {
-  __shared__ double sV[n][n + 1];
-  __shared__ double q[IND_WARPS][nnn], t1[IND_WARPS][nnn];
-  for (int t = threadIdx.x; t < nn; t += blockDim.x) sV[t / n][t % n] = c_Vinv[t];
+  constexpr int IR = (nnn + 31) / 32;
+  __shared__ int2 sV[n * IND_H];
+  __shared__ fx_t q[IND_WARPS][nnn], t1[IND_WARPS][nnn];
+  for (int t = threadIdx.x; t < n * IND_H; t += blockDim.x) sV[t] = c_VI[t];
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e = blockIdx.x * IND_WARPS + w;
   if (e >= d.nE) return;
   const double gm1 = d.gm1;
-  double *qw = q[w], *tw = t1[w];
+  fx_t *qw = q[w], *tw = t1[w];
+  int hi = 0;
+#pragma unroll 4
   for (int node = lane; node < nnn; node += 32) {
     const double *Ue = U + (size_t)e * 5 * nnn + node;
     const double r = Ue[0], m1 = Ue[nnn], m2 = Ue[2 * nnn], m3 = Ue[3 * nnn];
-    qw[node] = gm1 * (r * Ue[4 * nnn] - 0.5 * (m1 * m1 + m2 * m2 + m3 * m3));
+    const double x = gm1 * (r * Ue[4 * nnn] - 0.5 * (m1 * m1 + m2 * m2 + m3 * m3));
+    hi = max(hi, fx_hi_abs(x));
+    qw[node] = __double_as_longlong(x);
   }
-  __syncwarp();
-  for (int node = lane; node < nnn; node += 32) {  // xi: (i,j,k) -> (a,j,k)
-    const int a = node % n;
-    ind_pass(sV, qw, tw, node - a, 1, a);
-  }
-  __syncwarp();
-  for (int node = lane; node < nnn; node += 32) {  // eta
-    const int b = (node / n) % n;
-    ind_pass(sV, tw, qw, node - b * n, n, b);
-  }
-  __syncwarp();
-  for (int node = lane; node < nnn; node += 32) {  // zeta into t1
-    const int c = node / nn;
-    ind_pass(sV, qw, tw, node - c * nn, nn, c);
-  }
-  __syncwarp();
+  const int ex = fx_exponent(__reduce_max_sync(0xffffffffu, hi));
   double all = 0.0, shN = 0.0, shN1 = 0.0;
-  for (int node = lane; node < nnn; node += 32) {  // the shell energies
-    const int a = node % n, b = (node / n) % n, c = node / nn;
-    const int M = max(a, max(b, c));
-    const double m2 = tw[node] * tw[node];
-    all += m2;
-    if (M == N) shN += m2;
-    if (M == N - 1) shN1 += m2;
+  if (ex >= 525 && ex < 2047) {  // (energy ratios do not depend on the scale; below 1e-150 a zero indicator)
+    __syncwarp();
+    for (int node = lane; node < nnn; node += 32) qw[node] = fx_from(__longlong_as_double(qw[node]), ex, 4);
+    __syncwarp();
+    for (int node = lane; node < nnn; node += 32) {  // xi: (i,j,k) -> (a,j,k)
+      const int a = node % n;
+      ind_pass(sV + a * IND_H, qw, tw, node - a, 1, a);
+    }
+    __syncwarp();
+    for (int node = lane; node < nnn; node += 32) {  // eta
+      const int b = (node / n) % n;
+      ind_pass(sV + b * IND_H, tw, qw, node - b * n, n, b);
+    }
+    __syncwarp();
+    for (int node = lane; node < IR * 32; node += 32) {  // zeta, then the shell energies
+      if (node >= nnn) continue;
+      const int c = node / nn;
+      ind_pass(sV + c * IND_H, qw, tw, node - c * nn, nn, c);
+    }
+    __syncwarp();
+    for (int node = lane; node < nnn; node += 32) {
+      const int a = node % n, b = (node / n) % n, c = node / nn;
+      const int M = max(a, max(b, c));
+      const double m = (double)tw[node];
+      all += m * m;
+      if (M == N) shN += m * m;
+      if (M == N - 1) shN1 += m * m;
+    }
+  } else if (ex >= 2047) {
+    all = shN = shN1 = __longlong_as_double(0x7ff8000000000000ll);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -1341,6 +1353,10 @@ cudaError_t upload(const DgTables &t) {
         fvp[i * EO_H + m] = (float)vp[i * EO_H + m];
         fvm[i * EO_H + m] = (float)vm[i * EO_H + m];
       }
+  int2 VI[n * IND_H];
+  for (int i = 0; i < n; ++i)
+    for (int m = 0; m < IND_H; ++m)
+      VI[i * IND_H + m] = fx_halves((n % 2 && m == N / 2 ? 0.5L : 1.0L) * t.Vinv[i * n + m], 61);
   double ihx[n];
   float fihx[n];
   ihx[0] = 0.0;
@@ -1363,7 +1379,7 @@ cudaError_t upload(const DgTables &t) {
   err = err ? err : cudaMemcpyToSymbol(c_invw, t.invw, sizeof(double) * n);
   err = err ? err : cudaMemcpyToSymbol(c_xi, t.xi, sizeof(double) * n);
   err = err ? err : cudaMemcpyToSymbol(c_xh, t.xh, sizeof(double) * (n + 1));
-  err = err ? err : cudaMemcpyToSymbol(c_Vinv, t.Vinv, sizeof(double) * nn);
+  err = err ? err : cudaMemcpyToSymbol(c_VI, VI, sizeof(VI));
   err = err ? err : cudaMemcpyToSymbol(f_D, fD, sizeof(float) * nn);
   err = err ? err : cudaMemcpyToSymbol(f_D2, fD2, sizeof(float) * nn);
   err = err ? err : cudaMemcpyToSymbol(f_Dq, fDq, sizeof(float) * nn);
