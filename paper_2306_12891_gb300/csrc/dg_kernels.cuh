@@ -1291,8 +1291,23 @@ __global__ void __launch_bounds__(256) k_reduce_partials(const double *__restric
   if (lane == 0) out[c] = s;
 }
 
+// float(x 2^(1023 - e)) for a double whose biased exponent is at most e (zero where that is below 2^-126)
+__device__ __forceinline__ float scaled_float(double x, int e) {
+  const int h = __double2hiint(x), ex = (h >> 20) & 0x7ff, k = ex + 1023 - e;
+  const unsigned m = ((unsigned)h << 3 & 0x7fffffu) | ((unsigned)__double2loint(x) >> 29);
+  return k > 897 ? __uint_as_float(((unsigned)h & 0x80000000u) | (unsigned)(k - 896) << 23 | m) : 0.0f;
+}
+
+// cfl-free time step: min over nodes of 2J / ((2N+1) sum_d (|u.Ja^d| + c|Ja^d|)). The wave speed sum takes four FP64
+// square roots and a division (~75 FP64 instructions); it is estimated in FP32 first, from values scaled by their own
+// exponents (to 2e-6, the products' rounding added; 8e-6 is allowed), and evaluated in FP64 only where the estimate reaches the
+// block's largest sum / J so far. The node with the smallest step is never skipped, so the result is the minimum of
+// the same FP64 expression. N = 5, 24^3: 210 us, 477 with every node in FP64.
 __global__ void __launch_bounds__(256) k_max_dt(const DgDevice d, const double *__restrict__ U) {
   __shared__ double red[256];
+  __shared__ int s_top;  // high word of the block's largest sum / J
+  if (threadIdx.x == 0) s_top = 0;
+  __syncthreads();
   double best = 1e300;
   const long long total = (long long)d.nE * nnn;
   const double gam = d.gamma;
@@ -1302,15 +1317,44 @@ __global__ void __launch_bounds__(256) k_max_dt(const DgDevice d, const double *
     const double r = U[b], ir = 1.0 / r;
     const double u = U[b + nnn] * ir, v = U[b + 2 * nnn] * ir, w = U[b + 3 * nnn] * ir;
     const double p = (gam - 1.0) * (U[b + 4 * nnn] - 0.5 * r * (u * u + v * v + w * w));
-    const double c = sqrt(gam * p * ir);
-    double lam = 0.0;
+    const double c2 = gam * p * ir;
+    double J[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) J[k] = d.Ja[((size_t)e * 9 + k) * nnn + node];
+    const double ij = d.invJ[t];
+    // the estimate: velocities scaled by 2^-(eu - 1023), c^2 by its square, Ja by 2^-(ej - 1023)
+    const int hc = __double2hiint(c2) >> 20, hu = max(max(fx_hi_abs(u), fx_hi_abs(v)), fx_hi_abs(w)) >> 20;
+    const int eu = max(hu, ((hc + 1023) >> 1) + 1);
+    int hj = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) hj = max(hj, fx_hi_abs(J[k]));
+    const int ej = hj >> 20, eij = __double2hiint(ij) >> 20;
+    const float fu = scaled_float(u, eu), fv = scaled_float(v, eu), fw = scaled_float(w, eu);
+    const float fc = sqrtf(scaled_float(c2, 2 * eu - 1023));
+    float lam = 0.0f;
 #pragma unroll
     for (int dd = 0; dd < 3; ++dd) {
-      const double *Jd = d.Ja + ((size_t)e * 3 + dd) * 3 * nnn + node;
-      const double ax = Jd[0], ay = Jd[nnn], az = Jd[2 * nnn];
-      lam += fabs(u * ax + v * ay + w * az) + c * sqrt(ax * ax + ay * ay + az * az);
+      const float x = scaled_float(J[3 * dd], ej), y = scaled_float(J[3 * dd + 1], ej), z = scaled_float(J[3 * dd + 2], ej);
+      lam += fabsf(fu * x + fv * y + fw * z) + fc * sqrtf(x * x + y * y + z * z) +
+             1e-6f * (fabsf(fu * x) + fabsf(fv * y) + fabsf(fw * z));  // the products may cancel
     }
-    best = fmin(best, 2.0 * d.J[t] / ((2.0 * N + 1.0) * lam));
+    lam *= scaled_float(ij, eij);
+    // its high word as a double's, with the exponents put back (a value outside FP64's range counts as large)
+    const int eh = eu + ej + eij - 3 * 1023, fl = (int)__float_as_uint(lam);
+    const int h = (fl >> 3) + (896 << 20), top = *(volatile int *)&s_top;
+    const bool odd = hc < 0 || hc >= 2047 || hu >= 2047 || fl <= 0 || fl >= 0x7f000000 || abs(eh) > 900;
+    if (odd || h + (eh << 20) + 8 >= top) {
+      const double c = sqrt(c2);
+      double sum = 0.0;
+#pragma unroll
+      for (int dd = 0; dd < 3; ++dd)
+        sum += fabs(u * J[3 * dd] + v * J[3 * dd + 1] + w * J[3 * dd + 2]) +
+               c * sqrt(J[3 * dd] * J[3 * dd] + J[3 * dd + 1] * J[3 * dd + 1] + J[3 * dd + 2] * J[3 * dd + 2]);
+      const double x = 2.0 * d.J[t] / ((2.0 * N + 1.0) * sum);
+      best = fmin(best, x);
+      const int hs = __double2hiint(sum * ij);
+      if (!odd && hs > top) atomicMax(&s_top, hs);
+    }
   }
   red[threadIdx.x] = best;
   __syncthreads();
