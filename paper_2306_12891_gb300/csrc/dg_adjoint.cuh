@@ -19,7 +19,7 @@
 //   adj_volume  per element: the two-point flux differencing transposed pair by pair. With
 //               sums S = x_i + x_m the Kennedy-Gruber / Pirozzoli fluxes are polynomials in
 //               (S_rho, S_u, S_p, S_X), so each pair adds the same cotangent vector to both of its
-//               nodes' primitive accumulators; then per node the primitive cotangents (plus the
+//               nodes' primitive accumulators (in 64-bit fixed point); then per node the primitive cotangents (plus the
 //               viscous ones) are chained to the conservative variables, the face slots are added,
 //               and either Ubar is written or the LSERK(5,4) reverse stage is applied in place.
 #pragma once
@@ -454,23 +454,8 @@ __global__ void __launch_bounds__(LIFT_THREADS) k_adj_visc(const DgDevice d, con
 }
 
 // ---------------------------------------------------------------------------------------------
-// adjoint of the volume kernel
-// staged per element: P[6][PS] = (rho, u, v, w, 4p, X) with X = h (Pirozzoli) or e = E/rho (KG),
-// Lm[5][PS] = l, and per direction Acc[3][6][PS] = cotangents of (rho, u, v, w, 4p, X)
+// transposed pair terms in FP64 (the general path)
 // ---------------------------------------------------------------------------------------------
-constexpr int ADJ_NP = 6;
-constexpr int ADJ_SLOTS = ADJ_NP + 5 + 18;
-// elements per CTA and CTAs per SM of the adjoint volume kernel: its shared memory (29 staged slots
-// per element) is 1.4x the forward's, so at N = 5 one element per CTA lets three CTAs share an SM
-// (12 warps) where two elements per CTA fitted only one (7 warps)
-__host__ __device__ constexpr int adj_epb() { return N == 1 ? 8 : N == 2 ? 4 : N == 3 ? 2 : N == 4 ? 3 : 1; }
-constexpr int ADJ_EPB = adj_epb();
-constexpr int ADJ_THREADS = round32(3 * nn * ADJ_EPB);
-constexpr int ADJ_MINB = N == 5 ? 3 : N == 6 ? 2 : 1;
-
-// Transposed flux differencing along one line. The forward pair term (scaled by the folded
-// 1/2 factors) is c.F with F0 = S_rho V, F_k = F0 S_u,k + S_p S_j,k, F4 = F0 S_X (+ S_p V / 2 for KG),
-// V = S_u . S_j and c_v = D'_im l_i,v + D'_mi l_m,v (D' = D/4 for mass, D/8 otherwise).
 // one node's staged values for the transposed pair terms
 struct AdjNode {
   double r, u, v, w, p, x, l[5], jx, jy, jz;
@@ -517,176 +502,427 @@ __device__ __forceinline__ void adj_pair(const AdjNode &a, const AdjNode &b, dou
   g[5] = t4 * F0;
 }
 
-// Transposed flux differencing along one line, two rows at a time (as the forward line_fluxdiff2):
-// the cotangent sums of nodes i and i+1 stay in registers while partner m runs over i+2..N, so each
-// partner's staged values and partial sums are read (and written back) once for two pairs.
+// ---------------------------------------------------------------------------------------------
+// adjoint of the volume kernel, its transposed pair terms in the 64-bit fixed point of dg_fixed.cuh
+// (phases, lanes and general path as k_volume_fx). With the sums S = x_i + x_m and the pair cotangents
+// t_v = Q_im (l_i,v / w_i - l_m,v / w_m) w_0 (D_im l_i + D_mi l_m = Q_im (l_i / w_i - l_m / w_m)), both
+// nodes of a pair get the same cotangents of (rho, u, v, w, 4p, X):
+//   phi = t_0 + t_k S_u,k + t_4 S_X, F0 = S_rho V, V = S_u . S_J, gV = phi S_rho (+ 2 t_4 S_p for KG):
+//   (phi V, t_k F0 + gV S_J,k, t_k S_J,k (+ t_4 V / 2 for KG), t_4 F0), all times 1 / (8 w_0)
+// (l_0 doubled: its split-form factor is D/4, the others' D/8). 25 products a pair (28 for KG) against
+// ~49 FP64 instructions.
+// ---------------------------------------------------------------------------------------------
+struct FxAdj {
+  int ok;
+  int er, eu, ep, ex, ej, e0, e1, e4;  // exponents: rho, u, p, X, Ja, l of mass, momentum, energy
+  int av, aa, ab, af, ag, a0, ak, ax;  // windows of V, t_k S_u,k, t_4 S_X, F0, phi S_rho and the outputs
+  int pa, pb, p0;                      // right shifts of t_k S_u,k, t_4 S_X and t_0 to phi's scale
+  int va, vb;                          // KG: right shifts of phi S_rho and t_4 S_p to gV's
+  int kf, kv;                          // right shifts of F0 and gV before t_k F0 + gV S_J,k
+  int ga, gb;                          // right shifts of t_k S_J,k and (KG) t_4 V to the output's scale
+  int k0, k1, kp, kx;                  // cotangents are fixed value x 2^k / (8 w_0): rho, u, 4p, X
+};
+
+// upper bound of log2(2^a + 2^b) in 2^-20
+__device__ __forceinline__ int fx_lsum(int a, int b) {
+  const int d = abs(a - b) >> 20;
+  return max(a, b) + (d == 0 ? 1048576 : d == 1 ? 613400 : d == 2 ? 337600 : d == 3 ? 178400 : 91800);
+}
+
+// Bounds (value x scale, log2): S_rho, S_p < 63, S_u, S_J, S_X, l differences < 61; t < 61. V, phi, F0 and gV fill at
+// most 62.2 and a line's sum of each output at most 62.2, by windows and shifts from the element's maxima; the
+// halved sum of three directions then stays below 63, and every group of cross sums h l' + l h' too.
 template <int VF>
-__device__ __forceinline__ void adj_line(const double *__restrict__ P, const double *__restrict__ Lm, int pb, int ps,
-                                         const double *__restrict__ Jd, int gb, int gs, double *__restrict__ Ac) {
-#pragma unroll 1
-  for (int i = 0; i < n - 1; i += 2) {
-    const int a0 = pb + i * ps, a1 = a0 + ps;
-    const AdjNode n0 = adj_node(P, Lm, a0, Jd, gb + i * gs), n1 = adj_node(P, Lm, a1, Jd, gb + (i + 1) * gs);
-    double ac0[6], ac1[6];
+__device__ __forceinline__ FxAdj fx_adj_scales(const int *mx, int2 mj) {
+  // mx: high words: rho max, rho min, |u| max, p max, p min, x max, x min (minima signed), |l| of mass, momentum, energy,
+  // |u| + |v| + |w| max
+  FxAdj s;
+  s.er = fx_exponent(mx[0]); s.ep = fx_exponent(mx[3]); s.ex = fx_exponent(mx[5]); s.ej = fx_exponent(mj.x);
+  s.eu = max(fx_exponent(mx[2]), (1996 - s.er + s.ep) >> 1);
+  // exponents of l: a group far below the others' shares of phi takes a scale 2^-40 of theirs
+  const int r0 = fx_exponent(mx[7]), r1 = fx_exponent(mx[8]), r4 = fx_exponent(mx[9]);
+  const int ph = max(r0, max(r1 + s.eu, r4 + s.ex) - 1023);
+  s.e0 = max(r0, ph - 40); s.e1 = max(r1, ph - s.eu + 1023 - 40); s.e4 = max(r4, ph - s.ex + 1023 - 40);
+  const int lo = min(min(min(s.er, s.ep), min(s.ex, s.ej)), min(min(s.e0, s.e1), s.e4));
+  const int hi = max(max(max(s.er, s.ep), max(s.ex, s.ej)), max(max(max(s.e0, s.e1), s.e4), s.eu));
+  const int sr = 1084 - s.er, su = 1082 - s.eu, sp = 1084 - s.ep, sx = 1082 - s.ex, sj = 1082 - s.ej;
+  const int l0 = 1082 - s.e0, l1 = 1082 - s.e1, l4 = 1082 - s.e4;
+  // log2 bounds in 2^-20: of sums S and differences of l (twice the maxima), then of the products
+  constexpr int L = 1 << 20, LIM = (int)(62.2 * L);
+  const int lr = fx_lg(mx[0]) + L, lu = max(fx_lg(mx[2]), (s.eu - 1023) << 20) + L, lp = fx_lg(mx[3]) + L,
+            lx = fx_lg(mx[5]) + L, lj = fx_lg(mj.x) + L, lv = lu + fx_lg(mj.y) + L;
+  const int t0 = max(fx_lg(mx[7]), (s.e0 - 1023) << 20) + L, t1 = max(fx_lg(mx[8]), (s.e1 - 1023) << 20) + L,
+            t4 = max(fx_lg(mx[9]), (s.e4 - 1023) << 20) + L;
+  const int la = t1 + max(fx_lg(mx[10]), (s.eu - 1023) << 20) + L, lb = t4 + lx, lf = lr + lv,
+            lphi = fx_lsum(fx_lsum(la, lb), t0);
+  auto window = [&](int bound, int scale) { return min(max(((LIM - bound) >> 20) - scale, 0), 10); };
+  s.av = window(lv, su + sj - 64);
+  const int sv = su + sj - 64 + s.av;
+  s.aa = window(la, l1 + su - 64);
+  s.ab = window(lb, l4 + sx - 64);
+  const int fa = l1 + su - 64 + s.aa, fb = l4 + sx - 64 + s.ab;
+  const int sf = min(min(min(fa, fb), l0), (LIM - lphi) >> 20);  // phi
+  s.pa = min(fa - sf, 62); s.pb = min(fb - sf, 62); s.p0 = min(l0 - sf, 62);
+  s.af = window(lf, sr + sv - 64);
+  const int sF = sr + sv - 64 + s.af;  // F0
+  int lg = lphi + lr;
+  s.ag = window(lg, sf + sr - 64);
+  int sg = sf + sr - 64 + s.ag;  // gV
+  s.va = s.vb = 0;
+  if (VF == VF_KG) {
+    const int a = sg, b = l4 + sp - 62 - 1;  // t_4 S_p with window 2; the factor 2
+    lg = fx_lsum(lg, t4 + lp + L);
+    sg = min(min(a, b), (LIM - lg) >> 20);
+    s.va = min(a - sg, 62); s.vb = min(b - sg, 62);
+  }
+  const int lk = fx_lsum(t1 + lf, lg + lj) + FX_LGR, c0 = sf + sv - 64, cx = l4 + sF - 64;
+  int ka = l1 + sF - 64, kb = sg + sj - 64, sk = min(ka, kb);
+  s.kf = min(ka - sk, 62); s.kv = min(kb - sk, 62);
+  s.ak = window(lk, sk);
+  s.a0 = window(lphi + lv + FX_LGR, c0);
+  s.ax = window(t4 + lf + FX_LGR, cx);
+  const int pA = l1 + sj - 61, pB = l4 + sv - 62 + 1;  // t_k S_J,k with window 3; t_4 V with window 2, the factor 1/2
+  int lP = t1 + fx_lg(mj.y) + L + FX_LGR, sP = pA;
+  if (VF == VF_KG) {
+    lP = fx_lsum(lP, t4 + lv - L + FX_LGR);
+    sP = min(sP, pB);
+  }
+  sP = min(sP, (LIM - lP) >> 20);
+  s.ga = min(pA - sP, 62);
+  s.gb = VF == VF_KG ? min(pB - sP, 62) : 0;
+  s.k0 = 1 - (c0 + s.a0); s.k1 = 1 - (sk + s.ak); s.kp = 1 - sP; s.kx = 1 - (cx + s.ax);  // (halved sums)
+  const int km = max(max(abs(s.k0), abs(s.k1)), max(abs(s.kp), abs(s.kx)));
+  s.ok = mx[1] > 0 && mx[4] > 0 && mx[6] > 0 && s.er - (mx[1] >> 20) <= 8 && s.ep - (mx[4] >> 20) <= 8 &&
+         s.ex - (mx[6] >> 20) <= 8 && lo >= 850 && hi <= 1200 && km <= 900;
+  return s;
+}
+
+struct FxAdjNode {
+  fx_t r, u, v, w, p, x, jx, jy, jz, l[5];
+};
+// element slots (FX_PS each): 0-5 rho, u, v, w, p, X; 6 + 8 dir + c: metric terms (c < 3), weighted l (c = 3 + v);
+// a line's six cotangents of node i then replace the first six of its direction's eight
+constexpr int FXA_SLOTS = 30;
+template <int VF>
+__device__ __forceinline__ FxAdjNode fx_adj_load(const fx_t *__restrict__ S, int a, int dir) {
+  const fx_t *J = S + (6 + 8 * dir) * FX_PS + a;
+  FxAdjNode q{S[a], S[FX_PS + a], S[2 * FX_PS + a], S[3 * FX_PS + a], VF == VF_KG ? S[4 * FX_PS + a] : 0,
+              S[5 * FX_PS + a], J[0], J[FX_PS], J[2 * FX_PS]};
 #pragma unroll
-    for (int v = 0; v < 6; ++v) {
-      ac0[v] = (i == 0) ? 0.0 : Ac[v * PS + a0];
-      ac1[v] = (i == 0) ? 0.0 : Ac[v * PS + a1];
+  for (int v = 0; v < 5; ++v) q.l[v] = J[(3 + v) * FX_PS];
+  return q;
+}
+
+template <int VF>
+__device__ __forceinline__ void fx_adj_pair(const FxAdjNode &a, const FxAdjNode &b, FxD q, const FxAdj &c, fx_t g[6]) {
+  const FxD Sj[3] = {fx_biased(a.jx + b.jx), fx_biased(a.jy + b.jy), fx_biased(a.jz + b.jz)};
+  const FxD Su[3] = {fx_biased(a.u + b.u), fx_biased(a.v + b.v), fx_biased(a.w + b.w)};
+  const FxD Sr = fx_biased(a.r + b.r);
+  fx_t t0;
+  FxD t[4];  // momentum, energy
+  {
+    FxSum s = fx_zero(1);
+    fx_acc(s, q, fx_split(a.l[0] - b.l[0]));
+    t0 = fx_value(s, 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      s = fx_zero_biased(1);
+      fx_acc(s, q, fx_split(a.l[1 + k] - b.l[1 + k]));
+      t[k] = fx_biased(fx_value(s, 1));
     }
-    {
+  }
+  FxSum s = fx_zero_biased(c.av), z;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) fx_acc(s, Su[k], Sj[k]);
+  const FxD V = fx_biased(fx_value(s, c.av));
+  s = fx_zero(c.aa);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) fx_acc(s, t[k], Su[k]);
+  z = fx_zero(c.ab);
+  fx_acc(z, t[3], fx_biased(a.x + b.x));
+  const FxD phi = fx_split(fx_shr(fx_value(s, c.aa), c.pa) + fx_shr(fx_value(z, c.ab), c.pb) + fx_shr(t0, c.p0));
+  s = fx_zero(c.a0);
+  fx_acc(s, phi, V);
+  g[0] = fx_value(s, c.a0);
+  s = fx_zero(c.af);
+  fx_acc(s, Sr, V);
+  const fx_t F0 = fx_value(s, c.af);
+  const FxD Fk = fx_split(fx_shr(F0, c.kf));
+  s = fx_zero(c.ag);
+  fx_acc(s, phi, Sr);
+  fx_t gv = fx_value(s, c.ag);
+  s = fx_zero(3);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) fx_acc(s, t[k], Sj[k]);
+  g[4] = fx_shr(fx_value(s, 3), c.ga);
+  if (VF == VF_KG) {
+    z = fx_zero(2);
+    fx_acc(z, t[3], fx_biased(a.p + b.p));
+    gv = fx_shr(gv, c.va) + fx_shr(fx_value(z, 2), c.vb);
+    z = fx_zero(2);
+    fx_acc(z, t[3], V);
+    g[4] += fx_shr(fx_value(z, 2), c.gb);
+  }
+  const FxD gV = fx_split(fx_shr(gv, c.kv));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    s = fx_zero(c.ak);
+    fx_acc(s, t[k], Fk);
+    fx_acc(s, gV, Sj[k]);
+    g[1 + k] = fx_value(s, c.ak);
+  }
+  s = fx_zero(c.ax);
+  fx_acc(s, t[3], fx_split(F0));
+  g[5] = fx_value(s, c.ax);
+}
+
+// general path of one node in FP64, from the staged doubles: slots 0-5 as above, 6-10 l
+template <int VF>
+__device__ __noinline__ void fx_adj_general_node(const DgDevice &d, const double *S, size_t e, int node, double gp[6]) {
+  const int ijk[3] = {node % n, (node / n) % n, node / nn};
+  for (int v = 0; v < 6; ++v) gp[v] = 0.0;
+  for (int dd = 0; dd < 3; ++dd) {
+    const int id = ijk[dd], st = dd == 0 ? 1 : dd == 1 ? n : nn, ps = dd == 0 ? 1 : dd == 1 ? FX_SJ : FX_SK;
+    const double *Jd = d.Ja + (e * 3 + dd) * 3 * nnn;
+    auto load = [&](int m) {
+      const double *P = S + fx_idx(node) + (m - id) * ps;
+      const int gn = node + (m - id) * st;
+      AdjNode q{P[0], P[FX_PS], P[2 * FX_PS], P[3 * FX_PS], 4.0 * P[4 * FX_PS], P[5 * FX_PS]};
+      for (int k = 0; k < 5; ++k) q.l[k] = P[(6 + k) * FX_PS];
+      q.jx = Jd[gn]; q.jy = Jd[nnn + gn]; q.jz = Jd[2 * nnn + gn];
+      return q;
+    };
+    const AdjNode a = load(id);
+    for (int m = 0; m < n; ++m) {
+      if (m == id) continue;
       double g[6];
-      adj_pair<VF>(n0, n1, c_De[i * n + i + 1], c_Dr[i * n + i + 1], g);
-#pragma unroll
-      for (int v = 0; v < 6; ++v) { ac0[v] += g[v]; ac1[v] += g[v]; }
-    }
-#pragma unroll
-    for (int m = i + 2; m < n; ++m) {
-      const int am = pb + m * ps;
-      const AdjNode nm = adj_node(P, Lm, am, Jd, gb + m * gs);
-      double g0[6], g1[6];
-      adj_pair<VF>(n0, nm, c_De[i * n + m], c_Dr[i * n + m], g0);
-      adj_pair<VF>(n1, nm, c_De[(i + 1) * n + m], c_Dr[(i + 1) * n + m], g1);
-#pragma unroll
-      for (int v = 0; v < 6; ++v) {
-        ac0[v] += g0[v];
-        ac1[v] += g1[v];
-        const double gm = g0[v] + g1[v];
-        if (i == 0) Ac[v * PS + am] = gm;
-        else Ac[v * PS + am] += gm;
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < 6; ++v) {
-      Ac[v * PS + a0] = ac0[v];
-      Ac[v * PS + a1] = ac1[v];
+      adj_pair<VF>(a, load(m), c_De[id * n + m], c_Dr[id * n + m], g);
+      for (int v = 0; v < 6; ++v) gp[v] += g[v];
     }
   }
 }
 
+constexpr size_t FXA_SMEM = sizeof(fx_t) * FX_EPB * FXA_SLOTS * FX_PS;
+constexpr int FXA_MINB = 704 / FX_THREADS < 1 ? 1 : 704 / FX_THREADS;  // >= 80 registers per thread
+
+// One thread per node. The CTAs per SM give 80 registers at N = 3..5 (140 B spilled; with two thirds of the CTAs
+// and no spill N = 5 is 20 % slower, N = 3 3 % faster). Measured per launch, Pirozzoli + Navier-Stokes N = 5, 12^3:
+// 0.166 ms against 0.395 with FP64 line threads; KG Euler N = 3, 21 x 18 x 15: 94 against 241 us. Bound by issue and
+// the FMA-heavy pipe, like k_volume_fx.
 template <int VF>
-__global__ void __launch_bounds__(ADJ_THREADS, ADJ_MINB) k_adj_volume(const DgDevice d, const double *__restrict__ U,
+__global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDevice d, const double *__restrict__ U,
                                                               const double *lam, const double *__restrict__ fslots,
                                                               const double *__restrict__ cotW,
                                                               const double *__restrict__ sigma, double *out,
                                                               double *gbar, int mode, double dt, double A, double B,
                                                               int update_g) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  double *P = reinterpret_cast<double *>(sm_raw);  // [EPB][6][PS]
-  double *Lm = P + ADJ_EPB * ADJ_NP * PS;          // [EPB][5][PS]
-  double *Acc = Lm + ADJ_EPB * 5 * PS;             // [EPB][3][6][PS]
-  const int e0 = blockIdx.x * ADJ_EPB;
-  const double gam = d.gamma, gm1 = gam - 1.0;
-  // the thread's nodes (the same in staging and in the per-node part): their 1/rho stays in registers
-  constexpr int RN = (ADJ_EPB * nnn + ADJ_THREADS - 1) / ADJ_THREADS;
-  double irr[RN];
+  fx_t *S = reinterpret_cast<fx_t *>(sm_raw);  // [EPB][FXA_SLOTS][FX_PS]
+  __shared__ int s_mx[FX_EPB][11];
+  __shared__ FxAdj s_sc[FX_EPB];
+  __shared__ int2 s_rho[FX_H], s_Q[nn];
+  const int e0 = blockIdx.x * FX_EPB, tid = threadIdx.x;
+  const double gm1 = d.gamma - 1.0;
+  for (int t = tid; t < FX_EPB * 11; t += FX_THREADS) {
+    const int k = t % 11;
+    s_mx[t / 11][k] = (k == 1 || k == 4 || k == 6) ? 0x7fffffff : 0;
+  }
+  for (int t = tid; t < FX_H; t += FX_THREADS) s_rho[t] = c_rho[t * FX_H];  // w_0 / w
+  for (int t = tid; t < nn; t += FX_THREADS) s_Q[t] = c_Qx[t];
+  __syncthreads();
+  const int le = tid / nnn, node = tid % nnn, e = e0 + le;
+  const bool on = tid < FX_EPB * nnn && e < d.nE;
+  const int ijk[3] = {node % n, (node / n) % n, node / nn};
+  double r = 1.0, ir = 1.0, u[3], p = 1.0, X = 1.0, l[5];
+  {
+    int h[11] = {0, 0x7fffffff, 0, 0, 0x7fffffff, 0, 0x7fffffff, 0, 0, 0, 0};
+    if (on) {
+      double Uv[5];
+      load_state<double>(d, U, e, node, Uv);
+      r = Uv[0];
+      ir = 1.0 / r;
 #pragma unroll
-  for (int rr = 0; rr < RN; ++rr) {
-    const int t = threadIdx.x + rr * ADJ_THREADS;
-    if (t >= ADJ_EPB * nnn) continue;
-    const int le = t / nnn, node = t % nnn, e = e0 + le;
-    if (e >= d.nE) continue;
-    double Uv[5];
-    load_state<double>(d, U, e, node, Uv);
-    const double r = Uv[0], ir = 1.0 / r;
-    irr[rr] = ir;
-    const double u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
-    const double p = gm1 * (Uv[4] - 0.5 * (Uv[1] * u + Uv[2] * v + Uv[3] * w));
-    if (!(r > 0.0) || !(p > 0.0) || !isfinite(Uv[4])) flag_set(d.flag, 1);
-    const int pn = pidx(node);
-    double *Pe = P + le * ADJ_NP * PS + pn;
-    Pe[0] = r; Pe[PS] = u; Pe[2 * PS] = v; Pe[3 * PS] = w; Pe[4 * PS] = 4.0 * p;
-    Pe[5 * PS] = VF == VF_PIR ? (Uv[4] + p) * ir : Uv[4] * ir;
-    const double miJ = -d.invJ[(size_t)e * nnn + node];
-    // l = -lambda/J; the mass component doubled (its split-form factor is D/4, the others' D/8)
+      for (int k = 0; k < 3; ++k) u[k] = Uv[1 + k] * ir;
+      p = gm1 * (Uv[4] - 0.5 * (Uv[1] * u[0] + Uv[2] * u[1] + Uv[3] * u[2]));
+      if (!(r > 0.0) || !(p > 0.0) || !isfinite(Uv[4])) flag_set(d.flag, 1);
+      X = VF == VF_PIR ? (Uv[4] + p) * ir : Uv[4] * ir;
+      const double miJ = -d.invJ[(size_t)e * nnn + node];
+      // l = -lambda/J, the mass component doubled
 #pragma unroll
-    for (int k = 0; k < 5; ++k)
-      Lm[(le * 5 + k) * PS + pn] = (k == 0 ? 2.0 * miJ : miJ) * lam[((size_t)e * 5 + k) * nnn + node];
+      for (int k = 0; k < 5; ++k) l[k] = (k == 0 ? 2.0 * miJ : miJ) * lam[((size_t)e * 5 + k) * nnn + node];
+      h[0] = fx_hi_abs(r); h[1] = __double2hiint(r);
+      h[2] = max(max(fx_hi_abs(u[0]), fx_hi_abs(u[1])), fx_hi_abs(u[2]));
+      h[3] = fx_hi_abs(p); h[4] = __double2hiint(p);
+      h[5] = fx_hi_abs(X); h[6] = __double2hiint(X);
+      h[7] = fx_hi_abs(l[0]);
+      h[8] = max(max(fx_hi_abs(l[1]), fx_hi_abs(l[2])), fx_hi_abs(l[3]));
+      h[9] = fx_hi_abs(l[4]);
+      h[10] = fx_hi_abs(fabs(u[0]) + fabs(u[1]) + fabs(u[2]));
+    }
+    bool each = on;
+    if (FX_EPB == 1) {
+#pragma unroll
+      for (int k = 0; k < 11; ++k)
+        h[k] = (k == 1 || k == 4 || k == 6) ? __reduce_min_sync(0xffffffffu, h[k]) : __reduce_max_sync(0xffffffffu, h[k]);
+      each = (tid & 31) == 0 && on;
+    }
+    if (each) {
+#pragma unroll
+      for (int k = 0; k < 11; ++k) {
+        if (k == 1 || k == 4 || k == 6) atomicMin(&s_mx[le][k], h[k]);
+        else atomicMax(&s_mx[le][k], h[k]);
+      }
+    }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < ADJ_EPB * 3 * nn; t += blockDim.x) {
-    const int le = t / (3 * nn), r = t % (3 * nn), dir = r / nn, line = r % nn, e = e0 + le;
-    if (e >= d.nE) continue;
-    int pb, ps, gb, gs, a, b;
-    line_geom(dir, line, pb, ps, gb, gs, a, b);
-    adj_line<VF>(P + le * ADJ_NP * PS, Lm + le * 5 * PS, pb, ps, d.Ja + ((size_t)e * 3 + dir) * 3 * nnn, gb, gs,
-                 Acc + (le * 3 + dir) * ADJ_NP * PS);
+  int good = 1;
+  if (tid < FX_EPB && e0 + tid < d.nE) {
+    s_sc[tid] = fx_adj_scales<VF>(s_mx[tid], d.jmax[e0 + tid]);
+    good = s_sc[tid].ok;
   }
-  __syncthreads();
-  const bool ns = d.equations == 1;
-  const double iR = 1.0 / d.R;
+  const bool ok = __syncthreads_and(good);
+  if (ok) {
+    if (on) {
+      const FxAdj &c = s_sc[le];
+      constexpr fx_t HB = FX_BIAS / 2;
+      fx_t *Se = S + le * FXA_SLOTS * FX_PS + fx_idx(node);
+      Se[0] = fx_from(r, c.er, 1) + HB;
 #pragma unroll
-  for (int rr = 0; rr < RN; ++rr) {
-    const int t = threadIdx.x + rr * ADJ_THREADS;
-    if (t >= ADJ_EPB * nnn) continue;
-    const int le = t / nnn, node = t % nnn, e = e0 + le;
-    if (e >= d.nE) continue;
-    const int ijk[3] = {node % n, (node / n) % n, node / nn};
-    const int pn = pidx(node);
-    const double *Pe = P + le * ADJ_NP * PS + pn;
-    const double u[3] = {Pe[PS], Pe[2 * PS], Pe[3 * PS]}, p = 0.25 * Pe[4 * PS], X = Pe[5 * PS];
-    double gp[6];
+      for (int k = 0; k < 3; ++k) Se[(1 + k) * FX_PS] = fx_from(u[k], c.eu, 3) + HB;
+      if (VF == VF_KG) Se[4 * FX_PS] = fx_from(p, c.ep, 1) + HB;
+      Se[5 * FX_PS] = fx_from(X, c.ex, 3) + HB;
+      const double *Je = d.Ja + (size_t)e * 9 * nnn + node;
 #pragma unroll
-    for (int v = 0; v < 6; ++v)
-      gp[v] = Acc[(le * 3 + 0) * ADJ_NP * PS + v * PS + pn] + Acc[(le * 3 + 1) * ADJ_NP * PS + v * PS + pn] +
-              Acc[(le * 3 + 2) * ADJ_NP * PS + v * PS + pn];
-    const double ir = irr[rr];
-    double g_r = gp[0], g_u[3] = {gp[1], gp[2], gp[3]}, g_p = 4.0 * gp[4];
-    const double g_x = gp[5];
-    if (ns) {  // cotangents of (u, v, w, T) from the viscous adjoint, own part + the neighbours' face shares
-      double cw[4];
+      for (int k = 0; k < 9; ++k) Se[(6 + 8 * (k / 3) + k % 3) * FX_PS] = fx_from(__ldg(Je + k * nnn), c.ej, 3) + HB;
+      FxD lf[5];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) cw[q] = cotW[((size_t)e * 4 + q) * nnn + node];
+      for (int v = 0; v < 5; ++v) lf[v] = fx_split(fx_from(l[v], v == 0 ? c.e0 : v < 4 ? c.e1 : c.e4, 3));
 #pragma unroll
       for (int dd = 0; dd < 3; ++dd) {
-        const int id = ijk[dd];
-        if (id != 0 && id != N) continue;
-        const int f = 2 * dd + (id == N ? 1 : 0);
-        const int pp = dd == 0 ? ijk[1] : ijk[0], qq = dd == 2 ? ijk[1] : ijk[2];
-        int nb, fnb, nbnode, nbpq;
-        neighbour_node(d, e, f, pp, qq, nb, fnb, nbnode, nbpq);
-        const double *sg = sigma + ((size_t)nb * 6 + fnb) * 4 * nn + nbpq;
+        const FxD w = fx_const(s_rho[min(ijk[dd], N - ijk[dd])]);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) cw[q] += sg[q * nn];
+        for (int v = 0; v < 5; ++v) {
+          FxSum s = fx_zero(2);
+          fx_acc(s, w, lf[v]);
+          Se[(9 + 8 * dd + v) * FX_PS] = fx_value(s, 2);
+        }
       }
-      g_u[0] += cw[0];
-      g_u[1] += cw[1];
-      g_u[2] += cw[2];
-      g_p += cw[3] * ir * iR;         // T = p / (rho R)
-      g_r -= cw[3] * p * ir * ir * iR;
     }
-    // chain to U = (rho, m, E): u = m / rho, p = (gamma-1)(E - |m|^2 / (2 rho)), X = h = (E + p)/rho
-    // (Pirozzoli) or e = E/rho (KG). With gx = g_X/rho, p reaches U with weight a = (gamma-1) g_p, and
-    // for h also through E + p: a = (gamma-1)(g_p + gx), and dh/dE = gamma/rho = (gamma-1)/rho + 1/rho
-    const double q2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double gx = g_x * ir;
-    const double a = VF == VF_PIR ? gm1 * (g_p + gx) : gm1 * g_p;
-    double gU[5];
-    gU[0] = g_r - ir * (g_u[0] * u[0] + g_u[1] * u[1] + g_u[2] * u[2]) + (0.5 * a) * q2 - gx * X;
+    __syncthreads();
+    constexpr int GROUPS = (FX_EPB * nn + FX_LPW - 1) / FX_LPW;
+    const int lane = tid & 31, idx = lane % n, l0 = (lane / n) % FX_LPW * n;
+    for (int gr = tid >> 5; gr < 3 * GROUPS; gr += FX_THREADS / 32) {
+      const int dir = gr / GROUPS, g0 = (gr % GROUPS) * FX_LPW;
+      const bool own = lane < FX_LPW * n && g0 + lane / n < FX_EPB * nn;
+      const int ln = own ? g0 + lane / n : g0;  // lanes without a line of their own repeat the group's first one
+      const int lel = ln / nn, ll = ln % nn, la = ll % n, lb = ll / n;
+      const int ps = dir == 0 ? 1 : dir == 1 ? FX_SJ : FX_SK;
+      const int pb = dir == 0 ? FX_SJ * la + FX_SK * lb : dir == 1 ? la + FX_SK * lb : la + FX_SJ * lb;
+      fx_t *Sl = S + lel * FXA_SLOTS * FX_PS;
+      const FxAdjNode ni = fx_adj_load<VF>(Sl, pb + idx * ps, dir);
+      fx_t acc[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+      for (int s = 1; s <= n / 2; ++s) {
+        const int m = idx + s < n ? idx + s : idx + s - n;
+        fx_t g[6];
+        fx_adj_pair<VF>(ni, fx_adj_load<VF>(Sl, pb + m * ps, dir), fx_const(s_Q[idx * n + m]), s_sc[lel], g);
+        const int src = l0 + (idx >= s ? idx - s : idx - s + n);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) gU[1 + k] = ir * g_u[k] - a * u[k];
-    gU[4] = a + gx;
-    // advective surface terms: transposed Riemann-flux Jacobians in this element's face slots
+        for (int v = 0; v < 6; ++v) {
+          acc[v] += g[v];
+          if (2 * s != n) acc[v] += __shfl_sync(0xffffffffu, g[v], src);
+        }
+      }
+      __syncwarp();
+      if (own) {
+#pragma unroll
+        for (int v = 0; v < 6; ++v) Sl[(6 + 8 * dir + v) * FX_PS + pb + idx * ps] = acc[v];
+      }
+    }
+  } else if (on) {
+    double *Se = reinterpret_cast<double *>(S) + le * FXA_SLOTS * FX_PS + fx_idx(node);
+    Se[0] = r; Se[4 * FX_PS] = p; Se[5 * FX_PS] = X;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) Se[(1 + k) * FX_PS] = u[k];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) Se[(6 + k) * FX_PS] = l[k];
+  }
+  __syncthreads();
+  if (!on) return;
+  double gp[6];
+  if (ok) {
+    const fx_t *Se = S + le * FXA_SLOTS * FX_PS + fx_idx(node);
+    const FxAdj &c = s_sc[le];
+    const double w8 = 0.125 * c_invw[0];
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      const fx_t s3 = (Se[(6 + v) * FX_PS] >> 1) + (Se[(14 + v) * FX_PS] >> 1) + (Se[(22 + v) * FX_PS] >> 1);
+      gp[v] = w8 * fx_to(s3, v == 0 ? c.k0 : v < 4 ? c.k1 : v == 4 ? c.kp : c.kx);
+    }
+  } else {
+    double g[6];
+    fx_adj_general_node<VF>(d, reinterpret_cast<const double *>(S) + le * FXA_SLOTS * FX_PS, e, node, g);
+#pragma unroll
+    for (int v = 0; v < 6; ++v) gp[v] = g[v];
+  }
+  const bool ns = d.equations == 1;
+  const double iR = 1.0 / d.R;
+  double g_r = gp[0], g_u[3] = {gp[1], gp[2], gp[3]}, g_p = 4.0 * gp[4];
+  const double g_x = gp[5];
+  if (ns) {  // cotangents of (u, v, w, T) from the viscous adjoint, own part + the neighbours' face shares
+    double cw[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cw[q] = cotW[((size_t)e * 4 + q) * nnn + node];
 #pragma unroll
     for (int dd = 0; dd < 3; ++dd) {
       const int id = ijk[dd];
       if (id != 0 && id != N) continue;
       const int f = 2 * dd + (id == N ? 1 : 0);
-      const int pq = (dd == 0 ? ijk[1] : ijk[0]) + n * (dd == 2 ? ijk[1] : ijk[2]);
-      const double *fs = fslots + ((size_t)e * 6 + f) * 5 * nn + pq;
+      const int pp = dd == 0 ? ijk[1] : ijk[0], qq = dd == 2 ? ijk[1] : ijk[2];
+      int nb, fnb, nbnode, nbpq;
+      neighbour_node(d, e, f, pp, qq, nb, fnb, nbnode, nbpq);
+      const double *sg = sigma + ((size_t)nb * 6 + fnb) * 4 * nn + nbpq;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) gU[v] += fs[v * nn];
+      for (int q = 0; q < 4; ++q) cw[q] += sg[q * nn];
     }
-    const size_t gi = (size_t)e * 5 * nnn + node;
-    if (mode == 0) {
+    g_u[0] += cw[0];
+    g_u[1] += cw[1];
+    g_u[2] += cw[2];
+    g_p += cw[3] * ir * iR;         // T = p / (rho R)
+    g_r -= cw[3] * p * ir * ir * iR;
+  }
+  // chain to U = (rho, m, E): u = m / rho, p = (gamma-1)(E - |m|^2 / (2 rho)), X = h = (E + p)/rho
+  // (Pirozzoli) or e = E/rho (KG). With gx = g_X/rho, p reaches U with weight a = (gamma-1) g_p, and
+  // for h also through E + p: a = (gamma-1)(g_p + gx), and dh/dE = gamma/rho = (gamma-1)/rho + 1/rho
+  const double q2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  const double gx = g_x * ir;
+  const double a = VF == VF_PIR ? gm1 * (g_p + gx) : gm1 * g_p;
+  double gU[5];
+  gU[0] = g_r - ir * (g_u[0] * u[0] + g_u[1] * u[1] + g_u[2] * u[2]) + (0.5 * a) * q2 - gx * X;
 #pragma unroll
-      for (int v = 0; v < 5; ++v) out[gi + v * nnn] = gU[v];
-    } else {  // reverse LSERK stage: Ubar += dt * VJP; gbar = A gbar + B Ubar (gbar is lam, read above)
+  for (int k = 0; k < 3; ++k) gU[1 + k] = ir * g_u[k] - a * u[k];
+  gU[4] = a + gx;
+  // advective surface terms: transposed Riemann-flux Jacobians in this element's face slots
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        const double ub = out[gi + v * nnn] + dt * gU[v];
-        out[gi + v * nnn] = ub;
-        if (update_g) gbar[gi + v * nnn] = A * gbar[gi + v * nnn] + B * ub;
-      }
+  for (int dd = 0; dd < 3; ++dd) {
+    const int id = ijk[dd];
+    if (id != 0 && id != N) continue;
+    const int f = 2 * dd + (id == N ? 1 : 0);
+    const int pq = (dd == 0 ? ijk[1] : ijk[0]) + n * (dd == 2 ? ijk[1] : ijk[2]);
+    const double *fs = fslots + ((size_t)e * 6 + f) * 5 * nn + pq;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) gU[v] += fs[v * nn];
+  }
+  const size_t gi = (size_t)e * 5 * nnn + node;
+  if (mode == 0) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) out[gi + v * nnn] = gU[v];
+  } else {  // reverse LSERK stage: Ubar += dt * VJP; gbar = A gbar + B Ubar (gbar is lam, read above)
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const double ub = out[gi + v * nnn] + dt * gU[v];
+      out[gi + v * nnn] = ub;
+      if (update_g) gbar[gi + v * nnn] = A * gbar[gi + v * nnn] + B * ub;
     }
   }
 }
@@ -740,13 +976,12 @@ template <int VF>
 void launch_adj_volume_t(const DgDevice &d, const double *U, const double *lam, const double *fslots,
                          const double *cotW, const double *sigma, double *out, double *gbar, int mode, double dt,
                          double A, double B, int update_g, cudaStream_t s) {
-  const size_t smem = sizeof(double) * ADJ_EPB * ADJ_SLOTS * PS;
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(k_adj_volume<VF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_adj_volume<VF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FXA_SMEM);
     attr_set = true;
   }
-  k_adj_volume<VF><<<(d.nE + ADJ_EPB - 1) / ADJ_EPB, ADJ_THREADS, smem, s>>>(d, U, lam, fslots, cotW, sigma, out,
+  k_adj_volume<VF><<<(d.nE + FX_EPB - 1) / FX_EPB, FX_THREADS, FXA_SMEM, s>>>(d, U, lam, fslots, cotW, sigma, out,
                                                                             gbar, mode, dt, A, B, update_g);
 }
 

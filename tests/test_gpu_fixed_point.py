@@ -54,7 +54,7 @@ def _state(kind, xyz, N):
     if kind in ("range_ok", "range_general"):  # one corner of the box is thin: max / min of rho and p
         ratio = 100.0 if kind == "range_ok" else 3000.0
         dip = ratio ** -np.exp(-((xyz[:, 0] - 1) ** 2 + (xyz[:, 1] - 1) ** 2 + (xyz[:, 2] - 1) ** 2))
-        rho, p = rho * dip, p * dip
+        rho, p = rho * dip, p * dip ** 0.9  # (another exponent: equal wave speeds on both sides would tie LLF's max)
     return W.cons_from_prim(rho, *vel, p), mu
 
 
@@ -91,3 +91,32 @@ def test_nonfinite_values_pass_through_and_are_flagged(env, N):
     assert torch.isnan(Ut[0]).any()
     # elements are grouped per block: the block's others take the general path, equal to rounding
     assert torch.allclose(Ut[1:], clean[1:], rtol=0, atol=1e-11 * float(clean.abs().max()))
+
+
+@pytest.mark.parametrize("kind,lam_scale", [("mach_1e-6", (1, 1, 1, 1, 1)), ("mach_30", (1, 1, 1, 1, 1)), ("mach_1", (0, 0, 0, 0, 1)),
+                                            ("mach_1", (1e-20, 1, 1, 1, 1e20)), ("units", (1, 1, 1, 1, 1)),
+                                            ("range_ok", (1, 1, 1, 1, 0)), ("range_general", (1, 1, 1, 1, 1))])
+@pytest.mark.parametrize("N,nel,vf", [(1, (5, 2, 1), "kg"), (4, (2, 1, 1), "pirozzoli"), (7, (1, 1, 1), "kg")])
+def test_fixed_point_adjoint_volume_terms(env, kind, lam_scale, N, nel, vf):
+    """The adjoint volume kernel at the same scales, and with cotangents of very different sizes per variable:
+    sampled entries against the oracle's complex-step columns, within 1e-12 of each variable's sum of |terms|."""
+    dg, orc, torch = env
+    xyz, faces = W.box_mesh(N, nel, mapping=_map)
+    U, _ = _state(kind, xyz, N)
+    phys = dict(equations="euler", vflux=vf, sflux="llf")
+    lam = np.random.default_rng(N).standard_normal(U.shape) * np.reshape(lam_scale, (1, 5, 1, 1, 1))
+    gpu = dg.DG(N, xyz, faces, **phys)
+    got = gpu.rhs_vjp(torch.from_numpy(U).cuda(), torch.from_numpy(lam).cuda()).cpu().numpy().reshape(-1)
+    gpu.check()
+    oc = orc.Oracle(N, xyz, faces, complex_step=True, **phys)
+    cols = np.random.default_rng(7).choice(U.size, 60, replace=False)
+    var = (cols // U[0, 0].size) % 5
+    err, scl = np.zeros(5), np.zeros(5)
+    for j, v in zip(cols, var):
+        Z = U.astype(np.complex128)
+        Z.reshape(-1)[j] += 1e-30j
+        col = oc.rhs(Z).imag / 1e-30
+        err[v] = max(err[v], abs(got[j] - (col * lam).sum()))
+        scl[v] = max(scl[v], (np.abs(col) * np.abs(lam)).sum())
+    print(f"FIXED-POINT-ADJ {kind} {lam_scale} N={N} {vf}: {err / np.maximum(scl, 1e-300)}")
+    assert (err <= 1e-12 * scl).all(), (err, scl)
