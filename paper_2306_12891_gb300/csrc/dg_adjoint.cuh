@@ -82,7 +82,7 @@ __device__ void llf_vjp(const double UL[5], const double UR[5], const double nv[
   const double gm1 = gam - 1.0;
   const double rsL = rsq(UL[0]), rsR = rsq(UR[0]);
   const Side L = side_of(UL, nv, gm1, rsL * rsL), R = side_of(UR, nv, gm1, rsR * rsR);
-  const double cL = sqrt(gam * L.p * L.ir), cR = sqrt(gam * R.p * R.ir);
+  const double cL = sqr_int(gam * L.p * L.ir), cR = sqr_int(gam * R.p * R.ir);
   const double aL = fabs(L.un) + cL, aR = fabs(R.un) + cR;
   const bool rwins = aR > aL;  // the forward's max picks the right argument only when strictly larger
   const double lam = rwins ? aR : aL;
@@ -100,11 +100,11 @@ __device__ void llf_vjp(const double UL[5], const double UR[5], const double nv[
   // lam = |un_X| + sqrt(gamma p_X / rho_X) of the winning side X
   if (rwins) {
     cunR += clam * sgn_of(R.un);
-    cpR += clam * 0.5 * cR / R.p;
+    cpR += clam * 0.5 * cR * rcp_int(R.p);
     gR[0] -= clam * 0.5 * cR * R.ir;
   } else {
     cunL += clam * sgn_of(L.un);
-    cpL += clam * 0.5 * cL / L.p;
+    cpL += clam * 0.5 * cL * rcp_int(L.p);
     gL[0] -= clam * 0.5 * cL * L.ir;
   }
   side_back(UL, L, nv, gm1, cuL, cpL, cunL, cirL, gL);
@@ -121,7 +121,7 @@ __device__ void roe_vjp(const double UL[5], const double UR[5], const double nv[
   const Side L = side_of(UL, nv, gm1, rsL * rsL), R = side_of(UR, nv, gm1, rsR * rsR);
   // forward
   const double sL = UL[0] * rsL, sR = UR[0] * rsR;
-  const double iw = 1.0 / (sL + sR);
+  const double iw = rcp_int(sL + sR);
   double ut[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) ut[k] = (sL * L.u[k] + sR * R.u[k]) * iw;
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(LIFT_THREADS) k_adj_visc(const DgDevice d, con
     const int le = t / nnn, node = t % nnn, e = e0 + le;
     if (e >= d.nE) continue;
     const size_t gi = (size_t)e * 5 * nnn + node;
-    const double ir = 1.0 / U[gi];  // u as the lifting forms it
+    const double ir = rcp_int(U[gi]);  // u as the lifting forms it
     double *W = Ws + le * 3 * nnn + node;
     W[0] = U[gi + nnn] * ir;
     W[nnn] = U[gi + 2 * nnn] * ir;
@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
       double Uv[5];
       load_state<double>(d, U, e, node, Uv);
       r = Uv[0];
-      ir = 1.0 / r;
+      ir = rcp_int(r);
 #pragma unroll
       for (int k = 0; k < 3; ++k) u[k] = Uv[1 + k] * ir;
       p = gm1 * (Uv[4] - 0.5 * (Uv[1] * u[0] + Uv[2] * u[1] + Uv[3] * u[2]));

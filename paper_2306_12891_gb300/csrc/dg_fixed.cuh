@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
       const double *Je = d.Ja + (size_t)e * 9 * nnn + node;
 #pragma unroll
       for (int k = 0; k < 9; ++k) J[k] = __ldg(Je + k * nnn);
-      const double r = Uv[0], ir = 1.0 / r;
+      const double r = Uv[0], ir = rcp_int(r);
       const double u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
       const double p = gm1 * (Uv[4] - 0.5 * (Uv[1] * u + Uv[2] * v + Uv[3] * w));
       const double x = VF == VF_PIR ? (Uv[4] + p) * ir : Uv[4] * ir;
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
       if (al > 0.0) {
         double Uv[5];
         load_state<double>(d, U, e, node, Uv);
-        const double ir = 1.0 / Uv[0];
+        const double ir = rcp_int(Uv[0]);
         const double u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
         double *P = P0 + le * FX_SLOTS * FX_PS + fx_idx(node);
         P[0] = Uv[0]; P[FX_PS] = u; P[2 * FX_PS] = v; P[3 * FX_PS] = w;

@@ -11,15 +11,16 @@
 //   acc[6]    += wq rho|u|^2 / 2                  (kinetic energy)
 //   acc[7]    += wq (u . (rho u)_t - |u|^2 rho_t / 2)   (its rate)
 #pragma once
+#include "dg_recip.cuh"
 
 __device__ __forceinline__ void invariants_node(double gam, double wq, const double Uv[5], const double Tv[5],
                                                 double acc[8]) {
-  const double r = Uv[0], ir = 1.0 / r;
+  const double r = Uv[0], ir = rcp_int(r);
   const double u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
   const double q2 = u * u + v * v + w * w;
   const double p = (gam - 1.0) * (Uv[4] - 0.5 * r * q2);
   const double s = log(p) - gam * log(r);
-  const double ip = 1.0 / p;
+  const double ip = rcp_int(p);
   const double ev[5] = {(gam - s) / (gam - 1.0) - 0.5 * r * q2 * ip, r * u * ip, r * v * ip, r * w * ip, -r * ip};
 #pragma unroll
   for (int m = 0; m < 5; ++m) acc[m] += wq * Tv[m];

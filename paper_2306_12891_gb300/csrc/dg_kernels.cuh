@@ -34,6 +34,7 @@
 #include "dg_convert.cuh"
 #include "dg_internal.h"
 #include "dg_invariants_node.cuh"
+#include "dg_recip.cuh"
 #include "dg_wall.cuh"
 
 #ifndef DG_N
@@ -228,8 +229,12 @@ __global__ void __launch_bounds__(256) k_shadow(const DgDevice d, const double *
 // pointwise physics (pressure p' = p - p_ref enters the momentum flux; p_ref = 0 in FP64)
 // ---------------------------------------------------------------------------------------------
 
-__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rsq(double x) { return rsq_int(x); }
 __device__ __forceinline__ float rsq(float x) { return rsqrtf(x); }
+template <typename R> __device__ __forceinline__ R rcp(const R &x) { return R(1) / x; }
+template <> __device__ __forceinline__ double rcp<double>(const double &x) { return rcp_int(x); }
+template <typename R> __device__ __forceinline__ R root(const R &x) { return sqrt(x); }
+template <> __device__ __forceinline__ double root<double>(const double &x) { return sqr_int(x); }
 
 // one side of a Riemann problem: conservative state, velocity, p' and the true pressure, 1/sqrt(rho), 1/rho
 template <typename R>
@@ -271,9 +276,9 @@ __device__ __forceinline__ void log_ratio(R a, R b, R f, R &F, R &G) {
 template <typename R>
 __device__ __forceinline__ void ec_flux(R rL, R uL, R vL, R wL, R bL, R rR, R uR, R vR, R wR, R bR, const R a[3], R igm1,
                                         R pref, R F[5]) {
-  const R Sr = rL + rR, Sb = bL + bR, iSb = R(1) / Sb;
+  const R Sr = rL + rR, Sb = bL + bR, iSb = rcp<R>(Sb);
   R Fr, Gr, Fb, Gb;
-  log_ratio<R>(rL, rR, (rL - rR) / Sr, Fr, Gr);
+  log_ratio<R>(rL, rR, (rL - rR) * rcp<R>(Sr), Fr, Gr);
   log_ratio<R>(bL, bR, (bL - bR) * iSb, Fb, Gb);
   const R um = R(0.5) * (uL + uR), vm = R(0.5) * (vL + vR), wm = R(0.5) * (wL + wR);
   const R h0 = R(0.5) * Sr * iSb, phat = h0 + (R(0.5) * Sr - h0 * Sb) * iSb - pref;  // the quotient to its last bit
@@ -308,14 +313,15 @@ __device__ __forceinline__ void riemann_sides(int sf, const RSide<R> &L, const R
   const R irL = L.ir, irR = Q.ir, rsL = L.rs, rsR = Q.rs, pL = L.p, pR = Q.p;
   const R uL = L.u[0], vL = L.u[1], wL = L.u[2], uR = Q.u[0], vR = Q.u[1], wR = Q.u[2];
   if (sf == SF_EC) {
-    ec_flux<R>(UL[0], uL, vL, wL, R(0.5) * UL[0] / pL, UR[0], uR, vR, wR, R(0.5) * UR[0] / pR, nv, R(1) / gm1,
+    ec_flux<R>(UL[0], uL, vL, wL, R(0.5) * UL[0] * rcp<R>(pL), UR[0], uR, vR, wR, R(0.5) * UR[0] * rcp<R>(pR), nv,
+               rcp<R>(gm1),
                kShift<R> ? pref : R(0), F);
     return;
   }
   R FL[5], FR[5];
   const R unL = euler_flux<R>(L, href, nv, FL), unR = euler_flux<R>(Q, href, nv, FR);
   if (sf == SF_LLF) {
-    const R cL = sqrt(gam * pL * irL), cR = sqrt(gam * pR * irR);
+    const R cL = root<R>(gam * pL * irL), cR = root<R>(gam * pR * irR);
     const R lam = fmax(fabs(unL) + cL, fabs(unR) + cR);
 #pragma unroll
     for (int v = 0; v < 5; ++v) F[v] = R(0.5) * (FL[v] + FR[v] - lam * (UR[v] - UL[v]));
@@ -325,7 +331,7 @@ __device__ __forceinline__ void riemann_sides(int sf, const RSide<R> &L, const R
   // s = sqrt(rho), the weight of side k is s_k / (s_L + s_R), so the averages of u and H are
   // sum_k (m_k / s_k) / (s_L + s_R) = sum_k a_k m_k with a_k = (1/sqrt(rho_k)) / (s_L + s_R).
   const R sL = UL[0] * rsL, sR = UR[0] * rsR;
-  const R iw = R(1) / (sL + sR);
+  const R iw = rcp<R>(sL + sR);
   const R aL = rsL * iw, aR = rsR * iw;
   const R ut = aL * UL[1] + aR * UR[1], vt = aL * UL[2] + aR * UR[2], wt = aL * UL[3] + aR * UR[3];
   const R EpL = kShift<R> ? UL[4] + pL - pref + href : UL[4] + pL;  // E + p
@@ -602,7 +608,7 @@ __global__ void __launch_bounds__(FACE_THREADS) k_face(const DgDevice d, const d
 // (u, v, w, T) of one node from its state values (lifted quantities of BR1)
 template <typename R>
 __device__ __forceinline__ void lift_prim(const R Uv[5], R gm1, R iR, R pref, R Wn[4]) {
-  const R r = Uv[0], ir = R(1) / r;
+  const R r = Uv[0], ir = rcp<R>(r);
   const R u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
   R p = gm1 * (Uv[4] - R(0.5) * r * (u * u + v * v + w * w));
   if (kShift<R>) p += pref;
@@ -951,7 +957,7 @@ __global__ void __launch_bounds__(vol_threads<R, SC>(), vol_min_blocks<R, SC>())
     R Uv[5];
     load_state<R>(d, U, e, node, Uv);
     const R r = Uv[0], m1 = Uv[1], m2 = Uv[2], m3 = Uv[3], E = Uv[4];
-    const R ir = R(1) / r;
+    const R ir = rcp<R>(r);
     const R u = m1 * ir, v = m2 * ir, w = m3 * ir;
     const R pm = gm1 * (E - R(0.5) * (m1 * u + m2 * v + m3 * w));  // p' (= p in FP64)
     const R p = kShift<R> ? pm + pref : pm;
@@ -961,7 +967,7 @@ __global__ void __launch_bounds__(vol_threads<R, SC>(), vol_min_blocks<R, SC>())
     Pe[0] = r; Pe[PS] = u; Pe[2 * PS] = v; Pe[3 * PS] = w; Pe[4 * PS] = R(4) * pm;
     if (vf == VF_PIR) Pe[5 * PS] = (Et + p) * ir;
     else if (vf == VF_KG) { Pe[5 * PS] = Et * ir; Pe[6 * PS] = R(2) * p; }
-    else if (vf == VF_EC) Pe[6 * PS] = R(0.5) * r / p;  // beta
+    else if (vf == VF_EC) Pe[6 * PS] = R(0.5) * r * rcp<R>(p);  // beta
     else Pe[5 * PS] = Et + p;
     if (SC) Pe[7 * PS] = pm;
   }
