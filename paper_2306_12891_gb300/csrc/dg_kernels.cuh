@@ -534,7 +534,7 @@ __device__ __forceinline__ void wall_face(const DgDevice &d, const double *__res
   R tw[3] = {R(0), R(0), R(0)};
   if (Ut > R(0)) {
     int it;
-    const R utau = wall_utau<R>(Ut, (R)d.hwm[(size_t)f * nn + pq], Cst<R>::mu(d) * irx, (R)d.wm_uinf, (R)d.wm_b,
+    const R utau = wall_utau<R, true>(Ut, (R)d.hwm[(size_t)f * nn + pq], Cst<R>::mu(d) * irx, (R)d.wm_uinf, (R)d.wm_b,
                                 d.wm_vd, it);
     const R tau = Ux[0] * utau * utau;
 #pragma unroll
