@@ -85,7 +85,7 @@ struct dg_ctx {
   bool tape_all = false;
   double tape_dt = 0.0;
   double fac_dt = std::nan("");  // step size of the FP32-bulk stage factor d.facf (NaN: not formed yet)
-  // CUDA graph of one LSERK step, replayed by the multi-step calls on a library stream that is
+  // CUDA graph of up to kGraphSteps LSERK steps, replayed by the multi-step calls on a library stream that is
   // ordered after (and before) the caller's stream with events
   int use_graphs = 1;
   cudaStream_t gstream = nullptr;
@@ -95,7 +95,9 @@ struct dg_ctx {
   static constexpr int kCopyStreams = 4;
   cudaStream_t cstream[kCopyStreams] = {};
   cudaEvent_t cev[kCopyStreams + 1] = {};
+  static constexpr int kGraphSteps = 16;
   cudaGraphExec_t step_graph = nullptr;
+  int graph_steps = 0;
   const double *graph_U = nullptr;
   double graph_dt = 0.0;
   long long graph_launches = 0;
@@ -607,15 +609,15 @@ dg_status plain_steps(dg_ctx *c, double *U, double dt, int n_steps) {
   return DG_OK;
 }
 
-// capture one LSERK step on U with step dt into c->step_graph (launches go to the library stream)
-dg_status capture_step(dg_ctx *c, double *U, double dt) {
+// capture n_steps LSERK steps on U with step dt into c->step_graph (launches go to the library stream)
+dg_status capture_steps(dg_ctx *c, double *U, double dt, int n_steps) {
   if (c->step_graph) { cudaGraphExecDestroy(c->step_graph); c->step_graph = nullptr; }
   cudaStream_t user = c->stream;
   c->stream = c->gstream;
   const long long l0 = c->launches;
   cudaError_t e = cudaStreamBeginCapture(c->gstream, cudaStreamCaptureModeThreadLocal);
   dg_status st = e ? DG_ERR_CUDA : DG_OK;
-  if (st == DG_OK) st = plain_steps(c, U, dt, 1);
+  if (st == DG_OK) st = plain_steps(c, U, dt, n_steps);
   cudaGraph_t g = nullptr;
   if (!e) {
     const cudaError_t e2 = cudaStreamEndCapture(c->gstream, &g);
@@ -634,12 +636,13 @@ dg_status capture_step(dg_ctx *c, double *U, double dt) {
   if (st != DG_OK) return st;
   c->graph_U = U;
   c->graph_dt = dt;
+  c->graph_steps = n_steps;
   return DG_OK;
 }
 
-// n_steps LSERK steps. With graphs on (and kernel timing off) the step's launch sequence is
-// captured once per (U, dt) and replayed: one graph launch per step instead of 10-20 kernel
-// launches, which is what bounds small meshes.
+// n_steps LSERK steps. With graphs on (and kernel timing off) the launch sequence of up to kGraphSteps steps is
+// captured once per (U, dt) and replayed, one graph launch instead of 160-320 kernel launches; steps that do not fill
+// a graph are launched. (One step per graph left a gap between graphs that the dependent launches within do not have.)
 dg_status steps_impl(dg_ctx *c, double *U, double dt, int n_steps) {
   DG_TRY(refresh_shadow(c, U));
   DG_TRY(ensure_stage_factor(c, dt));
@@ -655,20 +658,23 @@ dg_status steps_impl(dg_ctx *c, double *U, double dt, int n_steps) {
   if (!(c->step_graph && c->graph_U == U && c->graph_dt == dt)) {
     DG_TRY(plain_steps(c, U, dt, 1));  // first step directly (also sets kernel attributes outside capture)
     --n_steps;
-    if (capture_step(c, U, dt) != DG_OK) {  // no graph on this stream: launch the kernels directly
-      c->use_graphs = 0;
+    if (capture_steps(c, U, dt, std::min(n_steps, dg_ctx::kGraphSteps)) != DG_OK) {
+      c->use_graphs = 0;  // no graph on this stream: launch the kernels directly
       c->err.clear();
       return plain_steps(c, U, dt, n_steps);
     }
   }
-  e = cudaEventRecord(c->gev_in, c->stream);
-  if (!e) e = cudaStreamWaitEvent(c->gstream, c->gev_in, 0);
-  for (int k = 0; k < n_steps && !e; ++k) e = cudaGraphLaunch(c->step_graph, c->gstream);
-  if (!e) e = cudaEventRecord(c->gev_out, c->gstream);
-  if (!e) e = cudaStreamWaitEvent(c->stream, c->gev_out, 0);
-  if (e) return cuda_fail(c, e, "step graph launch");
-  c->launches += c->graph_launches * n_steps;
-  return DG_OK;
+  const int replays = n_steps / c->graph_steps;
+  if (replays > 0) {
+    e = cudaEventRecord(c->gev_in, c->stream);
+    if (!e) e = cudaStreamWaitEvent(c->gstream, c->gev_in, 0);
+    for (int k = 0; k < replays && !e; ++k) e = cudaGraphLaunch(c->step_graph, c->gstream);
+    if (!e) e = cudaEventRecord(c->gev_out, c->gstream);
+    if (!e) e = cudaStreamWaitEvent(c->stream, c->gev_out, 0);
+    if (e) return cuda_fail(c, e, "step graph launch");
+    c->launches += c->graph_launches * replays;
+  }
+  return plain_steps(c, U, dt, n_steps % c->graph_steps);
 }
 // state copy by the SMs through the host-device link, 16 bytes per thread and step; for page-locked host
 // memory, which the device addresses directly

@@ -382,6 +382,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
   for (int t = tid; t < FX_H * FX_H; t += FX_THREADS) s_rho[t] = c_rho[t];
   for (int t = tid; t < nn; t += FX_THREADS) s_Q[t] = c_Qx[t];
   for (int t = tid; t < n * FX_QV; t += FX_THREADS) s_QV[t] = c_QV[t];
+  wait_for_previous();
   __syncthreads();
   // phase A: primitive quantities of the thread's node and the element maxima
   const int le = tid / nnn, node = tid % nnn, e = e0 + le;
@@ -495,6 +496,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
     for (int k = 0; k < 6; ++k) Se[k * FX_PS] = q[k];
   }
   __syncthreads();
+  let_next_start();
   // phase C: per node -- directions summed, surface terms, neighbour's viscous flux, blend, Jacobian, output / LSERK
   const int ijk[3] = {node % n, (node / n) % n, node / nn};
   double s[5];

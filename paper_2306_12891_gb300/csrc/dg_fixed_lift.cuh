@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice 
   if (tid < 2 * FX_EPB) s_mx[tid >> 1][tid & 1] = s_my[tid >> 1][tid & 1] = s_fv[tid >> 1][tid & 1] = 0;
   for (int t = tid; t < FX_H; t += FX_THREADS) s_rho[t] = c_rho[t * FX_H];  // w_0 / w
   for (int t = tid; t < n * FX_QV; t += FX_THREADS) s_QD[t] = c_QD[t];
+  wait_for_previous();
   __syncthreads();
   const int le = tid / nnn, node = tid % nnn, e = e0 + le;
   const bool on = tid < FX_EPB * nnn && e < d.nE;
@@ -200,6 +201,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice 
     __syncthreads();
     if (tid < FX_EPB) fx_lift_scales(s_sc[tid], s_my[tid][0], s_my[tid][1]);
     __syncthreads();
+    let_next_start();
     // phase C: per node -- metric contraction, stress, heat flux, contravariant viscous flux
     if (on) {
       const FxLift &c = s_sc[le];
