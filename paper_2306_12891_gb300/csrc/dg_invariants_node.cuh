@@ -13,15 +13,17 @@
 #pragma once
 #include "dg_recip.cuh"
 
-__device__ __forceinline__ void invariants_node(double gam, double wq, const double Uv[5], const double Tv[5],
-                                                double acc[8]) {
+// igm1 = 1/(gamma - 1); ln: the natural logarithm to use
+template <class Log>
+__device__ __forceinline__ void invariants_node(double gam, double igm1, double wq, const double Uv[5], const double Tv[5],
+                                                double acc[8], Log ln) {
   const double r = Uv[0], ir = rcp_int(r);
   const double u = Uv[1] * ir, v = Uv[2] * ir, w = Uv[3] * ir;
   const double q2 = u * u + v * v + w * w;
   const double p = (gam - 1.0) * (Uv[4] - 0.5 * r * q2);
-  const double s = log(p) - gam * log(r);
+  const double s = ln(p) - gam * ln(r);
   const double ip = rcp_int(p);
-  const double ev[5] = {(gam - s) / (gam - 1.0) - 0.5 * r * q2 * ip, r * u * ip, r * v * ip, r * w * ip, -r * ip};
+  const double ev[5] = {(gam - s) * igm1 - 0.5 * r * q2 * ip, r * u * ip, r * v * ip, r * w * ip, -r * ip};
 #pragma unroll
   for (int m = 0; m < 5; ++m) acc[m] += wq * Tv[m];
   acc[5] += wq * (ev[0] * Tv[0] + ev[1] * Tv[1] + ev[2] * Tv[2] + ev[3] * Tv[3] + ev[4] * Tv[4]);

@@ -34,6 +34,7 @@
 #include "dg_convert.cuh"
 #include "dg_internal.h"
 #include "dg_invariants_node.cuh"
+#include "dg_log.cuh"
 #include "dg_recip.cuh"
 #include "dg_wall.cuh"
 
@@ -1257,9 +1258,14 @@ __global__ void __launch_bounds__(256) k_spread(const DgDevice d, double *alpha_
 // ---------------------------------------------------------------------------------------------
 // reductions: integral invariants and the time-step estimate (deterministic two-pass, FP64)
 // ---------------------------------------------------------------------------------------------
+__constant__ LogEntry c_log[LOG_TABLE];
+
 __global__ void __launch_bounds__(256) k_invariants(const DgDevice d, const double *__restrict__ U,
                                                     const double *__restrict__ Ut) {
   __shared__ double red[8][256];
+  __shared__ LogEntry s_log[LOG_TABLE];
+  for (int t = threadIdx.x; t < LOG_TABLE; t += 256) s_log[t] = c_log[t];
+  __syncthreads();
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   const long long total = (long long)d.nE * nnn;
   const double gam = d.gamma;
@@ -1271,7 +1277,7 @@ __global__ void __launch_bounds__(256) k_invariants(const DgDevice d, const doub
     double Uv[5], Tv[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) { Uv[v] = U[b + v * nnn]; Tv[v] = Ut[b + v * nnn]; }
-    invariants_node(gam, wq, Uv, Tv, acc);
+    invariants_node(gam, d.igm1, wq, Uv, Tv, acc, [&](double x) { return log_int(x, s_log); });
   }
 #pragma unroll
   for (int m = 0; m < 8; ++m) red[m][threadIdx.x] = acc[m];
@@ -1419,7 +1425,10 @@ cudaError_t upload(const DgTables &t) {
   ihx[0] = 0.0;
   for (int i = 1; i < n; ++i) ihx[i] = 1.0 / (t.xi[i] - t.xi[i - 1]);
   for (int i = 0; i < n; ++i) fihx[i] = (float)ihx[i];
+  LogEntry lt[LOG_TABLE];
+  log_table(lt);
   cudaError_t err = fx_upload(t);
+  err = err ? err : cudaMemcpyToSymbol(c_log, lt, sizeof(lt));
   err = err ? err : fx_lift_upload(t);
   err = err ? err : cudaMemcpyToSymbol(c_ihx, ihx, sizeof(double) * n);
   err = err ? err : cudaMemcpyToSymbol(c_VP, vp, sizeof(vp));

@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(kThreads) k_invariants_chunks(int n, long long
   __shared__ double red[8][kThreads];
   const int nn = n * n, nnn = nn * n;
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  const double igm1 = 1.0 / (gam - 1.0);
   const long long begin = (long long)blockIdx.x * kChunk;
   const long long end = begin + kChunk < total ? begin + kChunk : total;
   for (long long t = begin + threadIdx.x; t < end; t += kThreads) {
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(kThreads) k_invariants_chunks(int n, long long
     double Uv[5], Tv[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) { Uv[v] = U[b + (size_t)v * nnn]; Tv[v] = Ut[b + (size_t)v * nnn]; }
-    invariants_node(gam, wq, Uv, Tv, acc);
+    invariants_node(gam, igm1, wq, Uv, Tv, acc, [](double x) { return log(x); });
   }
 #pragma unroll
   for (int m = 0; m < 8; ++m) red[m][threadIdx.x] = acc[m];
