@@ -230,7 +230,7 @@ dg_status dg_check(dg_ctx *ctx);
 dg_status dg_get_metrics(dg_ctx *ctx, double *Ja, double *J);
 
 /* The FP32-bulk volume operator without the blend (N = 3, 5, 7 and 16-byte aligned U, Ut, g):
- * 3 (default; N = 7, other N take mode 2): a persistent kernel whose line threads form each
+ * 3 (default; N = 7, other N take mode 1): a persistent kernel whose line threads form each
  * two-point flux once for both of its nodes (pair symmetry) while separate warps apply the FP64
  * epilogue to the previous element; inputs arrive by TMA bulk copies one element ahead.
  * 2: the same pipeline with one thread per node; 1: mode 2 without warp specialisation; 0: the

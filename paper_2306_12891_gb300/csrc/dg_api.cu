@@ -486,7 +486,7 @@ dg_status dg_init(const dg_mesh *mesh, int N, int nodes, const dg_params *prm, v
   d.href_f = (float)d.href;
   d.mu_f = (float)d.mu;
   d.kappa_f = (float)d.kappa;
-  d.use_tma = 3;  // N = 7: pair-symmetric line kernel; other N: warp-specialised node kernel
+  d.use_tma = 3;  // N = 7: pair-symmetric line kernel; other N: TMA-fed node kernel
   d.n_walls = n_walls;
   d.wm_index = prm->wm_index;
   d.wm_vd = prm->wm_van_driest ? 1 : 0;

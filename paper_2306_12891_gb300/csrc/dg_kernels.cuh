@@ -1596,7 +1596,11 @@ void launch_volume_f32(const DgDevice &d, const double *U, double *out, double *
     k_volume_f32_line<VF><<<blocks, LN_THREADS, LN_SMEM, s>>>(d, U, out, g, mode, first, dt, A, B);
     return;
   }
-  if (TMA_OK && d.use_tma >= 2 && aligned) {  // warp-specialised persistent kernel
+  // warp-specialised persistent kernel: on request, and where the line kernel cannot run at N = 7. At N = 3 and 5 its few
+  // warps per SM leave it behind the TMA-fed node kernel below, which gives the same bits (right-hand side / LSERK stage:
+  // N = 5, 17 x 13 x 11: 69.6 / 74 against 45.2 / 54 us; 32^3: 903 / 945 against 529 / 641 us; N = 3, 32^3: 373 / 380
+  // against 128 / 163 us)
+  if (TMA_OK && (d.use_tma == 2 || (d.use_tma == 3 && LN_OK)) && aligned) {
     static int grid_ws = 0;
     if (!grid_ws) {
       cudaFuncSetAttribute(k_volume_f32_ws<VF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WS_SMEM);

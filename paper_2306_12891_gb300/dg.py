@@ -328,7 +328,7 @@ class DG:
         return Ja, J
 
     def use_tma(self, mode=3):
-        """FP32-bulk volume kernel: 3 pair-symmetric line kernel (default; N = 7, else mode 2),
+        """FP32-bulk volume kernel: 3 pair-symmetric line kernel (default; N = 7, else mode 1),
         2 warp-specialised node kernel, 1 TMA node kernel, 0 plain node kernel."""
         self._check(lib().dg_use_tma(self._ctx, int(mode)), "dg_use_tma")
 
