@@ -293,10 +293,24 @@ __global__ void __launch_bounds__(128) k_adj_face(const DgDevice d, const double
 // The flux is linear in the lifted gradients except for the work term u.tau, whose derivative
 // needs the viscous stress tau at the state: the forward lifting records it per node (the record
 // the reverse sweep keeps with each stage state), so no gradient is formed here.
-// shared memory per element: W[3][nnn] (u, v, w), L[4][nnn] (l of momentum and energy),
-// H[12][nnn] (cotangent of the direction-d reference derivative of w_q), Om[3][nnn]
+//
+// One thread per node. In FP64 the node's two D^T sweeps are 24 n products of ~120 others, on a pipe of two
+// lanes per clock and SM (92 % busy, N = 5). They are formed in the fixed point of dg_fixed.cuh instead
+// (3 IMAD.WIDE each, ~25 lanes per clock), from values at the element's largest per variable; an element whose
+// values leave the range of the scales (infinities, NaN, magnitudes near the ends of FP64) keeps FP64 sweeps.
+// Windows (value x scale, log2): D_mi / 32 < 62, a column sum of |D| / 32 <= 0.81 (N = 7); l and H < 60; one
+// direction's cross sums < 62.4; results 2^-56 (2^-55 with three directions summed) of the largest value, where
+// the FP64 sums round at 2^-53 of their partial sums, ~10 times the largest value.
+// Per launch at N = 5, 12^3: 225 us with FP64 sweeps, 131 us (errors of the product against extended precision 0.77 to
+// 0.95 of those with FP64 kernels).
+// The diagonal of D in the second sweep, D_00 = -N(N+1)/4 = -D_NN, is the face term (1/w_b)(+-1/2): they cancel.
+// shared memory per element: L[4][nnn] (l of momentum and energy), H[12][nnn] (cotangent of the
+// direction-d reference derivative of w_q), as fixed-point values or (general path) doubles
 // ---------------------------------------------------------------------------------------------
-constexpr int ADJV_SLOTS = 22;
+constexpr int ADJV_SLOTS = 16;
+constexpr int ADJV_THREADS = round32(LIFT_EPB * nnn);
+constexpr int ADJV_BLOCKS = ADJV_THREADS >= 512 ? 1 : 896 / ADJV_THREADS;  // per SM (bounds the registers)
+constexpr int ADJV_DROP = 3;
 
 // the neighbour's volume node facing face point (pp, qq) of element e's face f
 __device__ __forceinline__ void neighbour_node(const DgDevice &d, size_t e, int f, int pp, int qq, int &nb, int &fnb,
@@ -310,40 +324,98 @@ __device__ __forceinline__ void neighbour_node(const DgDevice &d, size_t e, int 
   nbpq = p2 + n * q2;
 }
 
-__global__ void __launch_bounds__(LIFT_THREADS) k_adj_visc(const DgDevice d, const double *__restrict__ U,
-                                                           const double *__restrict__ lam,
-                                                           const double *__restrict__ tau, double *__restrict__ cotW,
-                                                           double *__restrict__ sigma) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  double *Ws = reinterpret_cast<double *>(sm_raw);  // [EPB][3][nnn]
-  double *Ls = Ws + LIFT_EPB * 3 * nnn;              // [EPB][4][nnn]
-  double *Hs = Ls + LIFT_EPB * 4 * nnn;              // [EPB][12][nnn]
-  double *Os = Hs + LIFT_EPB * 12 * nnn;             // [EPB][3][nnn]
-  // D in shared memory, rows padded: the sweeps index it by the thread's own node, which would
-  // serialise a constant-memory load
-  __shared__ double sD[n][n + 1];
-  for (int t = threadIdx.x; t < nn; t += blockDim.x) sD[t / n][t % n] = c_D[t];
-  const int e0 = blockIdx.x * LIFT_EPB;
-  for (int t = threadIdx.x; t < LIFT_EPB * nnn; t += blockDim.x) {
-    const int le = t / nnn, node = t % nnn, e = e0 + le;
-    if (e >= d.nE) continue;
-    const size_t gi = (size_t)e * 5 * nnn + node;
-    const double ir = rcp_int(U[gi]);  // u as the lifting forms it
-    double *W = Ws + le * 3 * nnn + node;
-    W[0] = U[gi + nnn] * ir;
-    W[nnn] = U[gi + 2 * nnn] * ir;
-    W[2 * nnn] = U[gi + 3 * nnn] * ir;
-    const double miJ = -d.invJ[(size_t)e * nnn + node];
+// the largest |x| of an element (high word) for its threads' values x[4][K], into mx[4]
+template <int K>
+__device__ __forceinline__ void adjv_max(const double (&x)[K][4], bool on, int *mx) {
+  constexpr bool WARP = LIFT_EPB == 1 || nnn % 32 == 0;  // a warp's nodes belong to one element
 #pragma unroll
-    for (int q = 0; q < 4; ++q) Ls[(le * 4 + q) * nnn + node] = miJ * lam[gi + (1 + q) * nnn];
+  for (int q = 0; q < 4; ++q) {
+    int h = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) h = max(h, on ? fx_hi_abs(x[k][q]) : 0);
+    if (WARP) {
+      h = __reduce_max_sync(0xffffffffu, h);
+      if (threadIdx.x % 32 == 0) atomicMax(mx + q, h);
+    } else if (on) {
+      atomicMax(mx + q, h);
+    }
+  }
+}
+// fixed-point exponents of the four variables; false: the element takes the FP64 sweeps
+__device__ __forceinline__ bool adjv_scale(const int *mx, int E[4]) {
+  bool ok = true;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int ex = fx_exponent(mx[q]);
+    E[q] = max(ex, 128);
+    ok = ok && (mx[q] == 0 || (ex >= 128 && ex <= 1900));
+  }
+  return ok;
+}
+__device__ __forceinline__ long long adjv_store(double x, bool fx, int E) {
+  return fx ? fx_from(x, E, ADJV_DROP) + FX_BIAS : __double_as_longlong(x);
+}
+// r[q] = sum_m D_mi x_q,m along a line (S at node 0 of it, q apart by nnn): fixed value, window a
+__device__ __forceinline__ void adjv_sweep(const long long *S, int st, const int2 *row, int a, fx_t r[4]) {
+  FxSum s[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) s[q] = fx_zero(a);
+#pragma unroll
+  for (int m = 0; m < n; ++m) {
+    const FxD w = fx_const(row[m]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) fx_acc(s[q], w, fx_biased(S[q * nnn + m * st]));
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) r[q] = fx_value(s[q], a);
+}
+__device__ __noinline__ double adjv_sweep_general(const long long *S, int st, int id) {
+  double r = 0.0;
+#pragma unroll 1
+  for (int m = 0; m < n; ++m)
+    if (m != id) r += c_D[m * n + id] * __longlong_as_double(S[m * st]);
+  return r;
+}
+
+__global__ void __launch_bounds__(ADJV_THREADS, ADJV_BLOCKS)
+    k_adj_visc(const DgDevice d, const double *__restrict__ U, const double *__restrict__ lam,
+               const double *__restrict__ tau, double *__restrict__ cotW, double *__restrict__ sigma) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  long long *Ls = reinterpret_cast<long long *>(sm_raw);  // [EPB][4][nnn]
+  long long *Hs = Ls + LIFT_EPB * 4 * nnn;                // [EPB][12][nnn]
+  // D^T in shared memory, rows padded: the sweeps index it by the thread's own node, which would
+  // serialise a constant-memory load
+  __shared__ int2 sD[n][n + 1];
+  __shared__ int s_mx[LIFT_EPB][2][4];
+  for (int t = threadIdx.x; t < nn; t += blockDim.x) sD[t / n][t % n] = c_DT[t];
+  for (int t = threadIdx.x; t < LIFT_EPB * 8; t += blockDim.x) (&s_mx[0][0][0])[t] = 0;
+  __syncthreads();
+  const int le = threadIdx.x / nnn < LIFT_EPB ? threadIdx.x / nnn : LIFT_EPB - 1, node = threadIdx.x % nnn;
+  const int e = blockIdx.x * LIFT_EPB + le;
+  const bool on = threadIdx.x < LIFT_EPB * nnn && e < d.nE;
+  const size_t gi = (size_t)e * 5 * nnn + node;
+  const int ijk[3] = {node % n, (node / n) % n, node / nn};
+  double l[1][4], u[3], iJ;
+  if (on) {
+    const double ir = rcp_int(U[gi]);  // u as the lifting forms it
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[k] = U[gi + (1 + k) * nnn] * ir;
+    iJ = d.invJ[(size_t)e * nnn + node];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) l[0][q] = -iJ * lam[gi + (1 + q) * nnn];
+  }
+  adjv_max<1>(l, on, s_mx[le][0]);
+  __syncthreads();
+  int E[4];
+  bool fx = adjv_scale(s_mx[le][0], E);
+  long long *L = Ls + le * 4 * nnn, *H = Hs + le * 12 * nnn;
+  if (on) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) L[q * nnn + node] = adjv_store(l[0][q], fx, E[q]);
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < LIFT_EPB * nnn; t += blockDim.x) {
-    const int le = t / nnn, node = t % nnn, e = e0 + le;
-    if (e >= d.nE) continue;
-    const int ijk[3] = {node % n, (node / n) % n, node / nn};
-    const double *W = Ws + le * 3 * nnn;
-    const double *L = Ls + le * 4 * nnn;
+  double h[3][4], om[3];
+  if (on) {
     // reverse seed: zeta[dd][q] = cotangent of the contravariant viscous flux Fv^dd_q at this node
     double zeta[3][4];
 #pragma unroll
@@ -351,13 +423,14 @@ __global__ void __launch_bounds__(LIFT_THREADS) k_adj_visc(const DgDevice d, con
       const int id = ijk[dd];
       const int st = dd == 0 ? 1 : dd == 1 ? n : nn;
       const int base = node - id * st;
+      if (fx) {
+        fx_t r[4];
+        adjv_sweep(L + base, st, sD[id], 4, r);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        double z = 0.0;
+        for (int q = 0; q < 4; ++q) zeta[dd][q] = fx_to(-r[q], E[q] - 1079);
+      } else {
 #pragma unroll
-        for (int m = 0; m < n; ++m)
-          if (m != id) z -= sD[m][id] * L[q * nnn + base + m * st];
-        zeta[dd][q] = z;
+        for (int q = 0; q < 4; ++q) zeta[dd][q] = -adjv_sweep_general(L + q * nnn + base, st, id);
       }
       if (id == 0 || id == N) {  // the neighbour's viscous divergence reads this node's flux
         const int f = 2 * dd + (id == N ? 1 : 0);
@@ -377,9 +450,7 @@ __global__ void __launch_bounds__(LIFT_THREADS) k_adj_visc(const DgDevice d, con
       for (int c = 0; c < 3; ++c) Ja[dd][c] = d.Ja[(((size_t)e * 3 + dd) * 3 + c) * nnn + node];
     // the lifting forms tau and the heat flux from J grad w with 1/J in mu and kappa; their
     // transposes carry the same factors, and with them the 1/J of H below
-    const double iJ = d.invJ[(size_t)e * nnn + node];
     const double mu = d.mu * iJ, kappa = d.kappa * iJ;
-    const double u[3] = {W[node], W[nnn + node], W[2 * nnn + node]};
     const double *tr = tau + (size_t)e * 6 * nnn + node;
     const double txx = tr[0], tyy = tr[nnn], tzz = tr[2 * nnn], txy = tr[3 * nnn], txz = tr[4 * nnn],
                  tyz = tr[5 * nnn];
@@ -390,7 +461,7 @@ __global__ void __launch_bounds__(LIFT_THREADS) k_adj_visc(const DgDevice d, con
     for (int c = 0; c < 3; ++c)
 #pragma unroll
       for (int q = 0; q < 4; ++q) Z[c][q] = Ja[0][c] * zeta[0][q] + Ja[1][c] * zeta[1][q] + Ja[2][c] * zeta[2][q];
-    double Y[3][3], om[3];
+    double Y[3][3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       om[k] = Z[0][3] * ta[k][0] + Z[1][3] * ta[k][1] + Z[2][3] * ta[k][2];
@@ -398,59 +469,70 @@ __global__ void __launch_bounds__(LIFT_THREADS) k_adj_visc(const DgDevice d, con
       for (int c = 0; c < 3; ++c) Y[k][c] = Z[c][k] + Z[c][3] * u[k];
     }
     const double trY = Y[0][0] + Y[1][1] + Y[2][2];
+    // mu (Y + Y^T - 2/3 tr Y), symmetric
     double Gm[4][3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 3; ++k) {
+      Gm[k][k] = 2.0 * mu * (Y[k][k] - trY * (1.0 / 3.0));
 #pragma unroll
-      for (int c = 0; c < 3; ++c) Gm[k][c] = mu * (Y[k][c] + Y[c][k]) - (k == c ? 2.0 / 3.0 * mu * trY : 0.0);
+      for (int c = 0; c < k; ++c) Gm[k][c] = Gm[c][k] = mu * (Y[k][c] + Y[c][k]);
+    }
 #pragma unroll
     for (int c = 0; c < 3; ++c) Gm[3][c] = kappa * Z[c][3];
-    double *H = Hs + le * 12 * nnn + node;
-#pragma unroll
-    for (int dd = 0; dd < 3; ++dd)
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        H[(dd * 4 + q) * nnn] = Ja[dd][0] * Gm[q][0] + Ja[dd][1] * Gm[q][1] + Ja[dd][2] * Gm[q][2];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) Os[(le * 3 + k) * nnn + node] = om[k];
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < LIFT_EPB * nnn; t += blockDim.x) {
-    const int le = t / nnn, node = t % nnn, e = e0 + le;
-    if (e >= d.nE) continue;
-    const int ijk[3] = {node % n, (node / n) % n, node / nn};
-    const double *H = Hs + le * 12 * nnn;
-    double cw[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int dd = 0; dd < 3; ++dd) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) h[dd][q] = Ja[dd][0] * Gm[q][0] + Ja[dd][1] * Gm[q][1] + Ja[dd][2] * Gm[q][2];
       const int id = ijk[dd];
-      const int st = dd == 0 ? 1 : dd == 1 ? n : nn;
-      const int base = node - id * st;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        double s = 0.0;
-#pragma unroll
-        for (int m = 0; m < n; ++m) s += sD[m][id] * H[(dd * 4 + q) * nnn + base + m * st];
-        cw[q] += s;
-      }
       if (id == 0 || id == N) {
         const int f = 2 * dd + (id == N ? 1 : 0);
         const int pq = (dd == 0 ? ijk[1] : ijk[0]) + n * (dd == 2 ? ijk[1] : ijk[2]);
         const double hs = (id == N ? 0.5 : -0.5) * c_invw[id];
         double *sg = sigma + ((size_t)e * 6 + f) * 4 * nn + pq;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const double h = hs * H[(dd * 4 + q) * nnn + node];
-          cw[q] -= h;
-          sg[q * nn] = h;
-        }
+        for (int q = 0; q < 4; ++q) sg[q * nn] = hs * h[dd][q];
       }
     }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) cw[k] += Os[(le * 3 + k) * nnn + node];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) cotW[((size_t)e * 4 + q) * nnn + node] = cw[q];
   }
+  adjv_max<3>(h, on, s_mx[le][1]);
+  __syncthreads();
+  fx = adjv_scale(s_mx[le][1], E);
+  if (on) {
+#pragma unroll
+    for (int dd = 0; dd < 3; ++dd)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) H[(dd * 4 + q) * nnn + node] = adjv_store(h[dd][q], fx, E[q]);
+  }
+  __syncthreads();
+  if (!on) return;
+  double cw[4];
+  if (fx) {
+    fx_t c[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int dd = 0; dd < 3; ++dd) {
+      const int st = dd == 0 ? 1 : dd == 1 ? n : nn;
+      fx_t r[4];
+      adjv_sweep(H + dd * 4 * nnn + node - ijk[dd] * st, st, sD[ijk[dd]], 3, r);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) c[q] += r[q];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cw[q] = fx_to(c[q], E[q] - 1078);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      cw[q] = 0.0;
+#pragma unroll
+      for (int dd = 0; dd < 3; ++dd) {
+        const int st = dd == 0 ? 1 : dd == 1 ? n : nn;
+        cw[q] += adjv_sweep_general(H + (dd * 4 + q) * nnn + node - ijk[dd] * st, st, ijk[dd]);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) cw[k] += om[k];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) cotW[((size_t)e * 4 + q) * nnn + node] = cw[q];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -969,7 +1051,7 @@ void launch_adj_visc(const DgDevice &d, const double *U, const double *lam, cons
     cudaFuncSetAttribute(k_adj_visc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr_set = true;
   }
-  k_adj_visc<<<(d.nE + LIFT_EPB - 1) / LIFT_EPB, LIFT_THREADS, smem, s>>>(d, U, lam, tau, cotW, sigma);
+  k_adj_visc<<<(d.nE + LIFT_EPB - 1) / LIFT_EPB, ADJV_THREADS, smem, s>>>(d, U, lam, tau, cotW, sigma);
 }
 
 template <int VF>

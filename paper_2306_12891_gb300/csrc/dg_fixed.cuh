@@ -28,6 +28,7 @@ __constant__ int2 c_Qx[nn];                       // Q_im = w_i D_im, zero diago
 constexpr int FX_QV = n % 2 == 0 ? EO_H : n;
 __constant__ int2 c_QV[n * FX_QV];
 constexpr int FX_H = (n + 1) / 2;                 // distinct node weights
+__constant__ int2 c_DT[nn];                       // [i][m] = D_mi / 32, zero diagonal, 2^62 (the adjoint's sweeps)
 __constant__ int2 c_rho[FX_H * FX_H];             // min(w_a, w_b) / w_a, 2^62: [a][b], a, b = distance to the face
 
 __device__ __forceinline__ fx_t fx_mad(int a, int b, fx_t c) {
@@ -677,8 +678,9 @@ int2 fx_halves(long double v, int bits) {  // v 2^bits rounded to nearest, balan
 
 // fixed-point tables from the extended-precision Q = W D and weights (host)
 cudaError_t fx_upload(const DgTables &t) {
-  int2 Q[nn], QV[n * FX_QV], rho[FX_H * FX_H];
+  int2 Q[nn], DT[nn], QV[n * FX_QV], rho[FX_H * FX_H];
   for (int i = 0; i < nn; ++i) Q[i] = fx_halves(t.Q[i], 63);
+  for (int i = 0; i < nn; ++i) DT[i] = fx_halves(t.Q[i % n * n + i / n] / t.wl[i % n] / 32, 62);
   for (int i = 0; i < n; ++i)
     for (int m = 0; m < FX_QV; ++m) {
       long double v = t.Q[i * n + m];
@@ -697,6 +699,7 @@ cudaError_t fx_upload(const DgTables &t) {
     }
   }
   cudaError_t err = cudaMemcpyToSymbol(c_Qx, Q, sizeof(Q));
+  err = err ? err : cudaMemcpyToSymbol(c_DT, DT, sizeof(DT));
   err = err ? err : cudaMemcpyToSymbol(c_Ct, Ct, sizeof(Ct));
   err = err ? err : cudaMemcpyToSymbol(c_QV, QV, sizeof(QV));
   return err ? err : cudaMemcpyToSymbol(c_rho, rho, sizeof(rho));

@@ -120,3 +120,37 @@ def test_fixed_point_adjoint_volume_terms(env, kind, lam_scale, N, nel, vf):
         scl[v] = max(scl[v], (np.abs(col) * np.abs(lam)).sum())
     print(f"FIXED-POINT-ADJ {kind} {lam_scale} N={N} {vf}: {err / np.maximum(scl, 1e-300)}")
     assert (err <= 1e-12 * scl).all(), (err, scl)
+
+
+@pytest.mark.parametrize("N,nel", [(1, (5, 3, 3)), (2, (3, 3, 1)), (3, (3, 1, 1)), (4, (2, 1, 1)), (5, (2, 1, 1)), (6, (1, 1, 1)),
+                                   (7, (2, 1, 1))])
+def test_adjoint_viscous_fixed_point_against_its_fp64_path(env, N, nel):
+    """The vector-Jacobian product is linear in the cotangent: scaled by 2^900 or 2^-930 it takes the FP64 path, and must
+    agree with the fixed-point result (cotangents everywhere, of energy only, and at one node) scaled alike. Fewer than
+    200 roundings lie on the way to an entry, and the sum of its |terms| is below 20 times the largest entry of its
+    variable: 200 x 20 x 2^-53 < 1e-12. A NaN reaches two elements far (the neighbours' viscous flux, theirs by the lifting)."""
+    dg, orc, torch = env
+    xyz, faces = W.box_mesh(N, nel, mapping=_map)
+    U, _ = _state("mach_1", xyz, N)
+    gpu = dg.DG(N, xyz, faces, equations="ns", vflux="pirozzoli", sflux="roe", mu=0.02)
+    Ud = torch.from_numpy(U).cuda()
+    rnd = np.random.default_rng(N).standard_normal(U.shape)
+    energy = rnd * np.reshape([0, 0, 0, 0, 1.0], (1, 5, 1, 1, 1))
+    point = np.zeros_like(U)
+    point[-1, 1:, N, 0, N // 2] = [1.0, -0.5, 1e-3, 1e-6]
+    for lam in (rnd, energy, point):
+        got = gpu.rhs_vjp(Ud, torch.from_numpy(lam).cuda()).cpu().numpy()
+        scl = np.abs(got).max(axis=(0, 2, 3, 4)).reshape(1, 5, 1, 1, 1)
+        for k in (900, -930):
+            ref = gpu.rhs_vjp(Ud, torch.from_numpy(np.ldexp(lam, k)).cuda()).cpu().numpy()
+            err = np.abs(np.ldexp(ref, -k) - got) / scl
+            assert err.max() <= 1e-12, (k, err.max(axis=(0, 2, 3, 4)))
+    gpu.check()
+    if nel[0] >= 5:  # (periodic: elements (2, 1, 0) and (3, 1, 0) are three steps away from element 0; a block's
+        # elements take the FP64 path together in the volume kernel: the same bound, not the same bits)
+        lam = rnd.copy()
+        lam[0, 2, 0, 0, 0] = np.nan
+        bad = gpu.rhs_vjp(Ud, torch.from_numpy(lam).cuda()).cpu().numpy()
+        good = gpu.rhs_vjp(Ud, torch.from_numpy(rnd).cuda()).cpu().numpy()
+        scl = np.abs(good).max(axis=(0, 2, 3, 4)).reshape(1, 5, 1, 1, 1)
+        assert np.isnan(bad[0]).any() and (np.abs(bad[7:9] - good[7:9]) <= 1e-12 * scl).all()
