@@ -18,6 +18,12 @@
 // (BR1 central) flux the same cancellation leaves -(1/(2 w_b)) phi_nb, the neighbour's outward
 // normal viscous flux. Pair symmetry F#(U_i,U_m) = F#(U_m,U_i) halves the two-point fluxes.
 //
+// FP64 path: the volume operator (KG and Pirozzoli, with or without the blend), the lifting, the indicator and the
+// adjoint's volume and viscous kernels form their sums in 64-bit fixed point on the integer pipes (dg_fixed.cuh,
+// dg_fixed_lift.cuh, dg_adjoint.cuh): this GPU's FP64 pipe takes 2 lanes per clock and SM, a 32 x 32 + 64-bit integer
+// multiply-add 25, so a product in three of those costs a quarter of an FMA. k_volume below serves FP64 for the EC and
+// central fluxes.
+//
 // Arithmetic type R: double for the FP64 path; float for the FP32-bulk path, where the flux,
 // lifting and accumulation arithmetic is FP32 while U is read as FP64, metrics and Jacobian are
 // computed in FP64 (the kernels read an FP32 rounding of Ja), and the LSERK register and state
