@@ -545,16 +545,6 @@ struct AdjNode {
   double r, u, v, w, p, x, l[5], jx, jy, jz;
 };
 
-__device__ __forceinline__ AdjNode adj_node(const double *__restrict__ P, const double *__restrict__ Lm, int a,
-                                            const double *__restrict__ Jd, int g) {
-  AdjNode q;
-  q.r = P[a]; q.u = P[PS + a]; q.v = P[2 * PS + a]; q.w = P[3 * PS + a]; q.p = P[4 * PS + a]; q.x = P[5 * PS + a];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) q.l[k] = Lm[k * PS + a];
-  q.jx = __ldg(Jd + g); q.jy = __ldg(Jd + nnn + g); q.jz = __ldg(Jd + 2 * nnn + g);
-  return q;
-}
-
 // the six primitive cotangents of the pair (i, m), shared by both nodes. The pair cotangents
 // c_v = D'_im l_i,v + D'_mi l_m,v are D'_im t_v with t_v = l_i,v + (D_mi/D_im) l_m,v (the mass part's
 // factor 2, D/4 against D/8, is in the staged l_0); D'_im = D_im/8 then scales phi, the pressure
@@ -760,28 +750,40 @@ __device__ __forceinline__ void fx_adj_pair(const FxAdjNode &a, const FxAdjNode 
   g[5] = fx_value(s, c.ax);
 }
 
-// general path of one node in FP64, from the staged doubles: slots 0-5 as above, 6-10 l
+// general path: the pair phase in FP64 on the staged doubles (slots as in the fixed-point phase; 4 p, l unweighted). Whole
+// product with every element general, N = 7, 12^3, Euler: 1327 us, 1832 with a thread per node that formed all its pairs
+// itself, 1240 with the former FP64 line kernel; N = 5, Navier-Stokes: 805, 941 and 941 us.
 template <int VF>
-__device__ __noinline__ void fx_adj_general_node(const DgDevice &d, const double *S, size_t e, int node, double gp[6]) {
-  const int ijk[3] = {node % n, (node / n) % n, node / nn};
-  for (int v = 0; v < 6; ++v) gp[v] = 0.0;
-  for (int dd = 0; dd < 3; ++dd) {
-    const int id = ijk[dd], st = dd == 0 ? 1 : dd == 1 ? n : nn, ps = dd == 0 ? 1 : dd == 1 ? FX_SJ : FX_SK;
-    const double *Jd = d.Ja + (e * 3 + dd) * 3 * nnn;
+__device__ __noinline__ void fx_adj_general_lines(double *S) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int gr = threadIdx.x >> 5; gr < 3 * FX_GROUPS; gr += FX_THREADS / 32) {
+    const FxLine q = fx_line(gr, lane);
+    double *Sl = S + q.lel * FXA_SLOTS * FX_PS + q.pb;
     auto load = [&](int m) {
-      const double *P = S + fx_idx(node) + (m - id) * ps;
-      const int gn = node + (m - id) * st;
-      AdjNode q{P[0], P[FX_PS], P[2 * FX_PS], P[3 * FX_PS], 4.0 * P[4 * FX_PS], P[5 * FX_PS]};
-      for (int k = 0; k < 5; ++k) q.l[k] = P[(6 + k) * FX_PS];
-      q.jx = Jd[gn]; q.jy = Jd[nnn + gn]; q.jz = Jd[2 * nnn + gn];
-      return q;
+      const double *P = Sl + m * q.ps, *J = P + (6 + 8 * q.dir) * FX_PS;
+      AdjNode a{P[0], P[FX_PS], P[2 * FX_PS], P[3 * FX_PS], P[4 * FX_PS], P[5 * FX_PS]};
+#pragma unroll
+      for (int v = 0; v < 5; ++v) a.l[v] = J[(3 + v) * FX_PS];
+      a.jx = J[0]; a.jy = J[FX_PS]; a.jz = J[2 * FX_PS];
+      return a;
     };
-    const AdjNode a = load(id);
-    for (int m = 0; m < n; ++m) {
-      if (m == id) continue;
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int s = 1; s <= n / 2; ++s) {
+      const int m = q.idx + s < n ? q.idx + s : q.idx + s - n, j = q.idx >= s ? q.idx - s : q.idx - s + n;
       double g[6];
-      adj_pair<VF>(a, load(m), c_De[id * n + m], c_Dr[id * n + m], g);
-      for (int v = 0; v < 6; ++v) gp[v] += g[v];
+      adj_pair<VF>(load(q.idx), load(m), c_De[q.idx * n + m], c_Dr[q.idx * n + m], g);
+#pragma unroll
+      for (int v = 0; v < 6; ++v) {
+        acc[v] += g[v];
+        if (2 * s != n) acc[v] += __shfl_sync(0xffffffffu, g[v], q.l0 + j);
+      }
+    }
+    __syncwarp();
+    if (q.own) {
+#pragma unroll
+      for (int v = 0; v < 6; ++v) Sl[(6 + 8 * q.dir + v) * FX_PS + q.idx * q.ps] = acc[v];
     }
   }
 }
@@ -893,15 +895,10 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
       }
     }
     __syncthreads();
-    constexpr int GROUPS = (FX_EPB * nn + FX_LPW - 1) / FX_LPW;
-    const int lane = tid & 31, idx = lane % n, l0 = (lane / n) % FX_LPW * n;
-    for (int gr = tid >> 5; gr < 3 * GROUPS; gr += FX_THREADS / 32) {
-      const int dir = gr / GROUPS, g0 = (gr % GROUPS) * FX_LPW;
-      const bool own = lane < FX_LPW * n && g0 + lane / n < FX_EPB * nn;
-      const int ln = own ? g0 + lane / n : g0;  // lanes without a line of their own repeat the group's first one
-      const int lel = ln / nn, ll = ln % nn, la = ll % n, lb = ll / n;
-      const int ps = dir == 0 ? 1 : dir == 1 ? FX_SJ : FX_SK;
-      const int pb = dir == 0 ? FX_SJ * la + FX_SK * lb : dir == 1 ? la + FX_SK * lb : la + FX_SJ * lb;
+    const int lane = tid & 31;
+    for (int gr = tid >> 5; gr < 3 * FX_GROUPS; gr += FX_THREADS / 32) {
+      const FxLine q = fx_line(gr, lane);
+      const int dir = q.dir, idx = q.idx, l0 = q.l0, lel = q.lel, pb = q.pb, ps = q.ps;
       fx_t *Sl = S + lel * FXA_SLOTS * FX_PS;
       const FxAdjNode ni = fx_adj_load<VF>(Sl, pb + idx * ps, dir);
       fx_t acc[6] = {0, 0, 0, 0, 0, 0};
@@ -918,18 +915,28 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
         }
       }
       __syncwarp();
-      if (own) {
+      if (q.own) {
 #pragma unroll
         for (int v = 0; v < 6; ++v) Sl[(6 + 8 * dir + v) * FX_PS + pb + idx * ps] = acc[v];
       }
     }
   } else if (on) {
     double *Se = reinterpret_cast<double *>(S) + le * FXA_SLOTS * FX_PS + fx_idx(node);
-    Se[0] = r; Se[4 * FX_PS] = p; Se[5 * FX_PS] = X;
+    const double *Je = d.Ja + (size_t)e * 9 * nnn + node;
+    Se[0] = r; Se[4 * FX_PS] = 4.0 * p; Se[5 * FX_PS] = X;
 #pragma unroll
     for (int k = 0; k < 3; ++k) Se[(1 + k) * FX_PS] = u[k];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) Se[(6 + k) * FX_PS] = l[k];
+    for (int dd = 0; dd < 3; ++dd) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) Se[(6 + 8 * dd + k) * FX_PS] = __ldg(Je + (3 * dd + k) * nnn);
+#pragma unroll
+      for (int v = 0; v < 5; ++v) Se[(9 + 8 * dd + v) * FX_PS] = l[v];
+    }
+  }
+  if (!ok) {
+    __syncthreads();
+    fx_adj_general_lines<VF>(reinterpret_cast<double *>(S));
   }
   __syncthreads();
   if (!on) return;
@@ -944,10 +951,9 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
       gp[v] = w8 * fx_to(s3, v == 0 ? c.k0 : v < 4 ? c.k1 : v == 4 ? c.kp : c.kx);
     }
   } else {
-    double g[6];
-    fx_adj_general_node<VF>(d, reinterpret_cast<const double *>(S) + le * FXA_SLOTS * FX_PS, e, node, g);
+    const double *Se = reinterpret_cast<const double *>(S) + le * FXA_SLOTS * FX_PS + fx_idx(node);
 #pragma unroll
-    for (int v = 0; v < 6; ++v) gp[v] = g[v];
+    for (int v = 0; v < 6; ++v) gp[v] = Se[(6 + v) * FX_PS] + Se[(14 + v) * FX_PS] + Se[(22 + v) * FX_PS];
   }
   const bool ns = d.equations == 1;
   const double iR = 1.0 / d.R;

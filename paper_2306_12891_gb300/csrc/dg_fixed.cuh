@@ -14,7 +14,7 @@
 // so with the pair symmetry Q_im = -Q_mi of the SBP operator Q = W D a pair's two shares cancel exactly.
 // Precision: all rounding happens at about 2^-61 of the largest flux sum the element can have, where FP64
 // rounds each flux and each partial sum at 2^-53 of itself. An element takes the general FP64 path of the
-// same kernel (fx_general_node) instead when a value is not finite, rho, p or h (e) is not positive or
+// same kernel (fx_general_lines) instead when a value is not finite, rho, p or h (e) is not positive or
 // spans more than 2^8 within the element, or the exponents leave a safe range.
 #pragma once
 
@@ -243,36 +243,83 @@ __device__ __forceinline__ void fx_viscous(const double *__restrict__ Fn, const 
   }
 }
 
-// general path of one node in FP64: flux differencing and viscous divergence, from the staged quantities
-// rho, u, v, w, p, h|e (doubles, slots 0-5)
+// Elements per CTA: one; CTAs of one or two warps at the lowest degrees, so that small meshes spread over the SMs
+constexpr int FX_EPB = N == 1 ? 8 : N == 2 ? 2 : 1;
+constexpr int FX_THREADS = round32(FX_EPB * nnn);
+// the line of the lane's node in group gr of the pair phase (lanes without a line of their own repeat the group's
+// first one): direction, node on the line, lane of node 0, element of the block, node 0 and stride in the element's
+// arrays (gb, gs) and in the staged ones (pb, ps)
+constexpr int FX_GROUPS = (FX_EPB * nn + FX_LPW - 1) / FX_LPW;  // warps' worth of lines per direction
+struct FxLine {
+  bool own;
+  int dir, idx, l0, lel, gb, gs, pb, ps;
+};
+__device__ __forceinline__ FxLine fx_line(int gr, int lane) {
+  FxLine q;
+  q.dir = gr / FX_GROUPS;
+  const int g0 = (gr % FX_GROUPS) * FX_LPW, l = (lane / n) % FX_LPW;
+  q.idx = lane % n;
+  q.l0 = l * n;
+  q.own = lane < FX_LPW * n && g0 + l < FX_EPB * nn;
+  const int ln = q.own ? g0 + l : g0;
+  q.lel = ln / nn;
+  const int ll = ln % nn, la = ll % n, lb = ll / n;
+  q.gb = q.dir == 0 ? n * (la + n * lb) : q.dir == 1 ? la + nn * lb : la + n * lb;
+  q.gs = q.dir == 0 ? 1 : q.dir == 1 ? n : nn;
+  q.ps = q.dir == 0 ? 1 : q.dir == 1 ? FX_SJ : FX_SK;
+  q.pb = q.dir == 0 ? FX_SJ * la + FX_SK * lb : q.dir == 1 ? la + FX_SK * lb : la + FX_SJ * lb;
+  return q;
+}
+
+// general path: the pair phase in FP64 on the staged doubles (slots as in the fixed-point phase, 4 p), each pair formed once
+// and its flux handed to the partner by shuffles. Bound by the FP64 pipe. Right-hand side with every element general, N = 7,
+// 12^3, Euler: 754 us, 1159 with a thread per node that formed all its pairs itself, 734 with the former FP64 line
+// kernel (n / 2 of the n (n - 1) / 2 pairs of a line are formed twice here); N = 3, 21 x 18 x 15: 229, 330 and 224 us.
 template <int VF>
-__device__ __noinline__ void fx_general_node(const DgDevice &d, const double *S, size_t e, int node, double s[5]) {
-  const int ijk[3] = {node % n, (node / n) % n, node / nn};
-  const int a = fx_idx(node);
-  for (int v = 0; v < 5; ++v) s[v] = 0.0;
-  for (int dd = 0; dd < 3; ++dd) {
-    const int id = ijk[dd];
-    const int st = dd == 0 ? 1 : dd == 1 ? n : nn, pst = dd == 0 ? 1 : dd == 1 ? FX_SJ : FX_SK;
-    const double *Jd = d.Ja + (e * 3 + dd) * 3 * nnn + node;
-    for (int m = 0; m < n; ++m) {
-      if (m == id) continue;
-      const int b = a + (m - id) * pst, off = (m - id) * st;
-      const double Sj[3] = {Jd[0] + Jd[off], Jd[nnn] + Jd[nnn + off], Jd[2 * nnn] + Jd[2 * nnn + off]};
-      const double Su = S[FX_PS + a] + S[FX_PS + b], Sv = S[2 * FX_PS + a] + S[2 * FX_PS + b], Sw = S[3 * FX_PS + a] + S[3 * FX_PS + b];
-      const double Vp = Su * Sj[0] + Sv * Sj[1] + Sw * Sj[2];
-      const double Sp = S[4 * FX_PS + a] + S[4 * FX_PS + b], F0 = (S[a] + S[b]) * Vp;
-      double F4 = F0 * (S[5 * FX_PS + a] + S[5 * FX_PS + b]);
-      if (VF == VF_KG) F4 += 2.0 * Sp * Vp;
-      const double c = c_De[id * n + m];
-      s[0] += c_Dq[id * n + m] * F0;
-      s[1] += c * (F0 * Su + 4.0 * Sp * Sj[0]);
-      s[2] += c * (F0 * Sv + 4.0 * Sp * Sj[1]);
-      s[3] += c * (F0 * Sw + 4.0 * Sp * Sj[2]);
-      s[4] += c * F4;
-      if (d.equations == 1) {
-        const double *Fv = d.Fv + (e * 12 + dd * 4) * nnn + node + off;
-        for (int q = 0; q < 4; ++q) s[1 + q] -= c_D[id * n + m] * Fv[q * nnn];
+__device__ __noinline__ void fx_general_lines(const DgDevice &d, double *S, int e0) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int gr = threadIdx.x >> 5; gr < 3 * FX_GROUPS; gr += FX_THREADS / 32) {
+    const FxLine q = fx_line(gr, lane);
+    double *Se = S + q.lel * FX_SLOTS * FX_PS, *Pi = Se + q.pb + q.idx * q.ps;
+    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    if (d.equations == 1) {
+      const double *Fn = d.Fv + ((size_t)min(e0 + q.lel, d.nE - 1) * 12 + q.dir * 4) * nnn + q.gb + q.idx * q.gs;
+      double f[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) f[v] = 8.0 * Fn[v * nnn];
+#pragma unroll 1
+      for (int m = 0; m < n; ++m) {
+        const double c = c_De[q.idx * n + m];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[1 + v] -= c * __shfl_sync(0xffffffffu, f[v], q.l0 + m);
       }
+    }
+#pragma unroll 1
+    for (int s = 1; s <= n / 2; ++s) {
+      const int m = q.idx + s < n ? q.idx + s : q.idx + s - n, j = q.idx >= s ? q.idx - s : q.idx - s + n;
+      const double *Pm = Se + q.pb + m * q.ps, *Ji = Pi + (6 + 3 * q.dir) * FX_PS, *Jm = Pm + (6 + 3 * q.dir) * FX_PS;
+      const double Sj[3] = {Ji[0] + Jm[0], Ji[FX_PS] + Jm[FX_PS], Ji[2 * FX_PS] + Jm[2 * FX_PS]};
+      const double Su[3] = {Pi[FX_PS] + Pm[FX_PS], Pi[2 * FX_PS] + Pm[2 * FX_PS], Pi[3 * FX_PS] + Pm[3 * FX_PS]};
+      const double Vp = Su[0] * Sj[0] + Su[1] * Sj[1] + Su[2] * Sj[2], Sp = Pi[4 * FX_PS] + Pm[4 * FX_PS];
+      double F[5];
+      F[0] = (Pi[0] + Pm[0]) * Vp;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) F[1 + k] = F[0] * Su[k] + Sp * Sj[k];
+      F[4] = F[0] * (Pi[5 * FX_PS] + Pm[5 * FX_PS]);
+      if (VF == VF_KG) F[4] += 0.5 * Sp * Vp;
+      const double ci = c_De[q.idx * n + m], cj = c_De[q.idx * n + j];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) {
+        acc[v] += ci * F[v];
+        if (2 * s != n) acc[v] += cj * __shfl_sync(0xffffffffu, F[v], q.l0 + j);
+      }
+    }
+    acc[0] *= 2.0;  // (the mass flux's factor is D / 4)
+    __syncwarp();
+    if (q.own) {
+#pragma unroll
+      for (int v = 0; v < 5; ++v) Pi[fx_slot(q.dir, v) * FX_PS] = acc[v];
     }
   }
 }
@@ -358,9 +405,6 @@ __device__ __noinline__ void fv_interface(const DgDevice &d, const double *__res
 // (32 warps) per SM at N = 7. A thread per line (half the pair evaluations' overhead, sums in 80 registers,
 // 168 in all) held 12 warps and measured 2.43 ms per launch at N = 7, 24^3, Navier-Stokes, Pirozzoli; this form
 // 1.74 ms, the FP64 line kernel before it 6.21 ms (N = 5, 24 x 12 x 12 channel: 0.197 against 0.586 ms).
-// Elements per CTA: one; CTAs of one or two warps at the lowest degrees, so that small meshes spread over the SMs
-constexpr int FX_EPB = N == 1 ? 8 : N == 2 ? 2 : 1;
-constexpr int FX_THREADS = round32(FX_EPB * nnn);
 constexpr size_t FX_SMEM = sizeof(fx_t) * FX_EPB * FX_SLOTS * FX_PS;
 constexpr int FX_MINB = 1024 / FX_THREADS < 32 ? 1024 / FX_THREADS : 32;  // 64 registers per thread
 
@@ -448,10 +492,9 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
     __syncthreads();
     // phase B: one lane per node of a line. Lane i forms the pairs (i, i + s mod n), s <= (n - 1) / 2, adds its
     // share and hands the partner's on by a shuffle; at s = n / 2 (n even) both nodes form the pair.
-    constexpr int GROUPS = (FX_EPB * nn + FX_LPW - 1) / FX_LPW;  // warps' worth of lines per direction
     const int lane = tid & 31;
-    for (int gr = tid >> 5; gr < 3 * GROUPS; gr += FX_THREADS / 32) {
-      const int dir = gr / GROUPS, g0 = (gr % GROUPS) * FX_LPW;
+    for (int gr = tid >> 5; gr < 3 * FX_GROUPS; gr += FX_THREADS / 32) {
+      const int dir = gr / FX_GROUPS, g0 = (gr % FX_GROUPS) * FX_LPW;
       const int idx = lane % n, l = (lane / n) % FX_LPW, l0 = l * n;
       // lanes without a line of their own repeat the group's first one
       const bool own = lane < FX_LPW * n && g0 + l < FX_EPB * nn;
@@ -494,7 +537,13 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
   } else if (on) {
     double *Se = reinterpret_cast<double *>(S) + le * FX_SLOTS * FX_PS + fx_idx(node);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) Se[k * FX_PS] = q[k];
+    for (int k = 0; k < 6; ++k) Se[k * FX_PS] = k == 4 ? 4.0 * q[k] : q[k];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) Se[(6 + k) * FX_PS] = J[k];
+  }
+  if (!ok) {
+    __syncthreads();
+    fx_general_lines<VF>(d, reinterpret_cast<double *>(S), e0);
   }
   __syncthreads();
   let_next_start();
@@ -522,10 +571,9 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
         s[v] = (double)sum * __hiloint2double(iwh + (int)((unsigned)(v == 0 ? k0 : v < 4 ? km : ke) << 20), iwl);
       }
     } else {
-      double sg[5];
-      fx_general_node<VF>(d, reinterpret_cast<const double *>(S) + le * FX_SLOTS * FX_PS, e, node, sg);
+      const double *Se = reinterpret_cast<const double *>(S) + le * FX_SLOTS * FX_PS + fx_idx(node);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) s[v] = sg[v];
+      for (int v = 0; v < 5; ++v) s[v] = Se[fx_slot(0, v) * FX_PS] + Se[fx_slot(1, v) * FX_PS] + Se[fx_slot(2, v) * FX_PS];
     }
 #pragma unroll
     for (int dd = 0; dd < 3; ++dd) {
