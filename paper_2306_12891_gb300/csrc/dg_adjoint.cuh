@@ -588,13 +588,14 @@ __device__ __forceinline__ void adj_pair(const AdjNode &a, const AdjNode &b, dou
 // ---------------------------------------------------------------------------------------------
 struct FxAdj {
   int ok;
-  int er, eu, ep, ex, ej, e0, e1, e4;  // exponents: rho, u, p, X, Ja, l of mass, momentum, energy
+  int er, eu, ep, ex, e0, e1, e4;      // exponents: rho, u, p, X, l of mass, momentum, energy
+  int e[3], top;                       // of the metric terms' directions, as FxScale
   int av, aa, ab, af, ag, a0, ak, ax;  // windows of V, t_k S_u,k, t_4 S_X, F0, phi S_rho and the outputs
   int pa, pb, p0;                      // right shifts of t_k S_u,k, t_4 S_X and t_0 to phi's scale
   int va, vb;                          // KG: right shifts of phi S_rho and t_4 S_p to gV's
   int kf, kv;                          // right shifts of F0 and gV before t_k F0 + gV S_J,k
   int ga, gb;                          // right shifts of t_k S_J,k and (KG) t_4 V to the output's scale
-  int k0, k1, kp, kx;                  // cotangents are fixed value x 2^k / (8 w_0): rho, u, 4p, X
+  int k0, k1, kp, kx;                  // cotangents are fixed value x 2^(k + e_d) / (8 w_0): rho, u, 4p, X
 };
 
 // upper bound of log2(2^a + 2^b) in 2^-20
@@ -607,24 +608,29 @@ __device__ __forceinline__ int fx_lsum(int a, int b) {
 // most 62.2 and a line's sum of each output at most 62.2, by windows and shifts from the element's maxima; the
 // halved sum of three directions then stays below 63, and every group of cross sums h l' + l h' too.
 template <int VF>
-__device__ __forceinline__ FxAdj fx_adj_scales(const int *mx, int2 mj) {
+__device__ __forceinline__ FxAdj fx_adj_scales(const int *mx, int4 mj) {
   // mx: high words: rho max, rho min, |u| max, p max, p min, x max, x min (minima signed), |l| of mass, momentum, energy,
   // |u| + |v| + |w| max
   FxAdj s;
-  s.er = fx_exponent(mx[0]); s.ep = fx_exponent(mx[3]); s.ex = fx_exponent(mx[5]); s.ej = fx_exponent(mj.x);
+  s.er = fx_exponent(mx[0]); s.ep = fx_exponent(mx[3]); s.ex = fx_exponent(mx[5]);
+  const int j0 = fx_exponent(mj.x), j1 = fx_exponent(mj.y), j2 = fx_exponent(mj.z);
+  s.e[0] = fx_unit(mj.x); s.e[1] = fx_unit(mj.y); s.e[2] = fx_unit(mj.z);
+  const int jt = max(s.e[0], max(s.e[1], s.e[2])), jb = min(s.e[0], min(s.e[1], s.e[2]));
+  s.top = jt - jb <= FX_NEAR ? jt : -1000;
+  constexpr int ej = 1023;
   s.eu = max(fx_exponent(mx[2]), (1996 - s.er + s.ep) >> 1);
   // exponents of l: a group far below the others' shares of phi takes a scale 2^-40 of theirs
   const int r0 = fx_exponent(mx[7]), r1 = fx_exponent(mx[8]), r4 = fx_exponent(mx[9]);
   const int ph = max(r0, max(r1 + s.eu, r4 + s.ex) - 1023);
   s.e0 = max(r0, ph - 40); s.e1 = max(r1, ph - s.eu + 1023 - 40); s.e4 = max(r4, ph - s.ex + 1023 - 40);
-  const int lo = min(min(min(s.er, s.ep), min(s.ex, s.ej)), min(min(s.e0, s.e1), s.e4));
-  const int hi = max(max(max(s.er, s.ep), max(s.ex, s.ej)), max(max(max(s.e0, s.e1), s.e4), s.eu));
-  const int sr = 1084 - s.er, su = 1082 - s.eu, sp = 1084 - s.ep, sx = 1082 - s.ex, sj = 1082 - s.ej;
+  const int lo = min(min(min(s.er, s.ep), min(s.ex, min(j0, min(j1, j2)))), min(min(s.e0, s.e1), s.e4));
+  const int hi = max(max(max(s.er, s.ep), max(s.ex, max(j0, max(j1, j2)))), max(max(max(s.e0, s.e1), s.e4), s.eu));
+  const int sr = 1084 - s.er, su = 1082 - s.eu, sp = 1084 - s.ep, sx = 1082 - s.ex, sj = 1082 - ej;
   const int l0 = 1082 - s.e0, l1 = 1082 - s.e1, l4 = 1082 - s.e4;
   // log2 bounds in 2^-20: of sums S and differences of l (twice the maxima), then of the products
   constexpr int L = 1 << 20, LIM = (int)(62.2 * L);
   const int lr = fx_lg(mx[0]) + L, lu = max(fx_lg(mx[2]), (s.eu - 1023) << 20) + L, lp = fx_lg(mx[3]) + L,
-            lx = fx_lg(mx[5]) + L, lj = fx_lg(mj.x) + L, lv = lu + fx_lg(mj.y) + L;
+            lx = fx_lg(mx[5]) + L, lj = 2 * L, lv = lu + mj.w + L;  // (|Ja^d| < 2 in its units)
   const int t0 = max(fx_lg(mx[7]), (s.e0 - 1023) << 20) + L, t1 = max(fx_lg(mx[8]), (s.e1 - 1023) << 20) + L,
             t4 = max(fx_lg(mx[9]), (s.e4 - 1023) << 20) + L;
   const int la = t1 + max(fx_lg(mx[10]), (s.eu - 1023) << 20) + L, lb = t4 + lx, lf = lr + lv,
@@ -656,7 +662,7 @@ __device__ __forceinline__ FxAdj fx_adj_scales(const int *mx, int2 mj) {
   s.a0 = window(lphi + lv + FX_LGR, c0);
   s.ax = window(t4 + lf + FX_LGR, cx);
   const int pA = l1 + sj - 61, pB = l4 + sv - 62 + 1;  // t_k S_J,k with window 3; t_4 V with window 2, the factor 1/2
-  int lP = t1 + fx_lg(mj.y) + L + FX_LGR, sP = pA;
+  int lP = t1 + mj.w + L + FX_LGR, sP = pA;
   if (VF == VF_KG) {
     lP = fx_lsum(lP, t4 + lv - L + FX_LGR);
     sP = min(sP, pB);
@@ -667,7 +673,7 @@ __device__ __forceinline__ FxAdj fx_adj_scales(const int *mx, int2 mj) {
   s.k0 = 1 - (c0 + s.a0); s.k1 = 1 - (sk + s.ak); s.kp = 1 - sP; s.kx = 1 - (cx + s.ax);  // (halved sums)
   const int km = max(max(abs(s.k0), abs(s.k1)), max(abs(s.kp), abs(s.kx)));
   s.ok = mx[1] > 0 && mx[4] > 0 && mx[6] > 0 && s.er - (mx[1] >> 20) <= 8 && s.ep - (mx[4] >> 20) <= 8 &&
-         s.ex - (mx[6] >> 20) <= 8 && lo >= 850 && hi <= 1200 && km <= 900;
+         s.ex - (mx[6] >> 20) <= 8 && lo >= 850 && hi <= 1200 && km <= 700 && mj.w < FX_FAR;
   return s;
 }
 
@@ -879,7 +885,7 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
       Se[5 * FX_PS] = fx_from(X, c.ex, 3) + HB;
       const double *Je = d.Ja + (size_t)e * 9 * nnn + node;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) Se[(6 + 8 * (k / 3) + k % 3) * FX_PS] = fx_from(__ldg(Je + k * nnn), c.ej, 3) + HB;
+      for (int k = 0; k < 9; ++k) Se[(6 + 8 * (k / 3) + k % 3) * FX_PS] = fx_from(__ldg(Je + k * nnn), 1023 + c.e[k / 3], 3) + HB;
       FxD lf[5];
 #pragma unroll
       for (int v = 0; v < 5; ++v) lf[v] = fx_split(fx_from(l[v], v == 0 ? c.e0 : v < 4 ? c.e1 : c.e4, 3));
@@ -947,8 +953,12 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
     const double w8 = 0.125 * c_invw[0];
 #pragma unroll
     for (int v = 0; v < 6; ++v) {
-      const fx_t s3 = (Se[(6 + v) * FX_PS] >> 1) + (Se[(14 + v) * FX_PS] >> 1) + (Se[(22 + v) * FX_PS] >> 1);
-      gp[v] = w8 * fx_to(s3, v == 0 ? c.k0 : v < 4 ? c.k1 : v == 4 ? c.kp : c.kx);
+      const int k = v == 0 ? c.k0 : v < 4 ? c.k1 : v == 4 ? c.kp : c.kx;
+      const fx_t a = Se[(6 + v) * FX_PS], b = Se[(14 + v) * FX_PS], z = Se[(22 + v) * FX_PS];
+      if (c.top != -1000)
+        gp[v] = w8 * fx_to((a >> (1 + c.top - c.e[0])) + (b >> (1 + c.top - c.e[1])) + (z >> (1 + c.top - c.e[2])), k + c.top);
+      else
+        gp[v] = w8 * (fx_to(a, k - 1 + c.e[0]) + fx_to(b, k - 1 + c.e[1]) + fx_to(z, k - 1 + c.e[2]));
     }
   } else {
     const double *Se = reinterpret_cast<const double *>(S) + le * FXA_SLOTS * FX_PS + fx_idx(node);

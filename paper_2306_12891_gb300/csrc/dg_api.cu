@@ -539,11 +539,15 @@ dg_status dg_init(const dg_mesh *mesh, int N, int nodes, const dg_params *prm, v
       DG_ALLOC(d.Fwall, (size_t)nF * 4 * nn);
     }
   }
-  DG_ALLOC(d.alpha_raw, (size_t)nE * 5);  // one allocation for the arrays with 8 bytes per element
-  d.alpha = d.alpha_raw + nE;
-  d.ijmax = d.alpha_raw + 2 * (size_t)nE;
-  d.jmax = reinterpret_cast<int2 *>(d.alpha_raw + 3 * (size_t)nE);
-  d.fvmax = reinterpret_cast<int *>(d.alpha_raw + 4 * (size_t)nE);
+  {  // one allocation for the arrays with 8 or 16 bytes per element
+    double *small;
+    DG_ALLOC(small, (size_t)nE * 6);
+    d.jmax = reinterpret_cast<int4 *>(small);
+    d.fvmax = reinterpret_cast<int *>(small + 2 * (size_t)nE);
+    d.ijmax = small + 3 * (size_t)nE;
+    d.alpha = small + 4 * (size_t)nE;
+    d.alpha_raw = small + 5 * (size_t)nE;
+  }
   DG_ALLOC(d.red, (size_t)DG_RED_DOUBLES);
   DG_ALLOC(d.flag, (size_t)1);
   DG_ALLOC(c->g, c->n_state);

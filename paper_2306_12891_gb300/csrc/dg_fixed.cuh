@@ -5,8 +5,8 @@
 // at 55 (measured). A pair flux is 30 FP64 instructions (~16 clocks per lane and SM); in fixed point it is
 // 13 products of three IMAD.WIDE each and ~40 adds and shifts (~2 clocks).
 //
-// Format: per element every quantity is scaled by a power of two taken from the element's largest value of
-// it, X = x 2^s with |X| < 2^62 (rho, p) or 2^60 (the rest): an FP64 significand has 53 bits, so an input
+// Format: per element every quantity (the metric terms: per direction) is scaled by a power of two taken from the
+// element's largest value of it, X = x 2^s with |X| < 2^62 (rho, p) or 2^60 (the rest): an FP64 significand has 53 bits, so an input
 // is exact down to 2^-7 of the element's maximum. A product keeps the high 64 of 128 bits: with X = 2^32 h +
 // l, h and l signed 32-bit halves, it is h h' + (h l' + l h') / 2^32; the dropped l l' is below a quarter
 // unit. Every product is rounded to nearest in a window chosen per element (FxScale), so that the largest
@@ -15,7 +15,8 @@
 // Precision: all rounding happens at about 2^-61 of the largest flux sum the element can have, where FP64
 // rounds each flux and each partial sum at 2^-53 of itself. An element takes the general FP64 path of the
 // same kernel (fx_general_lines) instead when a value is not finite, rho, p or h (e) is not positive or
-// spans more than 2^8 within the element, or the exponents leave a safe range.
+// spans more than 2^8 within the element, the element is stretched by more than 8 (FX_JSPAN), or the exponents leave a safe
+// range.
 #pragma once
 
 namespace {
@@ -84,16 +85,38 @@ __device__ __forceinline__ fx_t fx_from(double x, int E, int drop) {
 __device__ __forceinline__ int fx_exponent(int hi) { return (hi + 0x10) >> 20; }
 __device__ __forceinline__ int fx_hi_abs(double x) { return __double2hiint(x) & 0x7fffffff; }
 
+// Metric terms: each direction d has its own scale 2^-e_d, e_d the exponent of its largest |Ja^d_c| in the element (jmax).
+// All products of a direction's lines carry Ja^d once, so the windows below are those of metric terms below 2, and a
+// direction's sums come out in units of 2^e_d. Even so the wide directions' sums are rounded in windows made for the thin
+// one's pressure and velocity: the error of the right-hand side against that of FP64 (rms per variable, shear layers across
+// the thin direction, N = 3, 5, 7) is 0.59 to 0.68 on cubes, 0.64 to 0.85 at aspect ratio 8, 0.64 to 1.13 at 16 and up to 4
+// at 64 (one scale for all directions: 1.4 at 16, 4 at 64, 37 at 1024). Elements whose metric terms span more than FX_JSPAN
+// take the general path.
+constexpr int FX_JSPAN = 3;         // largest span of max_c |Ja^d_c| over the element's nodes and directions, log2
+constexpr int FX_FAR = 1 << 28;     // jmax.w of an element beyond it
+constexpr int FX_NEAR = 2;          // directions' exponents this close: sums added as integers
+__device__ __forceinline__ int fx_unit(int h) {  // e_d
+  return max(-340, min(340, fx_exponent(h) - 1023));
+}
+
+// |f| of direction d against 2^e_d, as a high word (unit: e_d 2^20); what is not finite, or beyond 2^477, counts as such
+__device__ __forceinline__ int fx_relative(double f, int unit) {
+  const int h = fx_hi_abs(f);
+  return h < (1500 << 20) ? h - unit : 0x7ff00000;
+}
+
 // per-element scales, from the maxima (high words) of the staged quantities, the metric terms and the
 // viscous flux
 struct FxScale {
   int ok;
-  int er, eu, ep, ex, ej;  // exponents E of rho, velocity, p, h (or e), metric terms
+  int er, eu, ep, ex;      // exponents E of rho, velocity, p, h (or e)
+  int e[3];                // e_d; Ja^d is taken with the exponent 1023 + e_d
+  int top;                 // largest e_d, or -1000 where they differ by more than FX_NEAR
   int dp, dx;              // extra bits dropped from p and h (e)
   int av, ag;              // windows of V and G
   int kg, kv;              // right shifts of G before the momentum product, of V before p V (KG)
-  int vm, ve;              // fx_from exponents of the viscous flux (momentum, energy)
-  int k0, km, ke;          // results are fixed value x 2^k x (1/w)
+  int vm, ve;              // fx_from exponents of the viscous flux (momentum, energy), e_d to be added
+  int k0, km, ke;          // results are fixed value x 2^(k + e_d) x (1/w)
 };
 constexpr int FX_AM = 3;  // window of the momentum and energy products
 
@@ -110,24 +133,28 @@ constexpr int FX_RB = N == 1 ? 0 : N <= 3 ? 1 : 2;
 // halved sum of three directions then stays below 62.9, and the cross sums h l' + l h' of every product
 // group below 63.
 template <int VF>
-__device__ __forceinline__ FxScale fx_scales(const int *mx, int2 mj, int mvm, int mve, bool ns) {
-  // mx: high words: rho max, rho min, |u| max, p max, p min, x max, x min (minima signed); mj: of the
-  // largest |Ja^d_c| and the largest sum_c |Ja^d_c|
+__device__ __forceinline__ FxScale fx_scales(const int *mx, int4 mj, int mvm, int mve, bool ns) {
+  // mx: high words: rho max, rho min, |u| max, p max, p min, x max, x min (minima signed); mj: jmax; mvm, mve: fvmax
   FxScale s;
-  s.er = fx_exponent(mx[0]); s.ep = fx_exponent(mx[3]); s.ex = fx_exponent(mx[5]); s.ej = fx_exponent(mj.x);
+  const int j0 = fx_exponent(mj.x), j1 = fx_exponent(mj.y), j2 = fx_exponent(mj.z);
+  s.e[0] = fx_unit(mj.x); s.e[1] = fx_unit(mj.y); s.e[2] = fx_unit(mj.z);
+  const int jt = max(s.e[0], max(s.e[1], s.e[2])), jb = min(s.e[0], min(s.e[1], s.e[2]));
+  s.top = jt - jb <= FX_NEAR ? jt : -1000;
+  s.er = fx_exponent(mx[0]); s.ep = fx_exponent(mx[3]); s.ex = fx_exponent(mx[5]);
+  constexpr int ej = 1023;
   s.eu = max(fx_exponent(mx[2]), (1996 - s.er + s.ep) >> 1);  // floor 2^-26 sqrt(p / rho): kg stays within 62
-  const int lo = min(min(s.er, s.ep), min(s.ex, min(s.ej, s.eu)));
-  const int hi = max(max(s.er, s.ep), max(s.ex, max(s.ej, s.eu)));
-  const int lr = fx_lg(mx[0]), lu = max(fx_lg(mx[2]), (s.eu - 1023) << 20), lp = fx_lg(mx[3]), lx = fx_lg(mx[5]), lj = fx_lg(mj.y);
+  const int lo = min(min(s.er, s.ep), min(min(s.ex, s.eu), min(j0, min(j1, j2))));
+  const int hi = max(max(s.er, s.ep), max(max(s.ex, s.eu), max(j0, max(j1, j2))));
+  const int lr = fx_lg(mx[0]), lu = max(fx_lg(mx[2]), (s.eu - 1023) << 20), lp = fx_lg(mx[3]), lx = fx_lg(mx[5]), lj = mj.w;
   const int lv = lu + lj;                                      // log2 of the V bound
   constexpr int L = 1 << 20, LIM = (int)(61.7 * L);
   // scales: fixed = value 2^s
-  const int st = 1084 - s.er, sv0 = 2102 - s.eu - s.ej;
+  const int st = 1084 - s.er, sv0 = 2102 - s.eu - ej;
   s.av = min((((int)(62.9 * L) - lv) >> 20) - sv0, 6);
   const int sv = sv0 + s.av;
   s.ag = min((((int)(62.3 * L) - lr - lv) >> 20) - (st + sv - 64), 4);
   const int sg = st + sv - 64 + s.ag;
-  const int xa = sg + 1022 - s.eu, xp = 2106 - s.ep - s.ej;    // momentum from G u, from p Ja
+  const int xa = sg + 1022 - s.eu, xp = 2106 - s.ep - ej;    // momentum from G u, from p Ja
   int xm = min(min(xa, xp), (LIM - (FX_LGR + L + max(lr + lv + lu, lp + lj))) >> 20);
   const int evm = fx_exponent(mvm), eve = fx_exponent(mve);
   if (ns) xm = min(xm, 1081 - evm);
@@ -136,7 +163,7 @@ __device__ __forceinline__ FxScale fx_scales(const int *mx, int2 mj, int mvm, in
   const int xe0 = sg + 1022 - s.ex;                            // energy from G h (G e)
   int be = lr + lv + lx, xe = xe0, xq = 0;
   if (VF == VF_KG) {  // and from (Q S_p) V
-    xq = 3123 - s.dp - s.ep - s.eu - s.ej + s.av;
+    xq = 3123 - s.dp - s.ep - s.eu - ej + s.av;
     xe = min(xe, xq);
     be = max(be, lp + lv) + L;
   }
@@ -149,8 +176,8 @@ __device__ __forceinline__ FxScale fx_scales(const int *mx, int2 mj, int mvm, in
   s.k0 = 2 - (sg - FX_RB); s.km = 2 - xm; s.ke = 2 - xe;  // 2 D F, and the halved sum of directions
   const int kmax = max(max(abs(s.k0), abs(s.km)), abs(s.ke));
   s.ok = mx[1] > 0 && mx[4] > 0 && mx[6] > 0 && s.er - (mx[1] >> 20) <= 8 && s.ep - (mx[4] >> 20) <= 8 &&
-         s.ex - (mx[6] >> 20) <= 8 && lo >= 700 && hi <= 1350 && kmax <= 900 && s.av >= 0 && s.ag >= 0 &&
-         s.kg >= 0 && s.kg <= 62 && s.dp >= 0 && s.dx >= 0 && s.kv <= 62 && (!ns || (evm < 2000 && eve < 2000));
+         s.ex - (mx[6] >> 20) <= 8 && lo >= 700 && hi <= 1350 && kmax <= 560 && mj.w < FX_FAR && s.av >= 0 && s.ag >= 0 &&
+         s.kg >= 0 && s.kg <= 62 && s.dp >= 0 && s.dx >= 0 && s.kv <= 62 && (!ns || (evm < 1500 && eve < 1500));
   return s;
 }
 
@@ -296,7 +323,7 @@ __device__ __noinline__ void fx_general_lines(const DgDevice &d, double *S, int 
       }
     }
 #pragma unroll 1
-    for (int s = 1; s <= n / 2; ++s) {
+    for (int s = n / 2; s > 0; --s) {  // the smaller factors first
       const int m = q.idx + s < n ? q.idx + s : q.idx + s - n, j = q.idx >= s ? q.idx - s : q.idx - s + n;
       const double *Pm = Se + q.pb + m * q.ps, *Ji = Pi + (6 + 3 * q.dir) * FX_PS, *Jm = Pm + (6 + 3 * q.dir) * FX_PS;
       const double Sj[3] = {Ji[0] + Jm[0], Ji[FX_PS] + Jm[FX_PS], Ji[2 * FX_PS] + Jm[2 * FX_PS]};
@@ -487,7 +514,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
       Se[4 * FX_PS] = fx_from(q[4], c.ep, 1 + c.dp) + HB;
       Se[5 * FX_PS] = fx_from(q[5], c.ex, 3 + c.dx) + HB;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) Se[(6 + k) * FX_PS] = fx_from(J[k], c.ej, 3) + HB;
+      for (int k = 0; k < 9; ++k) Se[(6 + k) * FX_PS] = fx_from(J[k], 1023 + c.e[k / 3], 3) + HB;
     }
     __syncthreads();
     // phase B: one lane per node of a line. Lane i forms the pairs (i, i + s mod n), s <= (n - 1) / 2, adds its
@@ -510,7 +537,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
       fx_t acc[5] = {0, 0, 0, 0, 0};
       if (ns) {
         const size_t el = min(e0 + lel, d.nE - 1);
-        fx_viscous(d.Fv + (el * 12 + dir * 4) * nnn + gb + idx * gs, s_QV, idx, l0, c.vm, c.ve, acc);
+        fx_viscous(d.Fv + (el * 12 + dir * 4) * nnn + gb + idx * gs, s_QV, idx, l0, c.vm + c.e[dir], c.ve + c.e[dir], acc);
       }
       const int av = c.av, ag = c.ag, kg = c.kg, kv = c.kv;
       const FxNode ni = fx_load(Se, ai, dir);
@@ -559,16 +586,32 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
                 r2 = fx_const(s_rho[a2 * FX_H + am]);
       const double iw = c_invw[am];
       const int iwh = __double2hiint(iw), iwl = __double2loint(iw);
-      const int k0 = s_sc[le].k0, km = s_sc[le].km, ke = s_sc[le].ke;
+      const FxScale &c = s_sc[le];
+      const int k0 = c.k0, km = c.km, ke = c.ke, e0 = c.e[0], e1 = c.e[1], e2 = c.e[2], top = c.top;
+      if (top != -1000) {
+        auto scaled = [](FxD r, int h) { return fx_split((((fx_t)r.h << 32) + r.l) >> h); };
+        const FxD q0 = scaled(r0, top - e0), q1 = scaled(r1, top - e1), q2 = scaled(r2, top - e2);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) {
-        FxSum f0{0, 0x40000000ll}, f1 = f0, f2 = f0;  // the three lo sums do not fit one
-        fx_acc(f0, r0, fx_split(Se[fx_slot(0, v) * FX_PS]));
-        fx_acc(f1, r1, fx_split(Se[fx_slot(1, v) * FX_PS]));
-        fx_acc(f2, r2, fx_split(Se[fx_slot(2, v) * FX_PS]));
-        // half the sum of the three directions (the factors carry 2^62)
-        const fx_t sum = ((f0.hi + f1.hi + f2.hi) << 1) + (f0.lo >> 31) + (f1.lo >> 31) + (f2.lo >> 31);
-        s[v] = (double)sum * __hiloint2double(iwh + (int)((unsigned)(v == 0 ? k0 : v < 4 ? km : ke) << 20), iwl);
+        for (int v = 0; v < 5; ++v) {
+          FxSum f0{0, 0x40000000ll}, f1 = f0, f2 = f0;  // the three lo sums do not fit one
+          fx_acc(f0, q0, fx_split(Se[fx_slot(0, v) * FX_PS]));
+          fx_acc(f1, q1, fx_split(Se[fx_slot(1, v) * FX_PS]));
+          fx_acc(f2, q2, fx_split(Se[fx_slot(2, v) * FX_PS]));
+          // half the sum of the three directions (the factors carry 2^62)
+          const fx_t sum = ((f0.hi + f1.hi + f2.hi) << 1) + (f0.lo >> 31) + (f1.lo >> 31) + (f2.lo >> 31);
+          s[v] = (double)sum * __hiloint2double(iwh + (int)((unsigned)((v == 0 ? k0 : v < 4 ? km : ke) + top) << 20), iwl);
+        }
+      } else {
+#pragma unroll
+        for (int v = 0; v < 5; ++v) {
+          const int k = v == 0 ? k0 : v < 4 ? km : ke;
+          auto part = [&](FxD r, int dir, int e) {
+            FxSum f{0, 0x40000000ll};
+            fx_acc(f, r, fx_split(Se[fx_slot(dir, v) * FX_PS]));
+            return (double)((f.hi << 1) + (f.lo >> 31)) * __hiloint2double(iwh + (int)((unsigned)(k + e) << 20), iwl);
+          };
+          s[v] = part(r0, 0, e0) + part(r1, 1, e1) + part(r2, 2, e2);
+        }
       }
     } else {
       const double *Se = reinterpret_cast<const double *>(S) + le * FX_SLOTS * FX_PS + fx_idx(node);
@@ -686,12 +729,12 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB)
   }
 }
 
-// largest |Ja^d_c| and largest sum_c |Ja^d_c| of each element (high words) and largest 1/J, for the fixed-point
-// scales (1/J: zero where it spans more than 2^8 in the element, which sends the lifting to its general path)
+// per element: jmax (see DgDevice) and the largest 1/J, for the fixed-point scales (1/J: zero where it spans more than 2^8
+// in the element, which sends the lifting to its general path)
 __global__ void __launch_bounds__(128) k_metric_max(const DgDevice d) {  // one warp per element
   const int e = blockIdx.x * 4 + threadIdx.x / 32, lane = threadIdx.x % 32;
   if (e >= d.nE) return;
-  int h = 0, h1 = 0;
+  int h[3] = {0, 0, 0}, h1[3] = {0, 0, 0}, small = 0x7fffffff;
   double lo = 1e300, hi = 0.0;
   for (int t = lane; t < nnn; t += 32) {
     const double ij = d.invJ[(size_t)e * nnn + t];
@@ -701,19 +744,27 @@ __global__ void __launch_bounds__(128) k_metric_max(const DgDevice d) {  // one 
     for (int dd = 0; dd < 3; ++dd) {
       const double *J = d.Ja + ((size_t)e * 3 + dd) * 3 * nnn + t;
       const double a = fabs(J[0]), b = fabs(J[nnn]), c = fabs(J[2 * nnn]);
-      h = max(max(h, fx_hi_abs(a)), max(fx_hi_abs(b), fx_hi_abs(c)));
-      h1 = max(h1, fx_hi_abs(a + b + c));
+      const int m = max(fx_hi_abs(a), max(fx_hi_abs(b), fx_hi_abs(c)));
+      h[dd] = max(h[dd], m);
+      small = min(small, m);
+      h1[dd] = max(h1[dd], fx_hi_abs(a + b + c));
     }
   }
-  h = __reduce_max_sync(0xffffffffu, h);
-  h1 = __reduce_max_sync(0xffffffffu, h1);
+  small = __reduce_min_sync(0xffffffffu, small);
+  int lg = 0, top = 0;
+#pragma unroll
+  for (int dd = 0; dd < 3; ++dd) {
+    h[dd] = __reduce_max_sync(0xffffffffu, h[dd]);
+    lg = max(lg, fx_lg(__reduce_max_sync(0xffffffffu, h1[dd])) - (fx_unit(h[dd]) << 20));
+    top = max(top, fx_exponent(h[dd]));
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
     hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   }
   if (lane == 0) {
-    d.jmax[e] = int2{h, h1};
+    d.jmax[e] = int4{h[0], h[1], h[2], top - fx_exponent(small) > FX_JSPAN ? FX_FAR : lg};
     d.ijmax[e] = hi <= 256.0 * lo ? hi : 0.0;
   }
 }

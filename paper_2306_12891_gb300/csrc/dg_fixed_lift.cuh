@@ -24,17 +24,33 @@ struct FxLift {
   int bu, bt;              // left shifts that bring the element's largest reference derivatives to full size
   int he, hk;              // right shifts of u.tau and of the heat flux to their common scale
   int kt, km, ke;          // stress, momentum and energy fluxes are fixed value x 2^k
+  int e[3];                // 2^20 times the metric terms' e_d (for fvmax)
 };
 
-// exponents, before the derivative sums
-__device__ __forceinline__ FxLift fx_lift_exponents(int mu_, int mt, int2 mj, double muj, double kaj) {
+// exponents, before the derivative sums. The three directions' terms of J grad w are added at the scale of the largest metric
+// term, so on a stretched element the stress between two small velocity components is resolved at 2^-59 of the largest
+// one's. That stays below the rounding of the pressure flux in FP64 unless the element is dominated by viscosity:
+// tested where the directions' metric terms differ by more than 4, from bounds of the viscous flux
+// (mu/J) max|Ja|^2 max|w| / w_0 and of the smallest pressure flux, with the pressure of the element's first node.
+__device__ __forceinline__ FxLift fx_lift_exponents(const DgDevice &d, const double *U, int e, int mu_, int mt) {
   FxLift s;
-  s.eu = fx_exponent(mu_); s.et = fx_exponent(mt); s.ej = fx_exponent(mj.x);
+  const int4 mj = d.jmax[e];
+  const double ij = d.ijmax[e] * c_invw[0], muj = d.mu * ij, kaj = d.kappa * ij;
+  const int h = max(mj.x, max(mj.y, mj.z)), hs = min(mj.x, min(mj.y, mj.z));
+  s.e[0] = fx_unit(mj.x) << 20; s.e[1] = fx_unit(mj.y) << 20; s.e[2] = fx_unit(mj.z) << 20;
+  s.eu = fx_exponent(mu_); s.et = fx_exponent(mt); s.ej = fx_exponent(h);
   s.em = fx_exponent(__double2hiint(muj)); s.ek = fx_exponent(__double2hiint(kaj));
+  const int lo = min(min(s.et, s.ej), min(s.em, s.ek)), hi = max(max(s.et, s.ej), max(max(s.em, s.ek), s.eu));
+  s.ok = lo >= 800 && hi <= 1150;
+  if (h - hs > (2 << 20)) {
+    double Uv[5];
+    load_state<double>(d, U, e, 0, Uv);
+    const int p = __double2hiint(d.gm1 * (Uv[4] - 0.5 * (Uv[1] * Uv[1] + Uv[2] * Uv[2] + Uv[3] * Uv[3]) / Uv[0]));
+    s.ok = s.ok && p > 0 && s.em + 2 * s.ej + s.eu - 2046 <= 1 + (p >> 20) + (hs >> 20);
+  }
   // a fluid at rest has no scale of its own; the floor is 2^-32 sqrt(kappa T / mu)
   s.eu = max(s.eu, (959 - s.em + s.et + s.ek) >> 1);
-  const int lo = min(min(s.et, s.ej), min(s.em, s.ek)), hi = max(max(s.et, s.ej), max(max(s.em, s.ek), s.eu));
-  s.ok = lo >= 800 && hi <= 1250;
+  s.ok = s.ok && s.eu <= 1150;
   return s;
 }
 
@@ -59,9 +75,9 @@ __device__ __forceinline__ double fx_to(fx_t x, int k) {  // x 2^k (k keeps the 
 }
 
 __device__ __noinline__ void fx_general_lift(const DgDevice &d, size_t e, int node, const double *W,
-                                             const double (*sD)[n + 1], double *tau, int *fvm) {
+                                             const double (*sD)[n + 1], double *tau, const int *unit, int *fvm) {
   lift_node<double>(d, node, W, sD, d.Ja + e * 9 * nnn, d.Wsurf + e * 24 * nn, d.invJ[e * nnn + node], d.mu, d.kappa,
-                    d.Fv + e * 12 * nnn, tau ? tau + e * 6 * nnn : nullptr, fvm);
+                    d.Fv + e * 12 * nnn, tau ? tau + e * 6 * nnn : nullptr, unit, fvm);
 }
 
 // element slots: 0-3 u, v, w, T; 4 + 4 dir + q derivative sums; then the face jumps [6][4][nn]
@@ -120,8 +136,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice 
   __syncthreads();
   int good = 1;
   if (tid < FX_EPB && e0 + tid < d.nE) {
-    const double ij = d.ijmax[e0 + tid] * c_invw[0];
-    s_sc[tid] = fx_lift_exponents(s_mx[tid][0], s_mx[tid][1], d.jmax[e0 + tid], d.mu * ij, d.kappa * ij);
+    s_sc[tid] = fx_lift_exponents(d, U, e0 + tid, s_mx[tid][0], s_mx[tid][1]);
     good = s_sc[tid].ok;
   }
   const bool ok = __syncthreads_and(good);
@@ -261,6 +276,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice 
         }
       }
       double *out = d.Fv + (size_t)e * 12 * nnn + node;
+      int fm[3] = {0, 0, 0};
       auto project = [&](int q, FxD f0, FxD f1, FxD f2) {
 #pragma unroll
         for (int dd = 0; dd < 3; ++dd) {
@@ -270,12 +286,17 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice 
           fx_acc(s, J[dd][2], f2);
           const double f = fx_to(fx_value(s, 3), q < 3 ? c.km : c.ke);
           out[(dd * 4 + q) * nnn] = f;
-          fvm[q / 3] = max(fvm[q / 3], fx_hi_abs(f));
+          fm[dd] = max(fm[dd], fx_hi_abs(f));  // (finite, below 2^700)
         }
       };
       project(0, t[0], t[3], t[4]);
       project(1, t[3], t[1], t[5]);
       project(2, t[4], t[5], t[2]);
+#pragma unroll
+      for (int dd = 0; dd < 3; ++dd) {
+        fvm[0] = max(fvm[0], fm[dd] - c.e[dd]);
+        fm[dd] = 0;
+      }
       fx_t gt[3];
       grad(3, gt);
       const FxD K = fx_split(fx_from(d.kappa * ijw, c.ek, 1));
@@ -289,6 +310,8 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice 
         return fx_split(fx_shr(fx_value(s, 3), c.he) + fx_shr(fx_value(k, 4), c.hk));
       };
       project(3, energy(t[0], t[3], t[4], gt[0]), energy(t[3], t[1], t[5], gt[1]), energy(t[4], t[5], t[2], gt[2]));
+#pragma unroll
+      for (int dd = 0; dd < 3; ++dd) fvm[1] = max(fvm[1], fm[dd] - c.e[dd]);
     }
   } else {  // general path: FP64
     double *W = reinterpret_cast<double *>(S);  // [EPB][4][nnn], then D padded
@@ -301,7 +324,7 @@ __global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice 
     __syncthreads();
     if (on) {
       int m[2] = {0, 0};
-      fx_general_lift(d, e, node, W + le * 4 * nnn, sD, tau, m);
+      fx_general_lift(d, e, node, W + le * 4 * nnn, sD, tau, s_sc[le].e, m);
       fvm[0] = m[0];
       fvm[1] = m[1];
     }

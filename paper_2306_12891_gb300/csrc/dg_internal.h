@@ -46,9 +46,11 @@ struct DgDevice {
   double *Ja;          // [nE][3 d][3 c][n^3]
   double *J;           // [nE][n^3]
   double *invJ;        // [nE][n^3]
-  int2 *jmax;          // [nE] high words of the largest |Ja^d_c| and sum_c |Ja^d_c| (fixed-point scales)
+  int4 *jmax;          // [nE] fixed-point scales: high words of the largest |Ja^d_c| of the three directions; largest
+                       // sum_c |Ja^d_c| against its direction's scale (log2 in 2^-20; FX_FAR: too stretched)
   double *ijmax;       // [nE] largest 1/J (0 where it spans more than 2^8)
-  int *fvmax;          // [nE][2] high words of the largest viscous flux |Fv| (momentum, energy), by the lifting
+  int *fvmax;          // [nE][2] high words of the largest viscous flux |Fv^d| / (scale of Ja^d) (momentum, energy),
+                       // by the lifting
   float *Jaf;          // FP32 copy of Ja for the FP32-bulk path (or null)
   double *nrm;         // [nF][4][n^2]: unit normal (x,y,z) outward from L, area factor s
   float *nrm_f;        // FP32 copy of nrm for the FP32-bulk path (or null)

@@ -634,6 +634,8 @@ __global__ void __launch_bounds__(FACE_THREADS) k_face(const DgDevice d, const d
 // BR1 lifting + viscous flux: grad w = (1/J)[sum_d Ja^d D_d w + sum_faces (1/w_b) s n_out (w* - w)],
 // then Fv^d = sum_c Ja^d_c Fv_c(U, grad w) stored per node (4 components: momentum, energy).
 // ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ int fx_relative(double f, int unit);  // dg_fixed.cuh
+
 // (u, v, w, T) of one node from its state values (lifted quantities of BR1)
 template <typename R>
 __device__ __forceinline__ void lift_prim(const R Uv[5], R gm1, R iR, R pref, R Wn[4]) {
@@ -656,7 +658,8 @@ template <typename R>
 __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *__restrict__ W,
                                           const R (*__restrict__ sD)[n + 1], const R *__restrict__ Jae,
                                           const R *__restrict__ Wse, R iJ, R mu, R kappa, R *__restrict__ out,
-                                          double *__restrict__ tau = nullptr, int *fvm = nullptr) {
+                                          double *__restrict__ tau = nullptr, const int *unit = nullptr,
+                                          int *fvm = nullptr) {
   const int ijk[3] = {node % n, (node / n) % n, node / nn};
   R Ja[3][3];
 #pragma unroll
@@ -722,8 +725,8 @@ __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *
     for (int q = 0; q < 4; ++q) {
       const R f = Ja[dd][0] * Fc[0][q] + Ja[dd][1] * Fc[1][q] + Ja[dd][2] * Fc[2][q];
       out[(dd * 4 + q) * nnn + node] = f;
-      // FP64: high words of the largest momentum and energy components, the volume kernel's scale
-      if constexpr (std::is_same<R, double>::value) fvm[q / 3] = max(fvm[q / 3], __double2hiint(f) & 0x7fffffff);
+      // FP64: high words of the largest momentum and energy components against the directions' metric scales (fvmax)
+      if constexpr (std::is_same<R, double>::value) fvm[q / 3] = max(fvm[q / 3], fx_relative(f, unit[dd]));
     }
 }
 

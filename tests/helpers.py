@@ -292,3 +292,58 @@ def saved_state_ulp_spread(name, path, sample, base, count=3, seed=20230622):
     for o in outs:
         spread = np.maximum(spread, per_var_max(o - base))
     return spread
+
+
+_EXT_MAIN = r"""
+int ext_rhs(int N, int nE, const double *xyz, int nF, const int *faces, int eq, int vf, int sf, double mu, const double *Ja,
+            const double *J, const double *U, double *hi, double *lo) {
+  const size_t nnn = (size_t)(N + 1) * (N + 1) * (N + 1), M = 5 * nE * nnn;
+  long double *x = malloc(sizeof *x * 3 * nE * nnn), *u = malloc(sizeof *u * M), *ut = malloc(sizeof *u * M);
+  for (size_t k = 0; k < 3 * nE * nnn; ++k) x[k] = xyz[k];
+  for (size_t k = 0; k < M; ++k) u[k] = U[k];
+  orc_problem pb;
+  memset(&pb, 0, sizeof pb);
+  pb.N = N; pb.n_elems = nE; pb.xyz = x; pb.n_faces = nF; pb.faces = faces; pb.equations = eq; pb.vflux = vf; pb.sflux = sf;
+  pb.gamma = 1.4; pb.R = 1; pb.mu = mu; pb.Pr = 0.72; pb.alpha_fixed = -1; pb.wm_index = 1;
+  int st;
+  orc_state *s = orc_create(&pb, &st);
+  if (!s) return -1;
+  for (size_t k = 0; k < 9 * nE * nnn; ++k) s->Ja[k] = Ja[k];
+  for (size_t k = 0; k < nE * nnn; ++k) s->J[k] = J[k];
+  orc_rhs(s, u, ut, 0, 0);
+  for (size_t k = 0; k < M; ++k) { hi[k] = (double)ut[k]; lo[k] = (double)(ut[k] - hi[k]); }
+  orc_destroy(s);
+  free(x); free(u); free(ut);
+  return 0;
+}
+"""
+
+
+def rounding_errors(orc, N, xyz, faces, U, Ja, J, results, equations, vflux, sflux, mu):
+    """Per variable, the rms difference of each of the given right-hand sides from the oracle's statements in long double
+    with the same metric terms (gamma = 1.4, R = 1, Pr = 0.72): the rounding errors of their arithmetic alone."""
+    import ctypes
+    import os
+    import subprocess
+
+    out = os.path.join(os.path.dirname(orc.LIB_PATH), "extended")
+    os.makedirs(out, exist_ok=True)
+    so = os.path.join(out, "liboracle_ext.so")
+    if not os.path.exists(so) or os.path.getmtime(so) < max(os.path.getmtime(f) for f in (orc.SRC, orc.HDR, __file__)):
+        def text(path):
+            t = open(path).read().replace("long double", "double").replace("double", "long double")
+            return t.replace("<math.h>", "<tgmath.h>")
+        with open(os.path.join(out, "dgsem_oracle.h"), "w") as f:
+            f.write(text(orc.HDR))
+        with open(os.path.join(out, "ext.c"), "w") as f:
+            f.write(text(orc.SRC) + _EXT_MAIN)
+        subprocess.check_call(["gcc", "-O2", "-w", "-std=c11", "-fPIC", "-shared", "-ffp-contract=off", "-o", so + ".tmp",
+                               os.path.join(out, "ext.c"), "-lm"])
+        os.replace(so + ".tmp", so)
+    arr = [np.ascontiguousarray(a, dtype=np.float64) for a in (xyz, Ja, J, U)]
+    fc = np.ascontiguousarray(faces, dtype=np.int32)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    hi, lo = np.zeros(U.shape), np.zeros(U.shape)
+    assert ctypes.CDLL(so).ext_rhs(N, xyz.shape[0], p(arr[0]), len(fc), p(fc), orc.EQUATIONS[equations], orc.VFLUX[vflux],
+                                   orc.SFLUX[sflux], ctypes.c_double(mu), p(arr[1]), p(arr[2]), p(arr[3]), p(hi), p(lo)) == 0
+    return [np.sqrt((((X - hi) - lo) ** 2).mean(axis=(0, 2, 3, 4))) for X in results]

@@ -8,7 +8,7 @@ inputs (tests/helpers.py); their flux scale holds the advective flux only, which
 import numpy as np
 import pytest
 
-from helpers import ULP_FACTOR, per_var_max, ulp_spread
+from helpers import ULP_FACTOR, per_var_max, rounding_errors, ulp_spread
 from paper_2306_12891_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -73,6 +73,53 @@ def test_fixed_point_volume_terms(env, kind, N, nel, vf):
     err = per_var_max(Ut - Ur)
     print(f"FIXED-POINT {kind} N={N} {vf}: error / bound {err / np.maximum(ULP_FACTOR * spread, 1e-300)}")
     assert (err <= ULP_FACTOR * spread).all(), (err, ULP_FACTOR * spread)
+
+
+def _stretched(N, ar, curved):
+    """Two elements (N = 2: 16) with the z-edge ar times shorter than the others (x-edge: half the y-edge), and a shear layer across it:
+    Mach 0.3 along x, spanwise and wall-normal velocities 10^-3 of it, or the same size (curved meshes)."""
+    def wave(x, y, z):
+        return x + 0.1 * np.sin(y), y + 0.1 * np.sin(x), z + 0.1 / ar * np.sin(x) * np.cos(y)
+    xyz, faces = W.box_mesh(N, (2, 1, 1) if N > 2 else (4, 2, 2), hi=(W.TWO_PI, W.TWO_PI, W.TWO_PI / ar), mapping=wave if curved else None)
+    x, y, z = xyz[:, 0], xyz[:, 1], ar * xyz[:, 2]
+    e = 0.3 if curved else 3e-4
+    rho = 1.0 + 0.1 * np.sin(z + 1.0) * np.cos(x)
+    p = (1.0 + 0.05 * np.cos(x - y) * np.sin(z)) / 1.4
+    vel = [0.3 * np.sin(z / 2 + 0.3) * (1 + 0.2 * np.cos(x)), e * np.cos(z + y), e * np.sin(x + y) * np.sin(z / 2) ** 2]
+    return xyz, faces, W.cons_from_prim(rho, *vel, p)
+
+
+@pytest.mark.parametrize("curved", [False, True])
+@pytest.mark.parametrize("ar", [1, 7, 64, 1024, 16384])
+@pytest.mark.parametrize("N,vf,eq,mu", [(2, "kg", "euler", 0.0), (3, "pirozzoli", "euler", 0.0), (5, "kg", "ns", 0.01),
+                                        (7, "pirozzoli", "ns", 1e-3), (7, "kg", "euler", 0.0)])
+def test_stretched_elements_round_no_more_than_fp64(env, ar, N, vf, eq, mu, curved):
+    """The rounding error of each variable against that of the kernels' FP64 path: density, momentum, energy and mu in units
+    2^350 times larger take it, and change no significand. Both are rms values over at least 50 entries of a few hundred
+    roundings each: of the same size (0.5 to 1.3) where the arithmetic resolves the same."""
+    dg, orc, torch = env
+    xyz, faces, U = _stretched(N, ar, curved)
+    out = []
+    for k in (0, -350):
+        phys = dict(equations=eq, vflux=vf, sflux="llf", mu=float(np.ldexp(mu, k)))
+        s = dg.DG(N, xyz, faces, **phys)
+        out.append(np.ldexp(s.rhs(torch.from_numpy(np.ldexp(U, k)).cuda()).cpu().numpy(), -k))
+        s.check()
+    Ja, J = (t.cpu().numpy() for t in s.metrics())
+    here, plain = rounding_errors(orc, N, xyz, faces, U, Ja, J, out, eq, vf, "llf", mu)
+    print(f"FIXED-POINT stretched {ar} curved={curved} N={N} {vf} {eq}: error / FP64 path's {np.round(here / plain, 2)}")
+    assert (here <= 1.5 * plain).all(), here / plain
+
+
+@pytest.mark.parametrize("N,ar", [(2, 64), (5, 1024)])
+def test_stretched_elements_vjp_takes_the_fp64_path(env, N, ar):
+    """The product is linear in the cotangent, and FP64 arithmetic commutes with a power of two: equal bits."""
+    dg, orc, torch = env
+    xyz, faces, U = _stretched(N, ar, True)
+    s = dg.DG(N, xyz, faces, equations="euler", vflux="pirozzoli", sflux="llf")
+    lam = np.random.default_rng(N).standard_normal(U.shape)
+    a, b = (s.rhs_vjp(torch.from_numpy(U).cuda(), torch.from_numpy(np.ldexp(lam, k)).cuda()).cpu().numpy() for k in (0, 300))
+    np.testing.assert_array_equal(a, np.ldexp(b, -300))
 
 
 def _time(torch, call, k=20):
