@@ -241,12 +241,12 @@ constexpr int FX_LPW = 32 / n;
 // viscous divergence of the lane's node along its line: -sum_m Q_im Fv_m / 2 for the four quantities.
 // n even: lane i < n/2 forms the sum with the even half of Q, lane N - i that with the odd half
 // (n^2/2 products per line and quantity instead of n^2)
-__device__ __forceinline__ void fx_viscous(const double *__restrict__ Fn, const int2 *__restrict__ sQ, int idx, int l0,
+__device__ __forceinline__ void fx_viscous(const double *Fn, const int2 *__restrict__ sQ, int idx, int l0,
                                            int vm, int ve, fx_t acc[5]) {
   const int2 *row = sQ + idx * FX_QV;
   double f64[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) f64[q] = __ldg(Fn + q * nnn);
+  for (int q = 0; q < 4; ++q) f64[q] = Fn[q * nnn];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const fx_t f = fx_from(f64[q], q < 3 ? vm : ve, 0);

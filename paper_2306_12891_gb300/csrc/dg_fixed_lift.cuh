@@ -89,8 +89,7 @@ constexpr size_t FXL_SMEM = sizeof(fx_t) * FX_EPB * FXL_ELEM;
 // latencies between its four barriers; FMA-heavy 41 %, ALU 48 %, FP64 pipe 35 %, DRAM 20 %. Measured per launch
 // at N = 7, 24^3: 1.00 ms (the FP64 line sweeps with a node-wise contraction 2.57 ms); N = 5, 24 x 12 x 12: 0.123
 // against 0.277 ms.
-__global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice d, const double *__restrict__ U,
-                                                                 double *__restrict__ tau) {
+__global__ void __launch_bounds__(FX_THREADS, FX_MINB) k_lift_fx(const DgDevice d, const double *U, double *tau) {
   constexpr int JR = (FX_EPB * 24 * nn + FX_THREADS - 1) / FX_THREADS;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   fx_t *S = reinterpret_cast<fx_t *>(sm_raw);  // [EPB][FXL_ELEM]

@@ -207,7 +207,9 @@ __device__ __forceinline__ void flag_set(int *flag, int bit) { atomicOr(flag, bi
 // its blocks are in their last phase, and the next one's blocks load their tables and geometry, which no kernel
 // writes, before they wait for its completion (and, each kernel having waited for its own predecessor, for all
 // earlier ones). Not earlier: with three kernels' blocks on the SMs the block scheduler doubles some up (10 steps at
-// N = 7, 4^3: 3.46 ms when every kernel signalled at its start, 2.77 ms without dependent launch).
+// N = 7, 4^3: 3.46 ms when every kernel signalled at its start, 2.77 ms without dependent launch). A kernel launched so may
+// be running while its predecessor writes, so it reads what the chain writes (state, face and viscous fluxes, jumps) by
+// plain loads: no __ldg and no __restrict__ on those, whose read-only path asks for data constant from the kernel's start.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -217,7 +219,7 @@ __device__ __forceinline__ double to_double(double x) { return x; }
 // five conservative values of node `node` of element e, in the arithmetic type: the FP64 state,
 // or in FP32 its shadow copy (E' = E - p_ref/(gamma-1) already applied, rounded once)
 template <typename R>
-__device__ __forceinline__ void load_state(const DgDevice &d, const double *__restrict__ U, size_t e, int node,
+__device__ __forceinline__ void load_state(const DgDevice &d, const double *U, size_t e, int node,
                                            R out[5]) {
   if (kShift<R>) {
     const float *Ue = d.Uf + e * 5 * nnn + node;
@@ -525,7 +527,7 @@ __global__ void __launch_bounds__(256) k_round_geometry(const DgDevice d) {
 // mirror state's face value, and the wall shear stress of the wall model as the viscous flux
 // ---------------------------------------------------------------------------------------------
 template <typename R, int SF>
-__device__ __forceinline__ void wall_face(const DgDevice &d, const double *__restrict__ U, int f, int pq, int eL,
+__device__ __forceinline__ void wall_face(const DgDevice &d, const double *U, int f, int pq, int eL,
                                           int fL, R pref, R href, R gam) {
   const int p = pq % n, q = pq / n;
   const int node = face_node(fL, p, q);
@@ -583,7 +585,7 @@ __device__ __forceinline__ void wall_face(const DgDevice &d, const double *__res
 // (192 faces): 18.5 us with 256 threads, 12.5 with 128, 64 or 32; at 24^3 817 / 824 / 812 / 812 us.
 constexpr int FACE_THREADS = 64;
 template <typename R, int SF>
-__global__ void __launch_bounds__(FACE_THREADS) k_face(const DgDevice d, const double *__restrict__ U) {
+__global__ void __launch_bounds__(FACE_THREADS) k_face(const DgDevice d, const double *U) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)d.nF * nn) return;
   const int f = (int)(t / nn), pq = (int)(t % nn), p = pq % n, q = pq / n;
@@ -657,7 +659,7 @@ __device__ __forceinline__ void lift_prim(const R Uv[5], R gm1, R iR, R pref, R 
 template <typename R>
 __device__ __forceinline__ void lift_node(const DgDevice &d, int node, const R *__restrict__ W,
                                           const R (*__restrict__ sD)[n + 1], const R *__restrict__ Jae,
-                                          const R *__restrict__ Wse, R iJ, R mu, R kappa, R *__restrict__ out,
+                                          const R *Wse, R iJ, R mu, R kappa, R *__restrict__ out,
                                           double *__restrict__ tau = nullptr, const int *unit = nullptr,
                                           int *fvm = nullptr) {
   const int ijk[3] = {node % n, (node / n) % n, node / nn};
