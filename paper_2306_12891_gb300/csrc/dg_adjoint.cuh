@@ -588,6 +588,7 @@ __device__ __forceinline__ void adj_pair(const AdjNode &a, const AdjNode &b, dou
 // ---------------------------------------------------------------------------------------------
 struct FxAdj {
   int ok;
+  int none;                            // no cotangent in the element: ok, the pair cotangents are zero
   int er, eu, ep, ex, e0, e1, e4;      // exponents: rho, u, p, X, l of mass, momentum, energy
   int e[3], top;                       // of the metric terms' directions, as FxScale
   int av, aa, ab, af, ag, a0, ak, ax;  // windows of V, t_k S_u,k, t_4 S_X, F0, phi S_rho and the outputs
@@ -620,7 +621,9 @@ __device__ __forceinline__ FxAdj fx_adj_scales(const int *mx, int4 mj) {
   constexpr int ej = 1023;
   s.eu = max(fx_exponent(mx[2]), (1996 - s.er + s.ep) >> 1);
   // exponents of l: a group far below the others' shares of phi takes a scale 2^-40 of theirs
-  const int r0 = fx_exponent(mx[7]), r1 = fx_exponent(mx[8]), r4 = fx_exponent(mx[9]);
+  s.none = (mx[7] | mx[8] | mx[9]) == 0;
+  const int r0 = s.none ? 1023 : fx_exponent(mx[7]), r1 = s.none ? 1023 : fx_exponent(mx[8]),
+            r4 = s.none ? 1023 : fx_exponent(mx[9]);
   const int ph = max(r0, max(r1 + s.eu, r4 + s.ex) - 1023);
   s.e0 = max(r0, ph - 40); s.e1 = max(r1, ph - s.eu + 1023 - 40); s.e4 = max(r4, ph - s.ex + 1023 - 40);
   const int lo = min(min(min(s.er, s.ep), min(s.ex, min(j0, min(j1, j2)))), min(min(s.e0, s.e1), s.e4));
@@ -848,7 +851,8 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
       h[5] = fx_hi_abs(X); h[6] = __double2hiint(X);
       h[7] = fx_hi_abs(l[0]);
       h[8] = max(max(fx_hi_abs(l[1]), fx_hi_abs(l[2])), fx_hi_abs(l[3]));
-      h[9] = fx_hi_abs(l[4]);
+      const int low = __double2loint(l[0]) | __double2loint(l[1]) | __double2loint(l[2]) | __double2loint(l[3]) | __double2loint(l[4]);
+      h[9] = max(fx_hi_abs(l[4]), low != 0 ? 1 : 0);  // (all three zero: no cotangent, subnormal ones included)
       h[10] = fx_hi_abs(fabs(u[0]) + fabs(u[1]) + fabs(u[2]));
     }
     bool each = on;
@@ -873,7 +877,11 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
     good = s_sc[tid].ok;
   }
   const bool ok = __syncthreads_and(good);
-  if (ok) {
+  // a block without a cotangent has no pair terms (most of them, for a product with a pointwise or wall-local quantity)
+  bool none = ok;
+#pragma unroll
+  for (int k = 0; k < FX_EPB; ++k) none = none && (e0 + k >= d.nE || s_sc[k].none);
+  if (ok && !none) {
     if (on) {
       const FxAdj &c = s_sc[le];
       constexpr fx_t HB = FX_BIAS / 2;
@@ -926,7 +934,7 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
         for (int v = 0; v < 6; ++v) Sl[(6 + 8 * dir + v) * FX_PS + pb + idx * ps] = acc[v];
       }
     }
-  } else if (on) {
+  } else if (on && !ok) {
     double *Se = reinterpret_cast<double *>(S) + le * FXA_SLOTS * FX_PS + fx_idx(node);
     const double *Je = d.Ja + (size_t)e * 9 * nnn + node;
     Se[0] = r; Se[4 * FX_PS] = 4.0 * p; Se[5 * FX_PS] = X;
@@ -946,8 +954,8 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
   }
   __syncthreads();
   if (!on) return;
-  double gp[6];
-  if (ok) {
+  double gp[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (ok && !none) {
     const fx_t *Se = S + le * FXA_SLOTS * FX_PS + fx_idx(node);
     const FxAdj &c = s_sc[le];
     const double w8 = 0.125 * c_invw[0];
@@ -960,7 +968,7 @@ __global__ void __launch_bounds__(FX_THREADS, FXA_MINB) k_adj_volume(const DgDev
       else
         gp[v] = w8 * (fx_to(a, k - 1 + c.e[0]) + fx_to(b, k - 1 + c.e[1]) + fx_to(z, k - 1 + c.e[2]));
     }
-  } else {
+  } else if (!ok) {
     const double *Se = reinterpret_cast<const double *>(S) + le * FXA_SLOTS * FX_PS + fx_idx(node);
 #pragma unroll
     for (int v = 0; v < 6; ++v) gp[v] = Se[(6 + v) * FX_PS] + Se[(14 + v) * FX_PS] + Se[(22 + v) * FX_PS];
