@@ -110,10 +110,10 @@ dg_status dg_rhs(dg_ctx *ctx, const double *U, double *Ut, double t);
 dg_status dg_lserk_step(dg_ctx *ctx, double *U, double dt, double t);
 
 /* n_steps LSERK steps of size dt starting at time t. By default (dg_use_graphs) the launch sequence
- * of up to 16 steps is captured into a CUDA graph on the first call for a given (U, dt) and replayed
- * for the remaining steps on a library stream ordered after and before the context stream by
- * events (asynchronous as before; the first step, and steps that do not fill a graph, are launched
- * directly). Kernel timing disables it. */
+ * of 16 steps is captured into a CUDA graph once a given (U, dt) has been asked for more than 32, that
+ * of fewer when two calls in a row leave as many, and replayed on a library stream ordered after and
+ * before the context stream by events (asynchronous as before; other steps are launched directly).
+ * Kernel timing disables it. */
 dg_status dg_lserk_steps(dg_ctx *ctx, double *U, double dt, double t, int n_steps);
 
 /* The same step on a HOST array U_host: copies it to a library-owned device buffer, steps, and
@@ -239,7 +239,7 @@ dg_status dg_get_metrics(dg_ctx *ctx, double *Ja, double *J);
  * order, so it agrees with them to FP32 rounding. No effect in FP64. DG_ERR_ARG for other values. */
 dg_status dg_use_tma(dg_ctx *ctx, int mode);
 
-/* 1 (default): multi-step calls replay a CUDA graph of up to 16 steps; 0: every kernel is launched. Both
+/* 1 (default): multi-step calls replay CUDA graphs of up to 16 steps; 0: every kernel is launched. Both
  * run the same kernels and give identical bits. */
 dg_status dg_use_graphs(dg_ctx *ctx, int enable);
 

@@ -85,7 +85,7 @@ struct dg_ctx {
   bool tape_all = false;
   double tape_dt = 0.0;
   double fac_dt = std::nan("");  // step size of the FP32-bulk stage factor d.facf (NaN: not formed yet)
-  // CUDA graph of up to kGraphSteps LSERK steps, replayed by the multi-step calls on a library stream that is
+  // CUDA graphs of LSERK steps, replayed by the multi-step calls on a library stream that is
   // ordered after (and before) the caller's stream with events
   int use_graphs = 1;
   cudaStream_t gstream = nullptr;
@@ -96,11 +96,15 @@ struct dg_ctx {
   cudaStream_t cstream[kCopyStreams] = {};
   cudaEvent_t cev[kCopyStreams + 1] = {};
   static constexpr int kGraphSteps = 16;
-  cudaGraphExec_t step_graph = nullptr;
-  int graph_steps = 0;
-  const double *graph_U = nullptr;
+  struct StepGraph {
+    cudaGraphExec_t exec = nullptr;
+    int steps = 0;
+    long long launches = 0;
+  } long_graph, short_graph;  // of kGraphSteps steps and of fewer
+  const double *graph_U = nullptr;  // the state and step size of the graphs, or of the last calls where there is none
   double graph_dt = 0.0;
-  long long graph_launches = 0;
+  long long graph_seen = 0;  // steps asked for with these
+  int graph_rest = 0;        // steps beyond whole long graphs in the last call
 };
 
 namespace {
@@ -112,6 +116,13 @@ dg_status fail(dg_ctx *c, dg_status s, const std::string &msg) {
 
 dg_status cuda_fail(dg_ctx *c, cudaError_t e, const char *where) {
   return fail(c, DG_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
+}
+
+void drop_graphs(dg_ctx *c) {
+  for (dg_ctx::StepGraph *g : {&c->long_graph, &c->short_graph}) {
+    if (g->exec) cudaGraphExecDestroy(g->exec);
+    *g = {};
+  }
 }
 
 template <class T>
@@ -385,7 +396,7 @@ dg_status dg_basis(int N, double *xi, double *w, double *D) {
 
 void dg_free(dg_ctx *c) {
   if (!c) return;
-  if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
+  drop_graphs(c);
   if (c->gev_in) cudaEventDestroy(c->gev_in);
   if (c->gev_out) cudaEventDestroy(c->gev_out);
   if (c->gstream) cudaStreamDestroy(c->gstream);
@@ -613,9 +624,9 @@ dg_status plain_steps(dg_ctx *c, double *U, double dt, int n_steps) {
   return DG_OK;
 }
 
-// capture n_steps LSERK steps on U with step dt into c->step_graph (launches go to the library stream)
-dg_status capture_steps(dg_ctx *c, double *U, double dt, int n_steps) {
-  if (c->step_graph) { cudaGraphExecDestroy(c->step_graph); c->step_graph = nullptr; }
+// capture n_steps LSERK steps on U with step dt into `graph` (launches go to the library stream)
+dg_status capture_steps(dg_ctx *c, double *U, double dt, int n_steps, dg_ctx::StepGraph &graph) {
+  if (graph.exec) { cudaGraphExecDestroy(graph.exec); graph = {}; }
   cudaStream_t user = c->stream;
   c->stream = c->gstream;
   const long long l0 = c->launches;
@@ -627,31 +638,45 @@ dg_status capture_steps(dg_ctx *c, double *U, double dt, int n_steps) {
     const cudaError_t e2 = cudaStreamEndCapture(c->gstream, &g);
     if (!e && e2) e = e2;
   }
-  c->graph_launches = c->launches - l0;
+  graph.launches = c->launches - l0;
+  graph.steps = n_steps;
   c->launches = l0;  // captured, not run
   c->stream = user;
-  if (!e && st == DG_OK) e = cudaGraphInstantiate(&c->step_graph, g, 0);
+  if (!e && st == DG_OK) e = cudaGraphInstantiate(&graph.exec, g, 0);
   if (g) cudaGraphDestroy(g);
   if (e) {
     cudaGetLastError();
-    c->step_graph = nullptr;
+    graph = {};
     return cuda_fail(c, e, "step graph");
   }
-  if (st != DG_OK) return st;
-  c->graph_U = U;
-  c->graph_dt = dt;
-  c->graph_steps = n_steps;
-  return DG_OK;
+  return st;
 }
 
-// n_steps LSERK steps. With graphs on (and kernel timing off) the launch sequence of up to kGraphSteps steps is
-// captured once per (U, dt) and replayed, one graph launch instead of 160-320 kernel launches; steps that do not fill
-// a graph are launched. (One step per graph left a gap between graphs that the dependent launches within do not have.)
+// n_steps LSERK steps. With graphs on (and kernel timing off) the launch sequence of kGraphSteps steps is captured for
+// (U, dt) and replayed, one graph launch instead of 160-320 kernel launches; the rest is replayed from a graph of its own,
+// or launched, which takes the device 1 to 2 % longer (N = 3, 4^3: 74.8 against 73.3 us a step; graphs of one step:
+// 75.8, for the gap between two graphs). Capturing costs the host more than launching (10 steps at N = 3, 4^3: a
+// call of 287 us, 169 launched), so the long graph waits until the steps asked for with this state and step size exceed
+// two of it, and the short one for a second call with the same rest: a loop that sets the step size anew before every
+// few steps launches directly.
 dg_status steps_impl(dg_ctx *c, double *U, double dt, int n_steps) {
   DG_TRY(refresh_shadow(c, U));
   DG_TRY(ensure_stage_factor(c, dt));
   if (n_steps <= 0) return DG_OK;
-  if (!c->use_graphs || c->timing || n_steps < 2) return plain_steps(c, U, dt, n_steps);
+  constexpr int K = dg_ctx::kGraphSteps;
+  if (c->graph_U != U || c->graph_dt != dt) {
+    drop_graphs(c);
+    c->graph_U = U;
+    c->graph_dt = dt;
+    c->graph_seen = 0;
+    c->graph_rest = 0;
+  }
+  const bool first = c->graph_seen == 0;
+  const bool again = n_steps % K > 1 && n_steps % K == c->graph_rest;
+  c->graph_rest = n_steps % K;
+  c->graph_seen += n_steps;
+  const bool use_long = n_steps >= K && (c->long_graph.exec || c->graph_seen > 2 * K);
+  if (!c->use_graphs || c->timing || !(use_long || again)) return plain_steps(c, U, dt, n_steps);
   cudaError_t e = cudaSuccess;
   if (!c->gstream) {
     e = cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking);
@@ -659,26 +684,27 @@ dg_status steps_impl(dg_ctx *c, double *U, double dt, int n_steps) {
     if (!e) e = cudaEventCreateWithFlags(&c->gev_out, cudaEventDisableTiming);
     if (e) return cuda_fail(c, e, "graph stream");
   }
-  if (!(c->step_graph && c->graph_U == U && c->graph_dt == dt)) {
-    DG_TRY(plain_steps(c, U, dt, 1));  // first step directly (also sets kernel attributes outside capture)
+  if (first) {  // a first step directly, which also sets kernel attributes outside the capture
+    DG_TRY(plain_steps(c, U, dt, 1));
     --n_steps;
-    if (capture_steps(c, U, dt, std::min(n_steps, dg_ctx::kGraphSteps)) != DG_OK) {
-      c->use_graphs = 0;  // no graph on this stream: launch the kernels directly
-      c->err.clear();
-      return plain_steps(c, U, dt, n_steps);
-    }
   }
-  const int replays = n_steps / c->graph_steps;
-  if (replays > 0) {
-    e = cudaEventRecord(c->gev_in, c->stream);
-    if (!e) e = cudaStreamWaitEvent(c->gstream, c->gev_in, 0);
-    for (int k = 0; k < replays && !e; ++k) e = cudaGraphLaunch(c->step_graph, c->gstream);
-    if (!e) e = cudaEventRecord(c->gev_out, c->gstream);
-    if (!e) e = cudaStreamWaitEvent(c->stream, c->gev_out, 0);
-    if (e) return cuda_fail(c, e, "step graph launch");
-    c->launches += c->graph_launches * replays;
+  const int rest = n_steps % K;
+  if ((use_long && !c->long_graph.exec && capture_steps(c, U, dt, K, c->long_graph) != DG_OK) ||
+      (again && c->short_graph.steps != rest && capture_steps(c, U, dt, rest, c->short_graph) != DG_OK)) {
+    c->use_graphs = 0;  // no graph on this stream: launch the kernels directly
+    c->err.clear();
+    return plain_steps(c, U, dt, n_steps);
   }
-  return plain_steps(c, U, dt, n_steps % c->graph_steps);
+  const int replays = use_long ? n_steps / K : 0;
+  e = cudaEventRecord(c->gev_in, c->stream);
+  if (!e) e = cudaStreamWaitEvent(c->gstream, c->gev_in, 0);
+  for (int k = 0; k < replays && !e; ++k) e = cudaGraphLaunch(c->long_graph.exec, c->gstream);
+  if (again && !e) e = cudaGraphLaunch(c->short_graph.exec, c->gstream);
+  if (!e) e = cudaEventRecord(c->gev_out, c->gstream);
+  if (!e) e = cudaStreamWaitEvent(c->stream, c->gev_out, 0);
+  if (e) return cuda_fail(c, e, "step graph launch");
+  c->launches += c->long_graph.launches * replays + (again ? c->short_graph.launches : 0);
+  return plain_steps(c, U, dt, n_steps - replays * K - (again ? rest : 0));
 }
 // state copy by the SMs through the host-device link, 16 bytes per thread and step; for page-locked host
 // memory, which the device addresses directly
@@ -955,7 +981,7 @@ dg_status dg_use_tma(dg_ctx *c, int enable) {
   if (!c) return DG_ERR_ARG;
   if (enable < 0 || enable > 3) return fail(c, DG_ERR_ARG, "dg_use_tma: mode 0, 1, 2 or 3");
   c->d.use_tma = enable;
-  if (c->step_graph) { cudaGraphExecDestroy(c->step_graph); c->step_graph = nullptr; }  // kernels change
+  drop_graphs(c);  // kernels change
   return DG_OK;
 }
 

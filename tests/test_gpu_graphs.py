@@ -75,3 +75,67 @@ def test_small_case_time_per_step(env):
     print(f"GRAPHS N=3 4^3 Euler: {res[False]:.1f} us/step launched, {res[True]:.1f} us/step replayed "
           f"(x{res[False] / res[True]:.2f})")
     assert res[True] < res[False]
+
+
+def _small(dg, torch):
+    w = W.WORKLOADS["tgv_euler_n3_4x4x4"]
+    xyz, faces = w.mesh()
+    s = dg.DG(w.N, xyz, faces, **w.physics())
+    U = torch.from_numpy(w.initial_state(xyz)).cuda()
+    return s, U, s.max_dt(U, w.cfl)
+
+
+@pytest.mark.parametrize("calls", [[40, 3, 33, 16, 50], [10] * 6, [2, 100], [17, 17, 17, 5], [16, 16, 16, 16, 1],
+                                   [33], [32, 1, 16], [50, 50, 2, 2, 2, 50], [9, 9, 25, 25, 9], [1, 1, 1, 20, 20]])
+def test_sequences_of_calls_are_bit_identical(env, calls):
+    """Calls that launch, capture, replay and mix the three give the bits and the launch count of launching every kernel."""
+    dg, torch = env
+    out = []
+    for graphs in (False, True):
+        s, U0, dt = _small(dg, torch)
+        s.use_graphs(graphs)
+        U, l0 = U0.clone(), s.launch_count()
+        for k in calls:
+            s.lserk_steps(U, dt, k)
+        s.check()
+        out.append((U, s.launch_count() - l0))
+    assert torch.equal(out[0][0], out[1][0])
+    assert out[0][1] == out[1][1]
+
+
+def test_a_new_step_size_before_every_few_steps_captures_nothing(env):
+    """Host time of a call of 10 steps, a new dt each time: a graph for it would be replayed once (or, of 16 steps, not at
+    all), so the call costs what it costs with graphs off."""
+    dg, torch = env
+    cost = {}
+    for graphs in (False, True):
+        s, U, dt = _small(dg, torch)
+        s.use_graphs(graphs)
+        times = []
+        for k in range(30):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            s.lserk_steps(U, dt * (1 + 1e-9 * k), 10)
+            times.append(time.perf_counter() - t0)
+        cost[graphs] = sorted(times)[15] * 1e6
+    print(f"GRAPHS host time of 10 steps with a new dt: {cost[False]:.0f} us off, {cost[True]:.0f} us on")
+    assert cost[True] < 1.3 * cost[False]
+
+
+def test_a_short_first_call_does_not_shorten_the_graph(env):
+    """3000 steps after a first call of 2 take what they take without it (one-step graphs: a gap at every step)."""
+    dg, torch = env
+    res = {}
+    for first in (0, 2):
+        s, U, dt = _small(dg, torch)
+        dt *= 0.01
+        if first:
+            s.lserk_steps(U, dt, first)
+        s.lserk_steps(U, dt, 100)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        s.lserk_steps(U, dt, 3000)
+        torch.cuda.synchronize()
+        res[first] = (time.perf_counter() - t0) / 3000 * 1e6
+    print(f"GRAPHS us/step after a first call of 0 and 2 steps: {res[0]:.2f} {res[2]:.2f}")
+    assert res[2] < 1.015 * res[0]
