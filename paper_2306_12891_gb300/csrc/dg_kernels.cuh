@@ -1587,7 +1587,7 @@ void launch_volume_f32(const DgDevice &d, const double *U, double *out, double *
   const bool aligned = !(((uintptr_t)U | (uintptr_t)out | (uintptr_t)g) & 15u);
   // pair-symmetric line kernel, warp-specialised. Its warp groups trade registers (setmaxnreg), which
   // is only safe if the block is launched with exactly the registers the split assumes; any other
-  // compiled count takes the warp-specialised node kernel instead.
+  // compiled count takes the plain node kernel instead.
   static int grid_ln = 0;  // > 0: usable, < 0: not usable
   if (LN_OK && d.use_tma == 3 && aligned && grid_ln == 0) {
     cudaFuncAttributes fa{};
@@ -1607,11 +1607,12 @@ void launch_volume_f32(const DgDevice &d, const double *U, double *out, double *
     k_volume_f32_line<VF><<<blocks, LN_THREADS, LN_SMEM, s>>>(d, U, out, g, mode, first, dt, A, B);
     return;
   }
-  // warp-specialised persistent kernel: on request, and where the line kernel cannot run at N = 7. At N = 3 and 5 its few
-  // warps per SM leave it behind the TMA-fed node kernel below, which gives the same bits (right-hand side / LSERK stage:
-  // N = 5, 17 x 13 x 11: 69.6 / 74 against 45.2 / 54 us; 32^3: 903 / 945 against 529 / 641 us; N = 3, 32^3: 373 / 380
-  // against 128 / 163 us)
-  if (TMA_OK && (d.use_tma == 2 || (d.use_tma == 3 && LN_OK)) && aligned) {
+  // warp-specialised persistent kernel, on request: its few warps per SM leave it behind another form at every degree, with
+  // the same bits. At N = 3 and 5 that is the TMA-fed node kernel below (right-hand side / LSERK stage: N = 5,
+  // 17 x 13 x 11: 69.6 / 74 against 45.2 / 54 us; 32^3: 903 / 945 against 529 / 641 us; N = 3, 32^3: 373 / 380 against
+  // 128 / 163 us); at N = 7, where the line kernel cannot run, the plain one (stage at 32^3: 1470 against 1363 us, TMA-fed
+  // 1679, line kernel 1017)
+  if (TMA_OK && d.use_tma == 2 && aligned) {
     static int grid_ws = 0;
     if (!grid_ws) {
       cudaFuncSetAttribute(k_volume_f32_ws<VF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WS_SMEM);
@@ -1625,7 +1626,7 @@ void launch_volume_f32(const DgDevice &d, const double *U, double *out, double *
     k_volume_f32_ws<VF><<<blocks, WS_THREADS, WS_SMEM, s>>>(d, U, out, g, mode, first, dt, A, B);
     return;
   }
-  if (TMA_OK && d.use_tma && aligned) {
+  if (TMA_OK && (d.use_tma == 1 || (d.use_tma == 3 && !LN_OK)) && aligned) {
     static int grid = 0;  // persistent: CTAs resident on all SMs at once
     if (!grid) {
       cudaFuncSetAttribute(k_volume_f32_tma<VF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TB_SMEM);
