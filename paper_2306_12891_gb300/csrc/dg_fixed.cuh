@@ -10,10 +10,13 @@
 // is exact down to 2^-7 of the element's maximum. A product keeps the high 64 of 128 bits: with X = 2^32 h +
 // l, h and l signed 32-bit halves, it is h h' + (h l' + l h') / 2^32; the dropped l l' is below a quarter
 // unit. Every product is rounded to nearest in a window chosen per element (FxScale), so that the largest
-// value it can take fills the word. Pair sums, sums over a line and over directions are exact integer adds,
-// so with the pair symmetry Q_im = -Q_mi of the SBP operator Q = W D a pair's two shares cancel exactly.
+// value it can take fills the word. Pair sums and sums over a line are exact integer adds, so with the pair symmetry
+// Q_im = -Q_mi of the SBP operator Q = W D the two shares of a pair, formed once and handed on, cancel exactly (the pairs
+// half a line apart at even n are formed at both nodes, with opposite factors, and cancel to a unit: products round half up).
 // Precision: all rounding happens at about 2^-61 of the largest flux sum the element can have, where FP64
-// rounds each flux and each partial sum at 2^-53 of itself. An element takes the general FP64 path of the
+// rounds each flux and each partial sum at 2^-53 of itself, and values are held to 2^-60 of the element's largest of
+// their kind. So the results are those of FP64 normwise, per element and variable; what is small beside the rest of its
+// element (a velocity component far below the largest, say) is not held to 53 bits of its own. An element takes the general FP64 path of the
 // same kernel (fx_general_lines) instead when a value is not finite, rho, p or h (e) is not positive or
 // spans more than 2^8 within the element, the element is stretched by more than 8 (FX_JSPAN), or the exponents leave a safe
 // range.

@@ -8,7 +8,8 @@
 // (-1/2 and 1/2 at the ends) included; the BR1 face jump w* - w of a direction adds to its end nodes' sums
 // with weight -1 and 1, and the weights 1 / w_d of the three directions enter as ratios to the largest.
 // A derivative is a sum with cancellation: FP64 forms it to 2^-53 of sum |D_im w_m|, this form to 2^-59 of
-// the element's largest value, and later products keep that absolute resolution.
+// the element's largest value, and later products keep that absolute resolution: FP64's accuracy in the norm of the
+// stress over the element, not for each of its components (see fx_lift_exponents).
 #pragma once
 
 namespace {

@@ -1345,8 +1345,9 @@ __device__ __forceinline__ float scaled_float(double x, int e) {
 
 // cfl-free time step: min over nodes of 2J / ((2N+1) sum_d (|u.Ja^d| + c|Ja^d|)). The wave speed sum takes four FP64
 // square roots and a division (~75 FP64 instructions); it is estimated in FP32 first, from values scaled by their own
-// exponents (to 2e-6, the products' rounding added; 8e-6 is allowed), and evaluated in FP64 only where the estimate reaches the
-// block's largest sum / J so far. The node with the smallest step is never skipped, so the result is the minimum of
+// exponents (to 2e-6, the products' rounding added), and evaluated in FP64 only where the estimate, with 8 units of a
+// double's high word on top (at least 3.3e-6 after the estimate's truncation to one), reaches the block's largest
+// sum / J so far. The node with the smallest step is never skipped, so the result is the minimum of
 // the same FP64 expression. N = 5, 24^3: 210 us, 477 with every node in FP64.
 __global__ void __launch_bounds__(256) k_max_dt(const DgDevice d, const double *__restrict__ U) {
   __shared__ double red[256];

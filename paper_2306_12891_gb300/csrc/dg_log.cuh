@@ -1,5 +1,6 @@
-// dg_log.cuh -- natural logarithm of a positive normal double on the integer pipes, to an absolute error of 2^-58 and
-// the roundings of the final sum, for sums in which it meets numbers of order one (the entropy of the integral
+// dg_log.cuh -- natural logarithm of a positive normal double on the integer pipes, to an absolute error of
+// 2^-58 + 2^-54 + 2.4e-17 |k| (ln m in fixed point, its conversion, the rounded ln 2 times the exponent k below) and half an
+// ulp of the result, for sums in which it meets numbers of order one (the entropy of the integral
 // diagnostics; CUDA's log is ~25 FP64 instructions, on a pipe of 2 lanes per clock and SM: two of them per node were
 // most of k_invariants, N = 5, 24^3 644 -> 330 us).
 //
