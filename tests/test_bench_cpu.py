@@ -22,7 +22,7 @@ def test_fp32_step_roofline_from_kernel_timings():
 
 
 def test_algorithmic_counts_are_positive_and_grow_with_degree():
-    for f in (lambda N: bench.volume_kernel_flops_per_element(N, True), bench.lift_kernel_flops_per_element,
+    for f in (lambda N: bench.volume_kernel_flops_per_element(N, True), lambda N: bench.volume_kernel_mads_per_element(N, True), bench.lift_kernel_flops_per_element,
               bench.adjoint_visc_flops_per_element, lambda N: bench.fv_subcell_flops_per_element(N, bench.LLF_FLOPS),
               lambda N: bench.adjoint_volume_flops_per_element(N, True)):
         vals = [f(N) for N in range(1, 8)]
