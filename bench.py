@@ -38,10 +38,10 @@ UNIT = "DOF-stage/s"
 STAGES = 5
 P0_TGV = 1.0 / (1.4 * 0.1 ** 2)  # background pressure of the Ma 0.1 Taylor-Green vortex
 # DRAM bytes per element of one volume-kernel launch (dram__bytes_read.sum + dram__bytes_write.sum),
-# from an ncu capture of the current kernel on the 24^3 case (a later LSERK stage: 2068.35 MB read,
-# 544.90 MB written for 13824 elements), scaled to a launch by the element count (the kernel's
+# from an ncu capture of the current kernel on the 24^3 case (a later LSERK stage: 2067.44 MB read,
+# 545.15 MB written for 13824 elements), scaled to a launch by the element count (the kernel's
 # traffic is per element). None once the kernel has changed since that capture.
-VOLUME_DRAM_BYTES_PER_ELEMENT = (2068.350720e6 + 544.896768e6) / 24 ** 3
+VOLUME_DRAM_BYTES_PER_ELEMENT = (2067.442176e6 + 545.152512e6) / 24 ** 3
 # DRAM bytes (read + write) of one FP32-bulk volume launch (pair-symmetric line kernel, stage factor) per
 # element, from one ncu capture at the full 32^3 size of the second stage of a step (3492.2 MB read,
 # 1625.3 MB written for 32768 elements)

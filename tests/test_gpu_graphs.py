@@ -123,7 +123,7 @@ def test_a_new_step_size_before_every_few_steps_captures_nothing(env):
 
 
 def test_a_short_first_call_does_not_shorten_the_graph(env):
-    """3000 steps after a first call of 2 take what they take without it (one-step graphs: a gap at every step)."""
+    """1600 steps after a first call of 2 take what they take without it (one-step graphs: a gap at every step)."""
     dg, torch = env
     res = {}
     for first in (0, 2):
@@ -132,10 +132,13 @@ def test_a_short_first_call_does_not_shorten_the_graph(env):
         if first:
             s.lserk_steps(U, dt, first)
         s.lserk_steps(U, dt, 100)
-        torch.cuda.synchronize()
-        t0 = time.perf_counter()
-        s.lserk_steps(U, dt, 3000)
-        torch.cuda.synchronize()
-        res[first] = (time.perf_counter() - t0) / 3000 * 1e6
+        times = []
+        for _ in range(3):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            s.lserk_steps(U, dt, 1600)
+            torch.cuda.synchronize()
+            times.append((time.perf_counter() - t0) / 1600 * 1e6)
+        res[first] = min(times)
     print(f"GRAPHS us/step after a first call of 0 and 2 steps: {res[0]:.2f} {res[2]:.2f}")
-    assert res[2] < 1.015 * res[0]
+    assert res[2] < 1.025 * res[0]  # (one-step graphs: 1.045)
