@@ -45,8 +45,8 @@ enum { DG_SFLUX_LLF = 0, DG_SFLUX_ROE = 1, DG_SFLUX_EC = 2 };
 /* DG_FP64: FP64 state, geometry and results; all arithmetic FP64 or, in the lifting and in the volume
  * operator of the KG and Pirozzoli fluxes, 64-bit fixed point scaled per element. Its rounding error is not above
  * FP64's in the norm of each variable over an element; what is small beside the rest of its element (a velocity
- * component far below the largest) is not held to 53 bits of its own. Elements stretched by more than 8, or whose
- * values span too much for one scale, are evaluated in FP64. DG_FP32_BULK: volume/surface/lifting arithmetic in FP32 with FP32
+ * component far below the largest) is not held to 53 bits of its own. Elements stretched by more than 8 to 16 (the
+ * metric terms' exponents are compared), or whose values span too much for one scale, are evaluated in FP64. DG_FP32_BULK: volume/surface/lifting arithmetic in FP32 with FP32
  * accumulation; LSERK state, metrics, Jacobian scaling and reductions stay FP64. U, Ut stay FP64. */
 enum { DG_FP64 = 0, DG_FP32_BULK = 1 };
 /* boundary kinds (faceR of a face with elemR = -1) */

@@ -18,8 +18,8 @@
 // their kind. So the results are those of FP64 normwise, per element and variable; what is small beside the rest of its
 // element (a velocity component far below the largest, say) is not held to 53 bits of its own. An element takes the general FP64 path of the
 // same kernel (fx_general_lines) instead when a value is not finite, rho, p or h (e) is not positive or
-// spans more than 2^8 within the element, the element is stretched by more than 8 (FX_JSPAN), or the exponents leave a safe
-// range.
+// spans more than 2^8 within the element, the exponents of its metric terms differ by more than FX_JSPAN (a stretch beyond 8 to
+// 16), or the exponents leave a safe range.
 #pragma once
 
 namespace {
